@@ -209,7 +209,7 @@ struct lbm_mix {
   size_t ev_used = 0;
   std::string err;
   // learned closure: FP32 master weights, Adam moments, gradient, bf16 image,
-  // accept/fallback counters, mini-batch scratch
+  // accept/fallback counters, gradient scratch
   int closure = 0;
   float *d_w = nullptr, *d_m = nullptr, *d_v = nullptr, *d_g = nullptr;
   unsigned char* d_img = nullptr;
@@ -217,8 +217,6 @@ struct lbm_mix {
   double* d_loss = nullptr;
   int adam_t = 0;
   lbm::MlpScratch z{};
-  float* z_base = nullptr;
-  long long z_rows = 0;
 
   size_t need_pops() const { return (size_t)(M + 2) * 27 * (size_t)N * store_elem_bytes(prec); }
   // side planes, then (16-bit storage) the two buffers of equilibrium records
@@ -259,17 +257,19 @@ struct lbm_mix {
     return LBM_OK;
   }
   lbm::MlpShape mlp_shape() const { return lbm::MlpShape{128, ks->mlp_F, ks->mlp_O, 3 * M}; }
-  // Mini-batch scratch for `rows` samples (grown on demand).
-  lbm_status ensure_train_scratch(long long rows) {
-    if (rows <= z_rows) return LBM_OK;
-    if (z_base) { cudaStreamSynchronize(stream); cudaFree(z_base); z_base = nullptr; z_rows = 0; }
-    const long long H = 128, O = ks->mlp_O;
-    lbm_status st = cuda(cudaMalloc(&z_base, sizeof(float) * (size_t)rows * (6 * H + 2 * O)), "cudaMalloc(training)");
+  // Scratch of the training gradient (first use): one partial per SM.
+  lbm_status ensure_train_scratch() {
+    if (z.part) return LBM_OK;
+    int sms = 0;
+    lbm_status st = cuda(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device), "device attribute");
     if (st != LBM_OK) return st;
-    float* q = z_base;
-    z.h1 = q; q += rows * H; z.a1 = q; q += rows * H; z.h2 = q; q += rows * H; z.a2 = q; q += rows * H;
-    z.d1 = q; q += rows * H; z.d2 = q; q += rows * H; z.out = q; q += rows * O; z.dout = q;
-    z_rows = rows;
+    const size_t loss_bytes = sizeof(double) * (size_t)sms;
+    void* q = nullptr;
+    st = cuda(cudaMalloc(&q, loss_bytes + 256 + sizeof(float) * (size_t)sms * ks->mlp_nw), "cudaMalloc(training)");
+    if (st != LBM_OK) return st;
+    z.loss = static_cast<double*>(q);
+    z.part = reinterpret_cast<float*>(static_cast<char*>(q) + (loss_bytes + 255) / 256 * 256);
+    z.blocks = sms;
     return LBM_OK;
   }
   lbm_status repack() {
@@ -1137,12 +1137,12 @@ lbm_status lbm_mix_closure_loss_grad(lbm_mix_t h, const float* features, const f
                                      float* grad, double* loss) {
   if (!h) return LBM_ERR_ARG;
   if (n <= 0 || n > (1LL << 30) || !features || !targets) return h->fail(LBM_ERR_ARG, "bad arguments");
-  lbm_status s = h->ensure_train_scratch(n);
+  lbm_status s = h->ensure_train_scratch();
   if (s != LBM_OK) return s;
   s = h->cuda(lbm::mlp_train_grad(h->stream, h->mlp_shape(), h->d_w, features, targets, (int)n, h->z,
                                   grad ? grad : h->d_g, h->d_loss), "training kernels");
   if (s != LBM_OK) return s;
-  h->launches += 16;
+  h->launches += 2;
   if (loss) {
     if ((s = h->cuda(cudaMemcpyAsync(loss, h->d_loss, sizeof(double), cudaMemcpyDeviceToHost, h->stream),
                      "copy loss")) != LBM_OK)
@@ -1158,7 +1158,7 @@ lbm_status lbm_mix_closure_train(lbm_mix_t h, const float* features, const float
   if (n <= 0 || batch <= 0 || steps < 0 || !(lr > 0.0) || !features || !targets)
     return h->fail(LBM_ERR_ARG, "bad arguments");
   const long long rows_max = batch < n ? batch : n;
-  lbm_status s = h->ensure_train_scratch(rows_max);
+  lbm_status s = h->ensure_train_scratch();
   if (s != LBM_OK) return s;
   const int F = h->ks->mlp_F, O = h->ks->mlp_O;
   const long long nw = h->ks->mlp_nw;
@@ -1170,7 +1170,7 @@ lbm_status lbm_mix_closure_train(lbm_mix_t h, const float* features, const float
     if (s != LBM_OK) return s;
     s = h->cuda(lbm::mlp_adam(h->stream, h->d_w, h->d_g, h->d_m, h->d_v, nw, (float)lr, ++h->adam_t), "Adam kernel");
     if (s != LBM_OK) return s;
-    h->launches += 17;
+    h->launches += 3;
     start += rows;
     if (start >= n) start = 0;
   }
@@ -1481,7 +1481,7 @@ lbm_status lbm_mix_destroy(lbm_mix_t h) {
   if (h->d_stage) cudaFree(h->d_stage);
   cudaFree(h->d_err); cudaFree(h->d_partials); cudaFree(h->d_sums); cudaFree(h->d_base);
   cudaFree(h->d_w); cudaFree(h->d_img); cudaFree(h->d_stats);
-  if (h->z_base) cudaFree(h->z_base);
+  if (h->z.loss) cudaFree(h->z.loss);
   if (h->d_jet) cudaFree(h->d_jet);
   for (cudaEvent_t e : h->ev_pool) cudaEventDestroy(e);
   delete h;

@@ -11,11 +11,12 @@ struct MlpShape {
   int valid;     // outputs that enter the loss (3M)
 };
 
-// Device scratch for one mini-batch of `rows` samples: [rows][H] for the
-// hidden pre-activations, activations and their gradients, [rows][O] for the
-// outputs and their gradients.
+// Device scratch of the gradient: the partial gradients [blocks][weights] and
+// losses [blocks] of up to `blocks` blocks (one per SM).
 struct MlpScratch {
-  float *h1, *a1, *h2, *a2, *d1, *d2, *out, *dout;
+  float* part;
+  double* loss;
+  int blocks;
 };
 
 // Gradient of the mean-squared loss at weights w over `rows` samples
@@ -23,9 +24,6 @@ struct MlpScratch {
 // into *d_loss (device).
 cudaError_t mlp_train_grad(cudaStream_t s, const MlpShape& sh, const float* w, const float* X, const float* T,
                            int rows, const MlpScratch& z, float* g, double* d_loss);
-// FP32 forward pass only (outputs in z.out).
-cudaError_t mlp_train_forward(cudaStream_t s, const MlpShape& sh, const float* w, const float* X, int rows,
-                              const MlpScratch& z);
 // One Adam step (step number t >= 1, beta1 0.9, beta2 0.999, eps 1e-8).
 cudaError_t mlp_adam(cudaStream_t s, float* w, const float* g, float* m, float* v, long long count, float lr, int t);
 
