@@ -1030,7 +1030,7 @@ static lbm_status halo_move(lbm_mix_t h, int face, int ghost, void* buf, int unp
   b += (size_t)lbm::NSIDE * seg * ss;
   const long long rw = h->p64.rec_w;
   if (e == cudaSuccess && rw > 0)
-    e = halo_copy<float>((float*)h->scratch + lbm::eq_rec_offset(N), b, 2, rw * N, z0 * plane * rw, seg * rw, unpack,
+    e = halo_copy<float>((float*)h->scratch + lbm::eq_rec_offset(N), b, 2 * (rw / 4), 4 * N, z0 * plane * 4, seg * 4, unpack,
                          h->stream);
   if ((s = h->cuda(e, unpack ? "halo unpack" : "halo pack")) != LBM_OK) return s;
   h->launches += rw > 0 ? 3 : 2;

@@ -606,7 +606,7 @@ __device__ __forceinline__ void collide_node(const DevParams<Real>& p, Store* __
         r.Gq = Gc * inv_theta; r.hq = hk * rho * inv_theta;
 #pragma unroll
         for (int a = 0; a < M; ++a) r.ra[a] = th.rho_a_dev[a];
-        store_rec<M>(eq_rec_buf(side, N, p.rec_w, PAR), n, p.rec_w, p.weak, r);
+        store_rec<M>(eq_rec_buf(side, N, p.rec_w, PAR), N, n, p.weak, r);
       }
     }
     const Real w0 = Real(1) - theta, w1 = Real(0.5) * theta;          // Eq. (w0)

@@ -49,7 +49,7 @@ init_rec_kernel(const DevParams<double> p, float* __restrict__ side, const doubl
   }
   const double j[3] = {rho * u[0], rho * u[1], rho * u[2]};
   const double rhoE = rho * (Umix + 0.5 * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]));
-  store_rec<M>(eq_rec_buf(side, N, p.rec_w, 1), n, p.rec_w, p.weak, eq_record64<M>(p, ra, rho, j, rhoE, u));
+  store_rec<M>(eq_rec_buf(side, N, p.rec_w, 1), N, n, p.weak, eq_record64<M>(p, ra, rho, j, rhoE, u));
 }
 
 // With 16-bit storage the stored value of each population is its deviation

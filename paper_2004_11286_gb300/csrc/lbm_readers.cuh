@@ -182,7 +182,7 @@ rec_from_pops_kernel(const DevParams<double> p, float* __restrict__ side, int bu
     for (int a = 0; a < M; ++a) rs += ra[a];
     for (int d = 0; d < 3; ++d) usp[d] = jsp[d] / rs;          // Eq. (uSPEC)
   }
-  store_rec<M>(eq_rec_buf(side, N, p.rec_w, buf), n, p.rec_w, p.weak, eq_record64<M>(p, ra, rho, j, rhoE, usp));
+  store_rec<M>(eq_rec_buf(side, N, p.rec_w, buf), N, n, p.weak, eq_record64<M>(p, ra, rho, j, rhoE, usp));
 }
 
 // Replaces the state by natural-layout full populations (no terms pending).

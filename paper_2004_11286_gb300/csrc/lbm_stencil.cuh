@@ -100,7 +100,7 @@ __device__ __forceinline__ void eq_incoming(const DevParams<float>& p, const flo
     if (WALL && arrives_from_wall(nb, I)) refl = true;
     else snd = nb.idx(-cx_of(I), -cy_of(I), -cz_of(I));
   }
-  const EqRec<M> r = load_rec<M>(rin, snd, p.rec_w, p.weak);
+  const EqRec<M> r = load_rec<M>(rin, N, snd, p.weak);
   if (WALL && refl) eq_shift<M, opp_of(I)>(p, r, sh);
   else eq_shift<M, I>(p, r, sh);
   cf = 0.0f; cg = 0.0f;
