@@ -190,10 +190,10 @@ __device__ __forceinline__ Nbr opaque(const Nbr& a) {
 
 // Halfway bounce-back at the walls normal to x: direction i arrives from
 // beyond a wall (its sender x - c_i is outside), or would leave through one.
-__device__ __forceinline__ bool arrives_from_wall(const Nbr& nb, int i) {
-  const int cx = cx_of(i);
+__device__ __forceinline__ bool arrives_from_wall_c(const Nbr& nb, int cx) {
   return (cx > 0 && (nb.wall & 1u)) || (cx < 0 && (nb.wall & 2u));
 }
+__device__ __forceinline__ bool arrives_from_wall(const Nbr& nb, int i) { return arrives_from_wall_c(nb, cx_of(i)); }
 __device__ __forceinline__ bool leaves_to_wall(const Nbr& nb, int i) {
   const int cx = cx_of(i);
   return (cx > 0 && (nb.wall & 2u)) || (cx < 0 && (nb.wall & 1u));

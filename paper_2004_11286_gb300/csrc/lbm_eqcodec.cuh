@@ -25,11 +25,11 @@
 // Record slots (floats), as deviations from the reference rest state where
 // the quantity has one (T_r, theta_r, RL of each lattice):
 //   [0..3]     u_x, u_y, u_z, dT                  mixture velocity, T - T_r
-//   [4..7]     dtheta, drho, drhoE, Gq            theta - theta_r, rho - RL_f, rho E - RL_g, Gq = Gc / theta
+//   [4..7]     dtheta, drho, dE0, Gq              theta - theta_r, rho - RL_f, E_0 less its rest value, Gq = Gc / theta
 //   [8..8+M)   drho_1 .. drho_M                   coupled species densities - RL_a
 //   [8+M]      hq = (H + u^2/2) rho / theta       first-moment factor of g^eq (then padding to 4)
 //   [..+3]     u_sp (weak coupling only)          velocity of the species subsystem
-// with Gc = rho (h + theta) / (2 theta), h = H + u^2/2.  The momentum and
+// with Gc = rho (h + theta) / (2 theta), h = H + u^2/2, E_0 = rho E - 3P/2 - Gc u^2.  The momentum and
 // energy shifts are formed as deviations without cancellation (the same
 // telescoped forms as the collision's equilibria), so the receiver recovers
 // the populations to FP32 rounding of their deviations.
@@ -61,7 +61,7 @@ __device__ __forceinline__ const float* eq_rec_buf(const float* side, long long 
 
 template <int M>
 struct EqRec {
-  float u[3], dth, dT, drho, drhoE, Gq, hq;
+  float u[3], dth, dT, drho, dE0, Gq, hq;
   float ra[M];      // species densities minus RL_a
   float usp[3];
 };
@@ -73,7 +73,7 @@ __device__ __forceinline__ EqRec<M> load_rec(const float* __restrict__ buf, long
   EqRec<M> r;
   const float4 a = __ldg(q), b = __ldg(q + N);
   r.u[0] = a.x; r.u[1] = a.y; r.u[2] = a.z; r.dT = a.w;
-  r.dth = b.x; r.drho = b.y; r.drhoE = b.z; r.Gq = b.w;
+  r.dth = b.x; r.drho = b.y; r.dE0 = b.z; r.Gq = b.w;
   constexpr int NT = (1 + M + 3) / 4;
   float t[4 * NT];
 #pragma unroll
@@ -98,7 +98,7 @@ __device__ __forceinline__ void store_rec(float* __restrict__ buf, long long N, 
                                           const EqRec<M>& r) {
   float4* q = reinterpret_cast<float4*>(buf) + node;
   q[0] = make_float4(r.u[0], r.u[1], r.u[2], r.dT);
-  q[N] = make_float4(r.dth, r.drho, r.drhoE, r.Gq);
+  q[N] = make_float4(r.dth, r.drho, r.dE0, r.Gq);
   constexpr int NT = (1 + M + 3) / 4;
   float t[4 * NT];
 #pragma unroll
@@ -111,83 +111,277 @@ __device__ __forceinline__ void store_rec(float* __restrict__ buf, long long N, 
   if (weak) q[(2 + NT) * N] = make_float4(r.usp[0], r.usp[1], r.usp[2], 0.0f);
 }
 
-// Product form Psi_I(xi, z) = prod_a (b_a + k_a z) with b_0 = 1 - xi^2,
-// b_{+-1} = (+-xi + xi^2)/2, k_0 = -1, k_{+-1} = 1/2 (Sec. 2.4), as the
-// cubic P0 + P1 z + P2 z^2 + P3 z^3 in z, so the species (one z each) share
-// the velocity part.
-template <int I>
-struct PsiCubic {
-  float P0, P1, P2;
-  static constexpr float kx = cx_of(I) == 0 ? -1.0f : 0.5f;
-  static constexpr float ky = cy_of(I) == 0 ? -1.0f : 0.5f;
-  static constexpr float kz = cz_of(I) == 0 ? -1.0f : 0.5f;
-  static constexpr float P3 = kx * ky * kz;
-  __device__ __forceinline__ PsiCubic(const float (&xi)[3]) {
-    auto b = [](int c, float x) { return c == 0 ? 1.0f - x * x : 0.5f * ((c > 0 ? x : -x) + x * x); };
-    const float bx = b(cx_of(I), xi[0]), by = b(cy_of(I), xi[1]), bz = b(cz_of(I), xi[2]);
-    P0 = bx * by * bz;
-    P1 = kx * by * bz + bx * ky * bz + bx * by * kz;
-    P2 = kx * ky * bz + kx * by * kz + bx * ky * kz;
-  }
-  __device__ __forceinline__ float operator()(float z) const { return P0 + z * (P1 + z * (P2 + z * P3)); }
-};
-
 // The shifts of direction I of every lattice, as deviations from the
 // reference rest state (the arithmetic works on d = f - b_ref):
 //   sh_L = f^eq_{L,I}(record) - b_ref_{L,I}.
 // Species (Eq. 27eq) as rho_a Psi_I(u_sp, R_a T) - b_ref; momentum (Eq. feq)
 // and energy (Eqs. gansatz, gieq) lattices in the telescoped deviation forms
 // of the collision (lbm_collide.cuh), which carry no O(f) cancellation.
+// f (lattice M): rho (Psi_I(u, theta) - W_I(theta_r)) + (rho - RL_f) W_I(theta_r)
+template <int I>
+__device__ __forceinline__ float eq_shift_f(const DevParams<float>& p, int M, const float (&u)[3], float dth,
+                                            float drho) {
+  const float x2[3] = {u[0] * u[0], u[1] * u[1], u[2] * u[2]};
+  return (p.RL[M] + drho) * pf_diff<float, I>(u, x2, p.thr, dth) + drho * pf_ref<float, I>(p.thr);
+}
+// g (lattice M + 1): w_I(theta) [E_I + q^eq . c_I / theta] + B_I . Z relative
+// to its rest value.  E_I less its rest value, dE_I = dE_0 + (drho/2) |c|^2 +
+// Gq (u . c)^2, and E_I itself differ by a constant of the velocity's length
+// (energy_rest), so the bracket's deviation is w_I dE_I + (w_I - W_I) (E_I - dE_I).
+template <class Real>
+__device__ __forceinline__ Real energy_rest(const DevParams<Real>& p, int M, int k2) {
+  return p.RL[M + 1] - Real(1.5) * p.RL[M] * p.thr + Real(0.5) * Real(k2) * p.RL[M];
+}
+template <int I>
+__device__ __forceinline__ float eq_shift_g(const DevParams<float>& p, int M, const float (&u)[3], float dth,
+                                            float drho, float dE0, float Gq, float hq) {
+  constexpr int k2 = c2_of(I);
+  constexpr int cx = cx_of(I), cy = cy_of(I), cz = cz_of(I);
+  const float theta = p.thr + dth;
+  const float uc = dotc<float, I>(u);
+  const float dEi = dE0 + 0.5f * (float)k2 * drho + Gq * uc * uc;
+  const float w0 = 1.0f - theta, w1 = 0.5f * theta;
+  const float r0 = 1.0f - p.thr, r1 = 0.5f * p.thr;
+  const float d0 = -dth, d1 = 0.5f * dth;
+  const float wx = cx ? w1 : w0, wy = cy ? w1 : w0, wz = cz ? w1 : w0;
+  const float rx = cx ? r1 : r0, ry = cy ? r1 : r0;
+  const float ddx = cx ? d1 : d0, ddy = cy ? d1 : d0, ddz = cz ? d1 : d0;
+  const float wyz = wy * wz;
+  const float dwi = ddx * wyz + rx * (ddy * wz + ry * ddz);
+  float sh = wx * wyz * (dEi + hq * uc) + dwi * energy_rest(p, M, k2);
+  if constexpr (k2 <= 1) {
+    const float z1 = 1.0f - 3.0f * theta;
+    const float zb = 0.5f * (z1 * (drho * theta + p.RL[M] * dth) - 3.0f * dth * p.Pr);
+    const float zG = z1 * Gq * theta;
+    if constexpr (k2 == 0) {
+      sh += 3.0f * zb + zG * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
+    } else {
+      constexpr int ax = cx ? 0 : (cy ? 1 : 2);
+      sh -= 0.5f * (zb + zG * u[ax] * u[ax]);
+    }
+  }
+  return sh;
+}
+// Species (Eq. 27eq): per axis Psi_c = b + k z with (b, k) = (1 - x^2, -1) or
+// ((x^2 +- x) / 2, 1/2), two species at a time in the lanes of paired FP32
+// instructions.
 template <int M, int I>
 __device__ __forceinline__ void eq_shift(const DevParams<float>& p, const EqRec<M>& r, float (&sh)[M + 2]) {
   constexpr int k2 = c2_of(I);
-  constexpr int cx = cx_of(I), cy = cy_of(I), cz = cz_of(I);
+  constexpr int cs[3] = {cx_of(I), cy_of(I), cz_of(I)};
   const float T = p.Tr + r.dT;
-  if (p.weak) {
-    const PsiCubic<I> ps(r.usp);
+  float b[3];
 #pragma unroll
-    for (int a = 0; a < M; ++a) sh[a] = (p.RL[a] + r.ra[a]) * ps(p.R_a[a] * T) - p.bref[a][k2];
-  } else {
-    const PsiCubic<I> ps(r.u);
-#pragma unroll
-    for (int a = 0; a < M; ++a) sh[a] = (p.RL[a] + r.ra[a]) * ps(p.R_a[a] * T) - p.bref[a][k2];
+  for (int d = 0; d < 3; ++d) {
+    const float x = p.weak ? r.usp[d] : r.u[d];
+    b[d] = cs[d] == 0 ? 1.0f - x * x : 0.5f * ((cs[d] > 0 ? x : -x) + x * x);
   }
-  const float rho = p.RL[M] + r.drho;
-  const float x2[3] = {r.u[0] * r.u[0], r.u[1] * r.u[1], r.u[2] * r.u[2]};
-  // f: rho (Psi_I(u, theta) - W_I(theta_r)) + (rho - RL_f) W_I(theta_r)
-  sh[M] = rho * pf_diff<float, I>(r.u, x2, p.thr, r.dth) + r.drho * pf_ref<float, I>(p.thr);
-  // g: w_I(theta) [E_I + q^eq . c_I / theta] + B_I . Z relative to its rest value
-  const float theta = p.thr + r.dth;
-  const float Gc = r.Gq * theta;
-  const float usq = x2[0] + x2[1] + x2[2];
-  const float dP = r.drho * theta + p.RL[M] * r.dth;
-  const float P = rho * theta;
-  const float E0 = (p.RL[M + 1] + r.drhoE) - 1.5f * P - Gc * usq;
-  const float dE0 = r.drhoE - 1.5f * dP - Gc * usq;
-  const float uc = dotc<float, I>(r.u);
-  const float ucu = r.Gq * uc * uc;
-  const float cc = 0.5f * (float)k2;
-  const float Ei = E0 + cc * rho + ucu;
-  const float dEi = dE0 + cc * r.drho + ucu;
-  const float w0 = 1.0f - theta, w1 = 0.5f * theta;
-  const float r0 = 1.0f - p.thr, r1 = 0.5f * p.thr;
-  const float d0 = -r.dth, d1 = 0.5f * r.dth;
-  const float wx = cx ? w1 : w0, wy = cy ? w1 : w0, wz = cz ? w1 : w0;
-  const float rx = cx ? r1 : r0, ry = cy ? r1 : r0, rz = cz ? r1 : r0;
-  const float ddx = cx ? d1 : d0, ddy = cy ? d1 : d0, ddz = cz ? d1 : d0;
-  const float dwi = ddx * wy * wz + rx * ddy * wz + rx * ry * ddz;
-  float bz = 0.0f;
-  if constexpr (k2 <= 1) {
-    const float z1 = 1.0f - 3.0f * theta;
-    const float zb = 0.5f * (z1 * dP - 3.0f * r.dth * p.Pr);
-    if constexpr (k2 == 0) {
-      bz = 3.0f * zb + z1 * Gc * usq;
-    } else {
-      constexpr int ax = cx ? 0 : (cy ? 1 : 2);
-      bz = -0.5f * (zb + z1 * Gc * x2[ax]);
+#pragma unroll
+  for (int a = 0; a + 1 < M; a += 2) {
+    const float2 z = mul2(make_float2(p.R_a[a], p.R_a[a + 1]), make_float2(T, T));
+    float2 f[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const float2 bb = make_float2(b[d], b[d]);
+      f[d] = cs[d] == 0 ? sub2(bb, z) : fma2(make_float2(0.5f, 0.5f), z, bb);
+    }
+    const float2 ra = add2(make_float2(p.RL[a], p.RL[a + 1]), make_float2(r.ra[a], r.ra[a + 1]));
+    const float2 s = fma2(mul2(ra, f[0]), mul2(f[1], f[2]), make_float2(-p.bref[a][k2], -p.bref[a + 1][k2]));
+    sh[a] = s.x;
+    sh[a + 1] = s.y;
+  }
+  if constexpr (M % 2) {
+    constexpr int a = M - 1;
+    const float z = p.R_a[a] * T;
+    float f[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) f[d] = cs[d] == 0 ? b[d] - z : b[d] + 0.5f * z;
+    sh[a] = (p.RL[a] + r.ra[a]) * f[0] * (f[1] * f[2]) - p.bref[a][k2];
+  }
+  sh[M] = eq_shift_f<I>(p, M, r.u, r.dth, r.drho);
+  sh[M + 1] = eq_shift_g<I>(p, M, r.u, r.dth, r.drho, r.dE0, r.Gq, r.hq);
+}
+
+// A record as loaded (the species velocity only under weak coupling).
+template <int M>
+struct RecLoad {
+  static constexpr int NT = (1 + M + 3) / 4;
+  float4 q[3 + NT];
+  __device__ __forceinline__ RecLoad(const float* __restrict__ buf, long long N, long long node, int weak) {
+    const float4* r = reinterpret_cast<const float4*>(buf) + node;
+#pragma unroll
+    for (int k = 0; k < 2 + NT; ++k) q[k] = __ldg(r + k * N);
+    q[2 + NT] = weak ? __ldg(r + (2 + NT) * N) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  }
+};
+
+// Equilibrium shifts of every lattice for one velocity (cx, cy, cz) given at
+// run time, from the sender's record (eq_shift of lbm_eqcodec.cuh with the
+// velocity as data): per axis the product-form factor is r + da, r the rest
+// factor at theta_r and da = be (x^2 + dz) + ga x, with (be, ga) = (1/2, c/2),
+// or (-1, 0) for c = 0.  sp: species pairs; dth: the sender's theta - theta_r.
+template <int M>
+__device__ __forceinline__ void eq_shift_dir(const DevParams<float>& p, const RecLoad<M>& rec, bool refl, int cx,
+                                             int cy, int cz, float2 (&sp)[(M + 1) / 2], float& sf, float& sg,
+                                             float& dth) {
+  constexpr int NT = RecLoad<M>::NT, NP = (M + 1) / 2;
+  const float4 A = rec.q[0], B = rec.q[1];
+  float t[4 * NT];
+#pragma unroll
+  for (int k = 0; k < NT; ++k) {
+    const float4 c = rec.q[2 + k];
+    t[4 * k] = c.x; t[4 * k + 1] = c.y; t[4 * k + 2] = c.z; t[4 * k + 3] = c.w;
+  }
+  const float sgn = refl ? -1.0f : 1.0f;          // f^eq of the opposite velocity is that of -u
+  float u[3] = {sgn * A.x, sgn * A.y, sgn * A.z};
+  dth = B.x;
+  const float bx = cx ? 0.5f : -1.0f, by = cy ? 0.5f : -1.0f, bz = cz ? 0.5f : -1.0f;
+  const float gx = 0.5f * cx, gy = 0.5f * cy, gz = 0.5f * cz;
+  const int k2 = cx * cx + cy * cy + cz * cz;
+  // mixture velocity: da = q + be dth with q = be x^2 + ga x
+  const float x2[3] = {u[0] * u[0], u[1] * u[1], u[2] * u[2]};
+  const float qx = bx * x2[0] + gx * u[0], qy = by * x2[1] + gy * u[1], qz = bz * x2[2] + gz * u[2];
+  {
+    float vx = qx, vy = qy, vz = qz;
+    if (p.weak) {
+      const float4 w = rec.q[2 + NT];
+      const float s0 = sgn * w.x, s1 = sgn * w.y, s2 = sgn * w.z;
+      vx = bx * s0 * s0 + gx * s0; vy = by * s1 * s1 + gy * s1; vz = bz * s2 * s2 + gz * s2;
+    }
+    const float2 ax = bcast<float2>(vx + (cx ? 0.0f : 1.0f)), ay = bcast<float2>(vy + (cy ? 0.0f : 1.0f)),
+                 az = bcast<float2>(vz + (cz ? 0.0f : 1.0f));
+    const float2 T = bcast<float2>(p.Tr + A.w);
+#pragma unroll
+    for (int q = 0; q < NP; ++q) {
+      const int a0 = 2 * q, a1 = 2 * q + 1 < M ? 2 * q + 1 : 2 * q;
+      const float2 z = mul2(make_float2(p.R_a[a0], p.R_a[a1]), T);
+      const float2 f = mul2(mul2(fma2(bcast<float2>(bx), z, ax), fma2(bcast<float2>(by), z, ay)),
+                            fma2(bcast<float2>(bz), z, az));
+      const float2 ra = add2(make_float2(p.RL[a0], p.RL[a1]), make_float2(t[a0], t[2 * q + 1]));
+      sp[q] = fma2(ra, f, make_float2(-p.bref[a0][k2], -p.bref[a1][k2]));
     }
   }
-  sh[M + 1] = dwi * Ei + rx * ry * rz * dEi + bz + wx * wy * wz * r.hq * uc;
+  const float r1 = 0.5f * p.thr, r0 = 1.0f - p.thr;
+  const float rx = cx ? r1 : r0, ry = cy ? r1 : r0, rz = cz ? r1 : r0;
+  const float rho = p.RL[M] + B.y, rr = rx * ry * rz;
+  const float wx = bx * dth, wy = by * dth, wz = bz * dth;      // w_c(theta) - w_c(theta_r)
+  {
+    const float dx = qx + wx, dy = qy + wy, dz = qz + wz, az = rz + dz;
+    sf = rho * (dx * ((ry + dy) * az) + rx * (dy * az + ry * dz)) + B.y * rr;
+  }
+  const float uc = cx * u[0] + cy * u[1] + cz * u[2];
+  const float dEi = B.z + 0.5f * k2 * B.y + B.w * uc * uc;
+  const float oz = rz + wz, oyz = (ry + wy) * oz;
+  sg = (rx + wx) * oyz * (dEi + t[M] * uc) + (wx * oyz + rx * (wy * oz + ry * wz)) * energy_rest(p, M, k2);
+  if (k2 <= 1) {
+    const float theta = p.thr + dth, z1 = 1.0f - 3.0f * theta;
+    const float zb = 0.5f * (z1 * (B.y * theta + p.RL[M] * dth) - 3.0f * dth * p.Pr), zG = z1 * B.w * theta;
+    if (k2 == 0) sg += 3.0f * zb + zG * (x2[0] + x2[1] + x2[2]);
+    else sg -= 0.5f * (zb + zG * (cx ? x2[0] : (cy ? x2[1] : x2[2])));
+  }
+}
+
+// What one sender adds to the populations it sent along the three velocities
+// (c_x = -1, 0, 1; c_y; c_z) of a row: the equilibrium shifts of every
+// lattice (as eq_shift_dir) and, on f and g, the deferred terms
+// c . X / 2 (faces) and w(theta) c . K.  The (y, z) factors, and all that
+// depends on the sender alone, are formed once for the three.
+template <int M>
+struct RowTerms {
+  static constexpr int NP = (M + 1) / 2;
+  float2 sp[3][NP];
+  float f[3], g[3];
+};
+// What a sender's RowTerms are formed from, as loaded: its record, K, and the
+// component of X that a face velocity of the row needs.
+template <int M>
+struct RowLoad {
+  RecLoad<M> rec;
+  float k[3], x;
+  __device__ __forceinline__ RowLoad(const DevParams<float>& p, const float* __restrict__ side,
+                                     const float* __restrict__ rin, long long snd, int cy, int cz)
+      : rec(rin, p.N, snd, p.weak) {
+    const long long N = p.N;
+    k[0] = __ldg(side + (SP_K + 0) * N + snd);
+    k[1] = cy ? __ldg(side + (SP_K + 1) * N + snd) : 0.0f;
+    k[2] = cz ? __ldg(side + (SP_K + 2) * N + snd) : 0.0f;
+    x = cy * cz == 0 ? __ldg(side + (SP_X + (cy ? 1 : (cz ? 2 : 0))) * N + snd) : 0.0f;
+  }
+};
+template <int M>
+__device__ __forceinline__ void row_terms(const DevParams<float>& p, const RowLoad<M>& in, int cy, int cz,
+                                          RowTerms<M>& out) {
+  constexpr int NT = RecLoad<M>::NT, NP = (M + 1) / 2;
+  const float4 A = in.rec.q[0], B = in.rec.q[1];
+  float t[4 * NT];
+#pragma unroll
+  for (int k = 0; k < NT; ++k) {
+    const float4 c = in.rec.q[2 + k];
+    t[4 * k] = c.x; t[4 * k + 1] = c.y; t[4 * k + 2] = c.z; t[4 * k + 3] = c.w;
+  }
+  const float dth = B.x, drho = B.y;
+  const float by = cy ? 0.5f : -1.0f, bz = cz ? 0.5f : -1.0f, gy = 0.5f * cy, gz = 0.5f * cz;
+  const int kyz = cy * cy + cz * cz;
+  const float x2 = A.x * A.x, hx = 0.5f * A.x;
+  const float qy = by * A.y * A.y + gy * A.y, qz = bz * A.z * A.z + gz * A.z;
+  {
+    float sx2 = x2, shx = hx, sy = qy, sz = qz;
+    if (p.weak) {
+      const float4 w = in.rec.q[2 + NT];
+      sx2 = w.x * w.x; shx = 0.5f * w.x;
+      sy = by * w.y * w.y + gy * w.y; sz = bz * w.z * w.z + gz * w.z;
+    }
+    const float2 ay = bcast<float2>(sy + (cy ? 0.0f : 1.0f)), az = bcast<float2>(sz + (cz ? 0.0f : 1.0f));
+    const float2 T = bcast<float2>(p.Tr + A.w), px = bcast<float2>(shx), mx = bcast<float2>(-shx);
+#pragma unroll
+    for (int q = 0; q < NP; ++q) {
+      const int a0 = 2 * q, a1 = 2 * q + 1 < M ? 2 * q + 1 : 2 * q;
+      const float2 z = mul2(make_float2(p.R_a[a0], p.R_a[a1]), T);
+      const float2 ra = add2(make_float2(p.RL[a0], p.RL[a1]), make_float2(t[a0], t[2 * q + 1]));
+      const float2 yz = mul2(mul2(ra, fma2(bcast<float2>(by), z, ay)), fma2(bcast<float2>(bz), z, az));
+      const float2 s = add2(bcast<float2>(sx2), z), hs = mul2(bcast<float2>(0.5f), s);
+      const float2 r0 = make_float2(-p.bref[a0][kyz], -p.bref[a1][kyz]);
+      const float2 r1 = make_float2(-p.bref[a0][kyz + 1], -p.bref[a1][kyz + 1]);
+      out.sp[0][q] = fma2(yz, add2(hs, mx), r1);
+      out.sp[1][q] = fma2(yz, sub2(bcast<float2>(1.0f), s), r0);
+      out.sp[2][q] = fma2(yz, add2(hs, px), r1);
+    }
+  }
+  const float r1 = 0.5f * p.thr, r0 = 1.0f - p.thr;
+  const float ry = cy ? r1 : r0, rz = cz ? r1 : r0, ryz = ry * rz;
+  const float wy = by * dth, wz = bz * dth, wx = 0.5f * dth;    // w_c(theta) - w_c(theta_r); x: c = 0 gives -dth
+  {
+    const float rho = p.RL[M] + drho;
+    const float dy = qy + wy, dz = qz + wz, az = rz + dz, ayz = (ry + dy) * az, fyz = dy * az + ry * dz;
+    const float hs = 0.5f * (x2 + dth), cf = 0.5f * in.x;
+    const float e1 = r1 * fyz, d1 = drho * (r1 * ryz);
+    out.f[0] = rho * ((hs - hx) * ayz + e1) + d1;
+    out.f[1] = rho * (r0 * fyz - (hs + hs) * ayz) + drho * (r0 * ryz);
+    out.f[2] = rho * ((hs + hx) * ayz + e1) + d1;
+    if (kyz == 0) { out.f[0] -= cf; out.f[2] += cf; }
+    if (kyz == 1) out.f[1] += (cy + cz) * cf;
+  }
+  const float oz = rz + wz, oyz = (ry + wy) * oz, dyz = wy * oz + ry * wz;
+  const float w1 = (r1 + wx) * oyz, w0 = (r0 - dth) * oyz;
+  const float c0 = (r0 * dyz - dth * oyz) * energy_rest(p, M, kyz), c1 = (wx * oyz + r1 * dyz) * energy_rest(p, M, kyz + 1);
+  const float uyz = cy * A.y + cz * A.z, kk = cy * in.k[1] + cz * in.k[2];
+  const float e0 = B.z + 0.5f * kyz * drho + kk, e1 = e0 + 0.5f * drho;
+  const float um = uyz - A.x, up = uyz + A.x, hq = t[M];
+  out.g[0] = w1 * (e1 + um * (B.w * um + hq) - in.k[0]) + c1;
+  out.g[1] = w0 * (e0 + uyz * (B.w * uyz + hq)) + c0;
+  out.g[2] = w1 * (e1 + up * (B.w * up + hq) + in.k[0]) + c1;
+  if (kyz <= 1) {
+    const float theta = p.thr + dth, z1 = 1.0f - 3.0f * theta;
+    const float zb = 0.5f * (z1 * (drho * theta + p.RL[M] * dth) - 3.0f * dth * p.Pr), zG = z1 * B.w * theta;
+    if (kyz == 0) {
+      const float bx = 0.5f * (zb + zG * x2);
+      out.g[0] -= bx;
+      out.g[1] += 3.0f * zb + zG * (x2 + A.y * A.y + A.z * A.z);
+      out.g[2] -= bx;
+    } else {
+      out.g[1] -= 0.5f * (zb + zG * (cy ? A.y * A.y : A.z * A.z));
+    }
+  }
 }
 
 // The record of a node from its coupled moments, in FP64 (initialisation
@@ -218,7 +412,8 @@ __device__ __forceinline__ EqRec<M> eq_record64(const DevParams<double>& p, cons
 #pragma unroll
   for (int c = 0; c < 3; ++c) { r.u[c] = (float)u[c]; r.usp[c] = (float)u_sp[c]; }
   r.dth = (float)(th - p.thr); r.dT = (float)(T - p.Tr);
-  r.drho = (float)(rho - p.RL[M]); r.drhoE = (float)(rhoE - p.RL[M + 1]);
+  r.drho = (float)(rho - p.RL[M]);
+  r.dE0 = (float)(rhoE - 1.5 * rho * th - Gc * usq - (p.RL[M + 1] - 1.5 * p.RL[M] * p.thr));
   r.Gq = (float)(Gc / th);
   r.hq = (float)(hk * rho / th);
 #pragma unroll

@@ -186,4 +186,32 @@ __device__ __forceinline__ float2 sub2(float2 a, float2 b) {
   return d;
 }
 
+// Two species' values of one quantity.
+template <class Real> struct Pair;
+template <> struct Pair<float> { using T = float2; };
+template <> struct Pair<double> { using T = double2; };
+__device__ __forceinline__ double2 mul2(double2 a, double2 b) { return make_double2(a.x * b.x, a.y * b.y); }
+__device__ __forceinline__ double2 add2(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ double2 sub2(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
+__device__ __forceinline__ double2 fma2(double2 a, double2 b, double2 c) {
+  return make_double2(a.x * b.x + c.x, a.y * b.y + c.y);
+}
+// The same arithmetic on one lattice's values.
+template <class T> __device__ __forceinline__ T vmul(T a, T b) { return a * b; }
+template <class T> __device__ __forceinline__ T vadd(T a, T b) { return a + b; }
+template <class T> __device__ __forceinline__ T vsub(T a, T b) { return a - b; }
+template <class T> __device__ __forceinline__ T vfma(T a, T b, T c) { return a * b + c; }
+#define LBM_PAIR_OPS(V)                                                                                   \
+  template <> __device__ __forceinline__ V vmul<V>(V a, V b) { return mul2(a, b); }                       \
+  template <> __device__ __forceinline__ V vadd<V>(V a, V b) { return add2(a, b); }                       \
+  template <> __device__ __forceinline__ V vsub<V>(V a, V b) { return sub2(a, b); }                       \
+  template <> __device__ __forceinline__ V vfma<V>(V a, V b, V c) { return fma2(a, b, c); }
+LBM_PAIR_OPS(float2)
+LBM_PAIR_OPS(double2)
+#undef LBM_PAIR_OPS
+template <class V, class Real> __device__ __forceinline__ V bcast(Real x) {
+  if constexpr (std::is_same<V, Real>::value) return x;
+  else { V v; v.x = x; v.y = x; return v; }
+}
+
 }  // namespace lbm
