@@ -15,6 +15,7 @@
 #pragma once
 
 #include "lbm_collide.cuh"
+#include "lbm_split.cuh"
 #include "lbm_batch.cuh"
 #include "lbm_readers.cuh"
 #include "lbm_frame.cuh"
@@ -263,12 +264,47 @@ struct Launch {
       collide_kernel<M, Real, Store, 1, CL, LD, WALL><<<grid_for(c.N, BS), BS, smem, c.stream>>>(
           P(c), (Store*)c.pops, side, c.err, c.mlp_img, c.mlp_stats, po);
   }
+  template <int BND>
+  static void split_launch(const LaunchCtx& c, int parity, Real* side) {
+    using C = Split<M>;
+    constexpr size_t smem = C::REALS * sizeof(Real);
+    static int resident = 0;                     // blocks the device holds at once
+    if (!resident) {
+      int dev = 0, sms = 1, per = 1;
+      cudaGetDevice(&dev);
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+      cudaFuncSetAttribute(collide_split_kernel<M, Real, Store, 0, BND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      cudaFuncSetAttribute(collide_split_kernel<M, Real, Store, 1, BND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, collide_split_kernel<M, Real, Store, 0, BND>, C::THREADS, smem);
+      resident = sms * (per > 0 ? per : 1);
+    }
+    PlaneOffsets po;
+    for (int k = 0; k < (M + 2) * Q; ++k) po.off[k] = (long long)k * c.N * (long long)sizeof(Store);
+    const int ntiles = (int)grid_for(c.N, 32);
+    const int grid = ntiles < resident ? ntiles : resident;
+    if (parity == 0)
+      collide_split_kernel<M, Real, Store, 0, BND><<<grid, C::THREADS, smem, c.stream>>>(P(c), (Store*)c.pops, side, c.err, ntiles, po);
+    else
+      collide_split_kernel<M, Real, Store, 1, BND><<<grid, C::THREADS, smem, c.stream>>>(P(c), (Store*)c.pops, side, c.err, ntiles, po);
+  }
   // Bulk row loads where the blocks are whole row segments and the stage
   // holds the stored type (FP64, FP32).
   template <int CL>
   static void collide(const LaunchCtx& c, int parity, Real* side) {
     // Walls normal to x (bounce-back), the opposed-jets frame: register
     // loads, exact closure (the host refuses both with the network closure).
+    if constexpr (CL == 0 && kSplit<M, Real, Store>) {
+      if constexpr (EQ) {
+        if (P(c).wall_x) split_launch<1>(c, parity, side);
+        else split_launch<0>(c, parity, side);
+      } else {
+        if (P(c).tvar) collide_launch<0, 0>(c, parity, side);
+        else if (P(c).wall_x) split_launch<1>(c, parity, side);
+        else if (P(c).frame) split_launch<2>(c, parity, side);
+        else split_launch<0>(c, parity, side);
+      }
+      return;
+    } else {
     if constexpr (CL == 0) {
       if (P(c).wall_x) {
         collide_launch<0, 0, 1>(c, parity, side);
@@ -288,6 +324,7 @@ struct Launch {
       }
     }
     collide_launch<CL, 0>(c, parity, side);
+    }
   }
   static cudaError_t step(const LaunchCtx& c, int parity) {
     Real* side = (Real*)c.side;

@@ -1,0 +1,803 @@
+// lbm_split.cuh -- the fused collide + stream with the lattices of a node
+// shared out over the warps of a block.
+//
+// A block takes tiles of 32 nodes, one per lane.  Per tile:
+//   1. the warps share out the 27 velocities: for each, the populations of
+//      every lattice are loaded, decoded, given the terms still due
+//      (lbm_stencil.cuh) and staged in shared memory.  The velocity is data of
+//      a loop, not unrolled: with 16-bit storage the unrolled decoding of the
+//      senders' equilibria overflows the instruction cache;
+//   2. warp r < NP takes the species pair (2r, 2r + 1), its two species the
+//      lanes of paired FP32 instructions, warp NP takes f, warp NP + 1 takes
+//      g, and each sums its lattices' moments;
+//   3. the node closure (coupling, thermodynamics, transport, the
+//      Stefan-Maxwell system) runs with LPN lanes per node, a species pair and
+//      two rows of the system per lane, sums and pivot rows by shuffles;
+//   4. each warp updates and stores its lattices.
+// Species and momentum updates are formed in moment space.  The product form
+// of Sec. 2.4 is Psi_c = (sum over p of) t_cp m_p per axis with
+// m = (1, xi, xi^2 + zeta), so a lattice's 27 values are one fixed transform
+// (t x t x t) of its 27 product moments, and everything added to a species
+// (its equilibrium and the forces of all other species, Eq. fstar1) is summed
+// as moments and transformed once.  Moments are kept halved per axis index
+// (hx = xi / 2, hs = (xi^2 + zeta) / 2), which makes the transform
+//   c = -1: m2 - m1,   c = 0: m0 - 2 m2,   c = +1: m2 + m1.
+// Equilibria enter as deviations from the reference rest state, telescoped
+// over the axes, as in lbm_collide.cuh.
+#pragma once
+
+#include "lbm_stencil.cuh"
+#include "lbm_collide.cuh"
+
+namespace lbm {
+
+// Product moments of a lattice's equilibrium deviation from the reference
+// rest state, divided by the lattice's density:
+//   e_pqr = a_p a_q a_r - r_p r_q r_r,  a = (1, hx, hs), r = (1, 0, hr),
+// telescoped with da = a - r = (0, hx, hd).
+template <class V>
+struct RestDeviation {
+  V h1[3], h2[3], d2[3], r2;
+  template <int P> __device__ __forceinline__ V a(int ax) const { return P == 1 ? h1[ax] : h2[ax]; }
+  template <int P> __device__ __forceinline__ V d(int ax) const { return P == 1 ? h1[ax] : d2[ax]; }
+  // (y, z) part: a_q a_r, and da_q a_r + r_q da_r
+  template <int Qy, int R> __device__ __forceinline__ V ayz() const {
+    if constexpr (Qy == 0) return a<R>(2);
+    else if constexpr (R == 0) return a<Qy>(1);
+    else return vmul(a<Qy>(1), a<R>(2));
+  }
+  template <int Qy, int R> __device__ __forceinline__ V fyz() const {
+    if constexpr (Qy == 0) return d<R>(2);
+    else if constexpr (R == 0) return d<Qy>(1);
+    else if constexpr (Qy == 1) return vmul(h1[1], a<R>(2));
+    else return vfma(d2[1], a<R>(2), vmul(r2, d<R>(2)));
+  }
+  template <int Pp, int Qy, int R> __device__ __forceinline__ V e() const {
+    constexpr bool yz0 = Qy == 0 && R == 0;
+    if constexpr (Pp == 0) return fyz<Qy, R>();
+    else if constexpr (yz0) return d<Pp>(0);
+    else if constexpr (Pp == 1) return vmul(h1[0], ayz<Qy, R>());
+    else return vfma(d2[0], ayz<Qy, R>(), vmul(r2, fyz<Qy, R>()));
+  }
+  // the moment of the rest state itself (zero unless every index is even)
+  template <int Pp, int Qy, int R> static constexpr int rest_power() {
+    return (Pp == 1 || Qy == 1 || R == 1) ? -1 : (Pp + Qy + R) / 2;
+  }
+};
+
+// The 27 velocities of moments given plane by plane (plane<R>(m): m[3q + p]).
+// emit<I>(value) for every velocity but the rest one, rest(value) last; the
+// rest value is the remainder of the zeroth moment m000.
+template <class Scalar, class V, class Plane, class Emit, class Rest>
+__device__ __forceinline__ void from_moments(V m000, Plane&& plane, Emit&& emit, Rest&& rest) {
+  auto xy = [&](auto R_, V (&t)[9]) {
+    V m[9];
+    plane(R_, m);
+    const V two = bcast<V>(Scalar(-2));
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      const V a = m[3 * q], b = m[3 * q + 1], c = m[3 * q + 2];
+      t[3 * q] = vsub(c, b); t[3 * q + 1] = vfma(two, c, a); t[3 * q + 2] = vadd(c, b);
+    }
+#pragma unroll
+    for (int x = 0; x < 3; ++x) {
+      const V a = t[x], b = t[3 + x], c = t[6 + x];
+      t[x] = vsub(c, b); t[3 + x] = vfma(two, c, a); t[6 + x] = vadd(c, b);
+    }
+  };
+  V t1[9], t2[9], s;
+  xy(std::integral_constant<int, 1>{}, t1);
+  xy(std::integral_constant<int, 2>{}, t2);
+  static_for<0, 9>([&](auto K_) {
+    constexpr int k = decltype(K_)::value;
+    const V lo = vsub(t2[k], t1[k]), hi = vadd(t2[k], t1[k]);
+    emit(std::integral_constant<int, k>{}, lo);
+    emit(std::integral_constant<int, 18 + k>{}, hi);
+    const V both = vadd(lo, hi);
+    s = k == 0 ? both : vadd(s, both);
+  });
+  xy(std::integral_constant<int, 0>{}, t1);
+  static_for<0, 9>([&](auto K_) {
+    constexpr int k = decltype(K_)::value;
+    if constexpr (k != 4) {
+      const V v = vsub(t1[k], vadd(t2[k], t2[k]));
+      emit(std::integral_constant<int, 9 + k>{}, v);
+      s = vadd(s, v);
+    }
+  });
+  rest(vsub(m000, s));
+}
+
+template <int M>
+struct Split {
+  static constexpr int NP = (M + 1) / 2;                       // species pairs, species warps
+  static constexpr int WARPS = NP + 2, THREADS = 32 * WARPS;
+  static constexpr int LPN = NP <= 1 ? 1 : (NP <= 2 ? 2 : 4);  // closure lanes per node, a species pair each
+  // Row stride of the closure's per-node pairs: its lanes (32 / LPN
+  // neighbouring nodes of LPN rows) fall in distinct banks.
+  static constexpr int LD = LPN == 1 ? 32 : 32 + 32 / LPN;
+  // Shared memory, in Reals; arrays of pairs first.
+  static constexpr int TAB = 0;                                // [8][LPN] constants, [M][LPN] phi_ab / m_b, C_ab
+  static constexpr int TABC = TAB + 2 * LPN * (8 + 2 * M);     // C_ab as [M a][NP b pairs]
+  static constexpr int STAGE = TABC + 2 * M * NP;              // species populations [27][NP][32] pairs
+  static constexpr int DIF = STAGE + 27 * NP * 64;             // force moments [26][NP][32] pairs
+  static constexpr int MOM = DIF;                              // species moments [4][LPN][LD] pairs (before DIF is written)
+  static constexpr int DIF_SIZE = NP > 1 ? 26 * NP * 64 : 0, MOM_SIZE = 8 * LPN * LD;
+  static constexpr int SP = DIF + (DIF_SIZE > MOM_SIZE ? DIF_SIZE : MOM_SIZE);   // closed species [7][LPN][LD] pairs
+  static constexpr int FG = SP + 14 * LPN * LD;                // f, g populations [27][2][32]
+  static constexpr int ND = FG + 27 * 64;                      // node rows [.][32]
+  static constexpr int REALS = ND + 24 * 32;
+};
+enum SplitTab { ST_RL, ST_YR, ST_IM, ST_CV, ST_CP, ST_MU, ST_LAM, ST_ILAM };
+enum SplitSp { SS_RA, SS_RD, SS_V, SS_BETA = SS_V + 3, SS_TY };
+enum SplitNode { SN_RHOD, SN_J, SN_RHOED = SN_J + 3, SN_S, SN_DT = SN_S + 6, SN_DTH, SN_OM, SN_OM1, SN_CP, SN_HYV,
+                 SN_USP = SN_HYV + 3, SN_RHOSP = SN_USP + 3 };
+static_assert(SN_RHOSP < 24, "node rows");
+
+// Sum of a quantity over the species of a node.
+template <int LPN, class V>
+__device__ __forceinline__ auto species_sum(V v) -> decltype(v.x) {
+  auto s = v.x + v.y;
+#pragma unroll
+  for (int o = LPN / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o, LPN);
+  return s;
+}
+
+// Gauss-Jordan elimination of the M x M system whose rows 2a, 2a + 1 lane a
+// of the group holds (columns diagonally dominant: no pivoting, see
+// sm_eliminate).
+template <int M, int LPN, class V>
+__device__ __forceinline__ void lanes_solve(V (&A)[M], V (&r)[3], int a) {
+  using T = decltype(A[0].x);
+  V dinv = bcast<V>(T(1));
+  auto from = [&](V v, int k) {
+    const T s = k % 2 ? v.y : v.x;
+    return LPN == 1 ? s : __shfl_sync(0xffffffffu, s, k / 2, LPN);
+  };
+#pragma unroll
+  for (int k = 0; k < M; ++k) {
+    const T inv = T(1) / from(A[k], k);
+    V l = vmul(A[k], bcast<V>(-inv));
+    if (a == k / 2) {
+      if (k % 2) { dinv.y = inv; l.y = T(0); } else { dinv.x = inv; l.x = T(0); }
+    }
+#pragma unroll
+    for (int b = k + 1; b < M; ++b) A[b] = vfma(l, bcast<V>(from(A[b], k)), A[b]);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) r[c] = vfma(l, bcast<V>(from(r[c], k)), r[c]);
+  }
+#pragma unroll
+  for (int c = 0; c < 3; ++c) r[c] = vmul(r[c], dinv);
+}
+
+// Node closure, species pair a of node nd (thermo_state, omega1_of, sm_solve
+// and the relaxation times, a lane per species pair).  Species past M hold
+// zeros and identity rows.
+template <int M, class Real>
+__device__ __forceinline__ void split_closure(const DevParams<Real>& p, Real* sm, int nd, int a, bool active,
+                                              unsigned* __restrict__ err) {
+  using C = Split<M>;
+  using V = typename Pair<Real>::T;
+  constexpr int LPN = C::LPN, LD = C::LD;
+  const V* tab = reinterpret_cast<const V*>(sm + C::TAB) + a;
+  auto cst = [&](int k) { return tab[k * LPN]; };
+  const V* mom = reinterpret_cast<const V*>(sm + C::MOM) + a * LD + nd;
+  V* sp = reinterpret_cast<V*>(sm + C::SP) + a * LD + nd;
+  Real* node = sm + C::ND + nd;
+  const V zero = bcast<V>(Real(0));
+  const bool on0 = 2 * a < M, on1 = 2 * a + 1 < M;
+  V rd = zero, ja[3] = {zero, zero, zero};
+  if (on0) {
+    rd = mom[0];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) ja[c] = mom[(c + 1) * LPN * LD];
+  }
+  const Real rho_dev = node[SN_RHOD * 32], rhoE_dev = node[SN_RHOED * 32];
+  Real j[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) j[c] = node[(SN_J + c) * 32];
+  const Real rho = p.RL[M] + rho_dev, inv_rho = Real(1) / rho;
+  const Real u[3] = {j[0] * inv_rho, j[1] * inv_rho, j[2] * inv_rho};
+  Real usp[3], rho_sp, sp_dev;
+  if (!p.weak) {
+    // Eqs. (rhoMATCH), (uMATCH): the slaved species takes the deficits
+    const bool s0 = 2 * a == p.slaved, s1 = 2 * a + 1 == p.slaved;
+    auto match = [&](V& v, Real total) {
+      if (s0) v.x = Real(0);
+      if (s1) v.y = Real(0);
+      const Real d = total - species_sum<LPN>(v);
+      if (s0) v.x = d;
+      if (s1) v.y = d;
+    };
+    match(rd, p.cS + rho_dev);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) { match(ja[c], j[c]); usp[c] = u[c]; }
+    rho_sp = rho;
+    sp_dev = p.cS + rho_dev;
+  } else {
+    sp_dev = species_sum<LPN>(rd);
+    rho_sp = p.Rsp + sp_dev;
+    const Real is = Real(1) / rho_sp;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) usp[c] = species_sum<LPN>(ja[c]) * is;
+  }
+  const V ra = vadd(cst(ST_RL), rd);
+  const V inv_sp = bcast<V>(Real(1) / rho_sp);
+  const V Y = vmul(ra, inv_sp);
+  const V dY = vmul(vfma(cst(ST_YR), bcast<V>(-sp_dev), rd), inv_sp);
+  const V im = cst(ST_IM), cv = cst(ST_CV), cp = cst(ST_CP);
+  const Real inv_m = species_sum<LPN>(vmul(Y, im)), d_inv_m = species_sum<LPN>(vmul(dY, im));
+  const Real Cv = species_sum<LPN>(vmul(Y, cv)), dCv = species_sum<LPN>(vmul(dY, cv));
+  const Real Cp = species_sum<LPN>(vmul(Y, cp));
+  const Real m = Real(1) / inv_m, R = p.R_U * inv_m, dR = p.R_U * d_inv_m;
+  const Real usq = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+  // Eq. (temperature2), T0 = 0
+  const Real dT = (p.cE + rhoE_dev - Real(0.5) * rho * usq - rho_dev * p.Cvr * p.Tr - rho * dCv * p.Tr) / (rho * Cv);
+  const Real T = p.Tr + dT, theta = R * T, dth = dR * T + p.Rr * dT, P = rho * theta;
+  if (a == 0 && active && (!(rho > Real(0)) || !(T > Real(0)) || !(rho_sp > Real(0)))) atomicOr(err, 1u);
+  Real Yb[M];
+#pragma unroll
+  for (int b = 0; b < M; ++b) {
+    const Real y = b % 2 ? Y.y : Y.x;
+    Yb[b] = LPN == 1 ? y : __shfl_sync(0xffffffffu, y, b / 2, LPN);
+  }
+  const V X = vmul(bcast<V>(m), vmul(Y, im));
+  Real om, om1;
+  if (p.omega_is_fixed) {
+    om = p.omega_fixed;
+  } else {
+    // Wilke, Eqs. (viscosityMixture), (wilkePhi); phi = phi_ab / m_b
+    const V* phi = tab + 8 * LPN;
+    V den = zero;
+#pragma unroll
+    for (int b = 0; b < M; ++b) den = vfma(phi[b * LPN], bcast<V>(Yb[b]), den);
+    const V num = vmul(cst(ST_MU), X);
+    V q;
+    q.x = on0 ? num.x / (m * den.x) : Real(0);
+    q.y = on1 ? num.y / (m * den.y) : Real(0);
+    om = Real(2) * P / (P + Real(2) * species_sum<LPN>(q));
+  }
+  if (p.omega1_is_fixed) {
+    om1 = p.omega1_fixed;
+  } else {
+    const Real s1 = species_sum<LPN>(vmul(X, cst(ST_LAM))), s2 = species_sum<LPN>(vmul(X, cst(ST_ILAM)));
+    const Real lam = Real(0.5) * (s1 + Real(1) / s2), pc = P * Cp;
+    om1 = Real(2) * pc / (pc + Real(2) * lam);
+  }
+  // Eqs. (tauab), (tau), (transform12): rows of the system for J_a = rho_a V_a
+  const V* cab = tab + (8 + M) * LPN;
+  const Real tm = p.R_U * T * m;
+  V A[M], r[3], diag = bcast<V>(Real(1)), it = zero;
+  const V hY = vmul(bcast<V>(Real(-0.5)), Y);
+#pragma unroll
+  for (int b = 0; b < M; ++b) {
+    const V itab = vmul(bcast<V>(tm), cab[b * LPN]);
+    const V f = vmul(itab, bcast<V>(Yb[b]));
+    it = vadd(it, f);
+    V h = vmul(bcast<V>(Real(0.5)), f);
+    if (a == b / 2) { if (b % 2) h.y = Real(0); else h.x = Real(0); }
+    diag = vadd(diag, h);
+    A[b] = vmul(hY, itab);
+  }
+#pragma unroll
+  for (int b = 0; b < M; ++b)
+    if (a == b / 2) { if (b % 2) A[b].y = diag.y; else A[b].x = diag.x; }
+#pragma unroll
+  for (int c = 0; c < 3; ++c) r[c] = vfma(ra, bcast<V>(-usp[c]), ja[c]);
+  if constexpr (sizeof(Real) == 4) {
+    // ill-conditioned systems are solved in FP64 (see sm_solve)
+    Real cond = Real(2) * (fmax(diag.x, diag.y) - Real(1));
+#pragma unroll
+    for (int o = LPN / 2; o > 0; o >>= 1) cond = fmax(cond, __shfl_xor_sync(0xffffffffu, cond, o, LPN));
+    const bool ill = cond + Real(1) > p.cond_bound;
+    if (__any_sync(0xffffffffu, ill)) {
+      const double tm64 = (double)p.R_U * (double)T * (double)m;
+      double2 A64[M], r64[3], d64 = make_double2(1.0, 1.0);
+#pragma unroll
+      for (int b = 0; b < M; ++b) {
+        const double hx = on0 ? 0.5 * tm64 * p.Cab64[on0 ? 2 * a : 0][b] : 0.0;
+        const double hy = on1 ? 0.5 * tm64 * p.Cab64[on1 ? 2 * a + 1 : 0][b] : 0.0;
+        if (2 * a != b) d64.x += hx * (double)Yb[b];
+        if (2 * a + 1 != b) d64.y += hy * (double)Yb[b];
+        A64[b] = make_double2(-hx * (double)Y.x, -hy * (double)Y.y);
+      }
+#pragma unroll
+      for (int b = 0; b < M; ++b)
+        if (a == b / 2) { if (b % 2) A64[b].y = d64.y; else A64[b].x = d64.x; }
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        r64[c] = make_double2((double)ja[c].x - (double)ra.x * (double)usp[c], (double)ja[c].y - (double)ra.y * (double)usp[c]);
+        const double sr = species_sum<LPN>(r64[c]);
+        r64[c].x -= (double)Y.x * sr;
+        r64[c].y -= (double)Y.y * sr;
+      }
+      lanes_solve<M, LPN>(A64, r64, a);
+      lanes_solve<M, LPN>(A, r, a);
+      if (ill) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) { r[c].x = (Real)r64[c].x; r[c].y = (Real)r64[c].y; }
+      }
+    } else {
+      lanes_solve<M, LPN>(A, r, a);
+    }
+  } else {
+    lanes_solve<M, LPN>(A, r, a);
+  }
+  V ir;
+  ir.x = (on0 && ra.x > p.rho_eps * rho_sp) ? Real(1) / ra.x : Real(0);
+  ir.y = (on1 && ra.y > p.rho_eps * rho_sp) ? Real(1) / ra.y : Real(0);
+  V beta;                                          // dt / (2 tau_a + dt)
+  beta.x = it.x / (Real(2) + it.x);
+  beta.y = it.y / (Real(2) + it.y);
+  sp[SS_RA * LPN * LD] = ra;
+  sp[SS_RD * LPN * LD] = rd;
+  sp[SS_BETA * LPN * LD] = beta;
+  sp[SS_TY * LPN * LD] = vmul(bcast<V>(tm), Y);
+  const V cr = vmul(cp, ra);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const V v = vmul(r[c], ir);
+    sp[(SS_V + c) * LPN * LD] = v;
+    const Real h = species_sum<LPN>(vmul(cr, v));  // sum_a (H_a / T) rho_a V_a
+    if (a == 0) node[(SN_HYV + c) * 32] = h;
+  }
+  if (a == 0) {
+    node[SN_DT * 32] = dT; node[SN_DTH * 32] = dth;
+    node[SN_OM * 32] = om; node[SN_OM1 * 32] = om1; node[SN_CP * 32] = Cp;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) node[(SN_USP + c) * 32] = usp[c];
+    node[SN_RHOSP * 32] = rho_sp;
+  }
+}
+
+// Where the host takes this kernel (constant heats, exact closure): from four
+// species.  There a thread per node needs 255 registers and a stage of 690 to
+// 1080 bytes, which leaves 4 to 8 warps on an SM.  Measured (GB300), collide
+// here against a thread per node: eight species FP32 128^3 1.95 against 3.18
+// ms, BF16 192^3 8.0 against 15.7 ms; but two species FP32 256^3 6.7 against
+// 3.3 ms, three species FP32 45x75x101 0.186 against 0.129 ms.
+#ifndef LBM_SPLIT_MIN_M
+#define LBM_SPLIT_MIN_M 4
+#endif
+template <int M, class Real, class Store>
+constexpr bool kSplit = M >= LBM_SPLIT_MIN_M;
+
+// Blocks per SM asked of the register allocator.
+#ifndef LBM_SPLIT_THREADS
+#define LBM_SPLIT_THREADS 576
+#endif
+template <int M, class Real>
+constexpr int split_min_blocks() {
+  constexpr long long bytes = (long long)Split<M>::REALS * sizeof(Real) + 1024;
+  constexpr int fit = (int)(227LL * 1024 / bytes);
+  constexpr int want = sizeof(Real) == 8 ? 1 : LBM_SPLIT_THREADS / Split<M>::THREADS;
+  return want < 1 ? 1 : (want < fit ? want : (fit < 1 ? 1 : fit));
+}
+
+// BND: 0 periodic, 1 bounce-back walls normal to x, 2 opposed-jets frame.
+template <int M, class Real, class Store, int PAR, int BND>
+__global__ void __launch_bounds__(Split<M>::THREADS, split_min_blocks<M, Real>())
+collide_split_kernel(const __grid_constant__ DevParams<Real> p, Store* __restrict__ pops, Real* __restrict__ side,
+                     unsigned* __restrict__ err, int ntiles, const __grid_constant__ PlaneOffsets po) {
+  using C = Split<M>;
+  using V = typename Pair<Real>::T;
+  constexpr int NP = C::NP, LPN = C::LPN, LD = C::LD;
+  constexpr bool EQ = kEqCodec<Store, Real>, WALL = BND == 1;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  Real* const sm = reinterpret_cast<Real*>(smem_raw);
+  const int tid = threadIdx.x, lane = tid & 31, role = tid >> 5;
+  V* const stage = reinterpret_cast<V*>(sm + C::STAGE) + lane;
+  Real* const fg = sm + C::FG + lane;
+  V* const dif = reinterpret_cast<V*>(sm + C::DIF) + lane;
+  Real* const node = sm + C::ND + lane;
+  const long long N = p.N;
+
+  // Constants by species pair (a lane-indexed read of the parameter block
+  // would be serialised).
+  {
+    Real* t = sm + C::TAB;
+    for (int k = tid; k < 2 * LPN; k += C::THREADS) {
+      const bool on = k < M;
+      const int a = on ? k : 0;
+      t[ST_RL * 2 * LPN + k] = on ? p.RL[a] : Real(0);
+      t[ST_YR * 2 * LPN + k] = on ? p.Yr[a] : Real(0);
+      t[ST_IM * 2 * LPN + k] = on ? p.inv_mass[a] : Real(0);
+      t[ST_CV * 2 * LPN + k] = on ? p.Cv_a[a] : Real(0);
+      t[ST_CP * 2 * LPN + k] = on ? p.Cp_a[a] : Real(0);
+      t[ST_MU * 2 * LPN + k] = on ? p.mu[a] : Real(0);
+      t[ST_LAM * 2 * LPN + k] = on ? p.lam[a] : Real(0);
+      t[ST_ILAM * 2 * LPN + k] = on ? p.inv_lam[a] : Real(0);
+    }
+    t += 16 * LPN;
+    for (int k = tid; k < M * 2 * LPN; k += C::THREADS) {
+      const int b = k / (2 * LPN), a = k % (2 * LPN);
+      t[k] = a < M ? p.phi[a][b] * p.inv_mass[b] : Real(0);
+      t[2 * LPN * M + k] = a < M ? p.Cab[a][b] : Real(0);
+    }
+    for (int k = tid; k < 2 * M * NP; k += C::THREADS) {
+      const int a = k / (2 * NP), b = k % (2 * NP);
+      sm[C::TABC + k] = b < M ? p.Cab[a][b] : Real(0);
+    }
+  }
+
+  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const long long n_raw = (long long)tile * 32 + lane;
+    bool active = n_raw < N;
+    const long long n = active ? n_raw : N - 1;
+    if constexpr (BND == 2) {
+      const long long x = n % p.nx, y = (n / p.nx) % p.ny;
+      if (x == 0 || x == p.nx - 1 || y == 0 || y == p.ny - 1) active = false;
+    }
+    const unsigned act = __ballot_sync(0xffffffffu, active);
+    const Nbr nb = make_nbr(p, n);
+    // Byte offset of slot `slot` at node `nn` within a lattice; lattice L of it.
+    auto off = [&](int slot, long long nn) { return nn * (long long)sizeof(Store) + po.off[slot]; };
+    auto at = [&](int L, long long o) {
+      return reinterpret_cast<Store*>(reinterpret_cast<char*>(pops) + (long long)L * po.off[Q] + o);
+    };
+
+    // ---- 1. load: the velocities shared out over the warps -------------------
+#pragma unroll 1
+    for (int i = role; i < Q; i += C::WARPS) {
+      const int cz = i / 9 - 1, cy = (i / 3) % 3 - 1, cx = i % 3 - 1;
+      const bool refl = WALL && arrives_from_wall_c(nb, cx);
+      const unsigned xs = cx == 0 ? nb.xs[1] : (cx > 0 ? nb.xs[0] : nb.xs[2]);
+      const unsigned ys = cy == 0 ? nb.ys[1] : (cy > 0 ? nb.ys[0] : nb.ys[2]);
+      const unsigned zs = cz == 0 ? nb.zs[1] : (cz > 0 ? nb.zs[0] : nb.zs[2]);
+      const long long snd = refl ? n : (long long)(xs + ys + zs);        // n - c_i, or n itself at a wall
+      const bool own = PAR == 0 || refl;                                 // aa_read_loc
+      const long long o = off(own ? i : Q - 1 - i, own ? n : snd);
+      Store raw[M + 2];
+#pragma unroll
+      for (int L = 0; L < M + 2; ++L) raw[L] = *at(L, o);
+      V v[NP];
+      Real fv, gv, th = Real(0);
+      if constexpr (EQ) {
+        float dth;
+        const RecLoad<M> rl(eq_rec_buf(side, N, p.rec_w, 1 - PAR), N, snd, p.weak);
+        eq_shift_dir<M>(p, rl, refl, cx, cy, cz, v, fv, gv, dth);
+        th = p.thr + dth;
+      } else {
+        if (i != 13) th = side_ld(side + SP_THR * N + snd);
+#pragma unroll
+        for (int q = 0; q < NP; ++q) v[q] = bcast<V>(Real(0));
+        fv = gv = Real(0);
+      }
+      if (i != 13) {
+        // the deferred terms (incoming_corr_th)
+        Real kc = Real(0);
+        if (cx) { const Real k = side_ld(side + (SP_K + 0) * N + snd); kc += cx > 0 ? k : -k; }
+        if (cy) { const Real k = side_ld(side + (SP_K + 1) * N + snd); kc += cy > 0 ? k : -k; }
+        if (cz) { const Real k = side_ld(side + (SP_K + 2) * N + snd); kc += cz > 0 ? k : -k; }
+        const Real w0 = Real(1) - th, w1 = Real(0.5) * th;
+        const Real cg = (cx ? w1 : w0) * (cy ? w1 : w0) * (cz ? w1 : w0) * kc;
+        gv += refl ? -cg : cg;
+        if (cx * cx + cy * cy + cz * cz == 1) {
+          const Real X = side_ld(side + (SP_X + (cx ? 0 : (cy ? 1 : 2))) * N + snd);
+          const Real cf = (cx + cy + cz > 0 ? Real(0.5) : Real(-0.5)) * X;
+          fv += refl ? -cf : cf;
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < NP; ++q) {
+        V d;
+        d.x = codec_decode<Store, Real>(p, raw[2 * q], 2 * q);
+        d.y = 2 * q + 1 < M ? codec_decode<Store, Real>(p, raw[2 * q + 1], 2 * q + 1) : Real(0);
+        d = EQ ? vadd(d, v[q]) : d;
+        if (2 * q + 1 >= M) d.y = Real(0);
+        stage[(i * NP + q) * 32] = d;
+      }
+      fg[(2 * i) * 32] = codec_decode<Store, Real>(p, raw[M], M) + fv;
+      fg[(2 * i + 1) * 32] = codec_decode<Store, Real>(p, raw[M + 1], M + 1) + gv;
+    }
+    __syncthreads();
+
+    // ---- 2. moments, each warp its own lattices' ---------------------------
+    Real q3[3] = {Real(0), Real(0), Real(0)};     // g: energy flux
+    if (role < NP) {
+      V r4[4];
+      static_for<0, Q>([&](auto I_) {
+        constexpr int i = decltype(I_)::value;
+        const V v = stage[(i * NP + role) * 32];
+        r4[0] = i == 0 ? v : vadd(r4[0], v);
+        static_for<0, 3>([&](auto A_) {
+          constexpr int c = c_of(i, decltype(A_)::value);
+          V& t = r4[1 + decltype(A_)::value];
+          if constexpr (i == 0) t = vsub(bcast<V>(Real(0)), v);         // c = (-1, -1, -1)
+          else if constexpr (c > 0) t = vadd(t, v);
+          else if constexpr (c < 0) t = vsub(t, v);
+        });
+      });
+      V* mom = reinterpret_cast<V*>(sm + C::MOM) + role * LD + lane;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) mom[c * LPN * LD] = r4[c];
+    } else if (role == NP) {
+      Real rho_dev = Real(0), j[3] = {Real(0), Real(0), Real(0)}, S[6] = {Real(0), Real(0), Real(0), Real(0), Real(0), Real(0)};
+      static_for<0, Q>([&](auto I_) {
+        constexpr int i = decltype(I_)::value;
+        constexpr int cx = cx_of(i), cy = cy_of(i), cz = cz_of(i);
+        const Real v = fg[2 * i * 32];
+        rho_dev += v;
+        if (cx) { j[0] += cx * v; S[0] += v; }
+        if (cy) { j[1] += cy * v; S[1] += v; }
+        if (cz) { j[2] += cz * v; S[2] += v; }
+        if (cx && cy) S[3] += (cx * cy) * v;
+        if (cx && cz) S[4] += (cx * cz) * v;
+        if (cy && cz) S[5] += (cy * cz) * v;
+      });
+      node[SN_RHOD * 32] = rho_dev;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) node[(SN_J + c) * 32] = j[c];
+#pragma unroll
+      for (int c = 0; c < 6; ++c) node[(SN_S + c) * 32] = S[c];
+    } else {
+      Real rhoE_dev = Real(0);
+      static_for<0, Q>([&](auto I_) {
+        constexpr int i = decltype(I_)::value;
+        const Real v = fg[(2 * i + 1) * 32];
+        rhoE_dev += v;
+        if (cx_of(i)) q3[0] += cx_of(i) * v;
+        if (cy_of(i)) q3[1] += cy_of(i) * v;
+        if (cz_of(i)) q3[2] += cz_of(i) * v;
+      });
+      node[SN_RHOED * 32] = rhoE_dev;
+    }
+    __syncthreads();
+
+    // ---- 3. node closure -----------------------------------------------------
+    if (role < LPN) split_closure<M, Real>(p, sm, tid / LPN, tid % LPN, (act >> (tid / LPN)) & 1u, err);
+    __syncthreads();
+
+    // ---- 4. update, store --------------------------------------------------
+    const Nbr nbw = opaque(nb);
+    const long long nw = opaque_idx(n);
+    const Real dT = node[SN_DT * 32];
+    if (role < NP) {
+      const int a0 = 2 * role;
+      const bool two = M % 2 == 0 || role < NP - 1;
+      const V* sp = reinterpret_cast<const V*>(sm + C::SP) + lane;
+      auto pick = [&](int k) { return sp[(k * LPN + role) * LD]; };
+      V z, dz;                                        // R_a T and R_a (T - T_r)
+      z.x = p.R_a[a0]; z.y = p.R_a[a0 + (two ? 1 : 0)];
+      RestDeviation<V> e;
+      const V half = bcast<V>(Real(0.5));
+      e.r2 = vmul(z, bcast<V>(Real(0.5) * p.Tr));
+      dz = vmul(z, bcast<V>(dT));
+      z = vmul(z, bcast<V>(p.Tr + dT));
+      V b1[3], b2[3], f1[3], f2[3];                   // halved moments of u + V; differences Psi(u) - Psi(u + V)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const Real x = node[(SN_USP + c) * 32];
+        const V Vc = pick(SS_V + c);
+        const V x2 = bcast<V>(x * x);
+        e.h1[c] = bcast<V>(Real(0.5) * x);
+        e.h2[c] = vmul(half, vadd(x2, z));
+        e.d2[c] = vmul(half, vadd(x2, dz));
+        f1[c] = vmul(bcast<V>(Real(-0.5)), Vc);
+        f2[c] = vmul(f1[c], vadd(bcast<V>(x + x), Vc));
+        b1[c] = vsub(e.h1[c], f1[c]);
+        b2[c] = vsub(e.h2[c], f2[c]);
+      }
+      // Force moments of each species (density apart): a_p a_q a_r - b_p b_q b_r
+      // with f = a - b, telescoped: f_p a_q a_r + b_p (f_q a_r + b_q f_r).
+      V own[NP > 1 ? 1 : 26];
+      auto fsel = [&](auto P_, int ax) { return decltype(P_)::value == 1 ? f1[ax] : f2[ax]; };
+      auto bsel = [&](auto P_, int ax) { return decltype(P_)::value == 1 ? b1[ax] : b2[ax]; };
+      static_for<0, 9>([&](auto K_) {
+        constexpr int qy = decltype(K_)::value % 3, r = decltype(K_)::value / 3;
+        using QC = std::integral_constant<int, qy>;
+        using RC = std::integral_constant<int, r>;
+        V E;
+        if constexpr (qy == 0 && r == 0) E = bcast<V>(Real(0));
+        else if constexpr (qy == 0) E = fsel(RC{}, 2);
+        else if constexpr (r == 0) E = fsel(QC{}, 1);
+        else E = vfma(fsel(QC{}, 1), e.template a<r>(2), vmul(bsel(QC{}, 1), fsel(RC{}, 2)));
+        static_for<0, 3>([&](auto P_) {
+          constexpr int pp = decltype(P_)::value, t = pp + 3 * qy + 9 * r - 1;
+          if constexpr (t >= 0) {
+            V D;
+            if constexpr (pp == 0) D = E;
+            else if constexpr (qy == 0 && r == 0) D = fsel(P_, 0);
+            else D = vfma(fsel(P_, 0), e.template ayz<qy, r>(), vmul(bsel(P_, 0), E));
+            if constexpr (NP > 1) dif[(t * NP + role) * 32] = D;
+            else own[t] = D;
+          }
+        });
+      });
+      // weights of the force moments: (beta_a - 1) (Y_a / tau_ab) rho_b, species b in pairs
+      const V beta = pick(SS_BETA), tY = pick(SS_TY), ra = pick(SS_RA), rd = pick(SS_RD);
+      const V bm = vsub(beta, bcast<V>(Real(1))), w = vmul(bm, tY);
+      const V cv = vsub(bcast<V>(Real(1)), vadd(beta, beta));       // 1 - 2 beta
+      const V ce = EQ ? vsub(bcast<V>(Real(0)), cv) : vadd(beta, beta);
+      V k0[NP], k1[NP];
+#pragma unroll
+      for (int q = 0; q < NP; ++q) {
+        const V* cab = reinterpret_cast<const V*>(sm + C::TABC) + a0 * NP + q;
+        const V rb = sp[(SS_RA * LPN + q) * LD];
+        k0[q] = vmul(vmul(bcast<V>(w.x), cab[0]), rb);
+        k1[q] = two ? vmul(vmul(bcast<V>(w.y), cab[NP]), rb) : bcast<V>(Real(0));
+      }
+      if constexpr (NP > 1) asm volatile("bar.sync 1, %0;" ::"n"(NP * 32) : "memory");
+      const V cra = vmul(ce, ra), crd = vmul(ce, rd);
+      V rest_w[4];                                     // crd times the rest moments
+      rest_w[0] = crd;
+#pragma unroll
+      for (int k = 1; k < 4; ++k) rest_w[k] = vmul(rest_w[k - 1], e.r2);
+      auto plane = [&](auto R_, V (&mm)[9]) {
+        constexpr int r = decltype(R_)::value;
+        static_for<0, 9>([&](auto K_) {
+          constexpr int k = decltype(K_)::value, pp = k % 3, qy = k / 3, t = pp + 3 * qy + 9 * r - 1;
+          constexpr int rp = RestDeviation<V>::template rest_power<pp, qy, r>();
+          V s;
+          if constexpr (t < 0) {
+            s = crd;
+          } else {
+            if constexpr (rp >= 0) s = vfma(cra, e.template e<pp, qy, r>(), rest_w[rp]);
+            else s = vmul(cra, e.template e<pp, qy, r>());
+            V s0 = bcast<V>(Real(0)), s1 = s0;
+#pragma unroll
+            for (int q = 0; q < NP; ++q) {
+              V D;
+              if constexpr (NP > 1) D = dif[(t * NP + q) * 32]; else D = own[t];
+              s0 = q == 0 ? vmul(k0[q], D) : vfma(k0[q], D, s0);
+              s1 = q == 0 ? vmul(k1[q], D) : vfma(k1[q], D, s1);
+            }
+            s.x += s0.x + s0.y;
+            s.y += s1.x + s1.y;
+          }
+          mm[k] = s;
+        });
+      };
+      auto put = [&](auto I_, V val) {
+        constexpr int i = decltype(I_)::value;
+        long long nn; int slot;
+        aa_write_loc<WALL>(PAR, nbw, nw, i, nn, slot);
+        const long long o = off(slot, nn);
+        const V out = vfma(cv, stage[(i * NP + role) * 32], val);
+        if (active) {
+          codec_store<Store, Real>(p, at(a0, o), 0, a0, out.x);
+          if (two) codec_store<Store, Real>(p, at(a0 + 1, o), 0, a0 + 1, out.y);
+        }
+      };
+      from_moments<Real, V>(crd, plane, put, [&](V val) { put(std::integral_constant<int, 13>{}, val); });
+    } else {
+      const Real rho_dev = node[SN_RHOD * 32], dth = node[SN_DTH * 32], om = node[SN_OM * 32], om1 = node[SN_OM1 * 32];
+      const Real rho = p.RL[M] + rho_dev, inv_rho = Real(1) / rho, theta = p.thr + dth, T = p.Tr + dT;
+      const Real j[3] = {node[SN_J * 32], node[(SN_J + 1) * 32], node[(SN_J + 2) * 32]};
+      const Real u[3] = {j[0] * inv_rho, j[1] * inv_rho, j[2] * inv_rho};
+      const Real P = rho * theta, Cp = node[SN_CP * 32];
+      const Real usq = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+      if (role == NP) {
+        if (active) {
+          // side fields (Eqs. Xalpha, corrFourier; see collide_node)
+          const Real a3 = Real(1) - Real(3) * theta;
+#pragma unroll
+          for (int c = 0; c < 3; ++c) side[(SP_PHI + c) * N + n] = j[c] * a3 - rho * u[c] * u[c] * u[c];
+          side[SP_COM * N + n] = Real(1) / om - Real(0.5);
+          side[SP_CP * N + n] = Cp;
+          side[SP_S * N + n] = Real(0.5) * (Real(2) - om1) * P * T / theta;
+          side[SP_TH * N + n] = theta;
+        }
+        // momentum lattice, Eqs. (feq), (fwithcorrection)
+        RestDeviation<Real> e;
+        e.r2 = Real(0.5) * p.thr;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          const Real x2 = u[c] * u[c];
+          e.h1[c] = Real(0.5) * u[c];
+          e.h2[c] = Real(0.5) * (x2 + theta);
+          e.d2[c] = Real(0.5) * (x2 + dth);
+        }
+        const Real cv = Real(1) - om, ce = EQ ? -cv : om;
+        const Real cra = ce * rho, crd = ce * rho_dev;
+        const Real rest_w[4] = {crd, crd * e.r2, crd * e.r2 * e.r2, crd * e.r2 * e.r2 * e.r2};
+        auto plane = [&](auto R_, Real (&mm)[9]) {
+          constexpr int r = decltype(R_)::value;
+          static_for<0, 9>([&](auto K_) {
+            constexpr int k = decltype(K_)::value, pp = k % 3, qy = k / 3;
+            constexpr int rp = RestDeviation<Real>::template rest_power<pp, qy, r>();
+            if constexpr (pp + qy + r == 0) mm[k] = crd;
+            else if constexpr (rp >= 0) mm[k] = cra * e.template e<pp, qy, r>() + rest_w[rp];
+            else mm[k] = cra * e.template e<pp, qy, r>();
+          });
+        };
+        auto put = [&](auto I_, Real val) {
+          constexpr int i = decltype(I_)::value;
+          long long nn; int slot;
+          aa_write_loc<WALL>(PAR, nbw, nw, i, nn, slot);
+          if (active) codec_store<Store, Real>(p, at(M, off(slot, nn)), 0, M, cv * fg[2 * i * 32] + val);
+        };
+        from_moments<Real, Real>(crd, plane, put, [&](Real val) { put(std::integral_constant<int, 13>{}, val); });
+      } else {
+        // energy lattice (see collide_node for the closed form)
+        const Real rhoE_dev = node[SN_RHOED * 32];
+        const Real dP = rho_dev * theta + p.RL[M] * dth;
+        const Real hk = Cp * T + Real(0.5) * usq, inv_theta = Real(1) / theta;
+        const Real Gc = rho * (hk + theta) * Real(0.5) * inv_theta;
+        const Real dE0 = rhoE_dev - Real(1.5) * dP - Gc * usq;
+        Real dZ[3], mvec[3], qt[3];
+        {
+          const Real z1 = Real(1) - Real(3) * theta;
+          const Real zb = Real(0.5) * (z1 * dP - Real(3) * dth * p.Pr);
+#pragma unroll
+          for (int c = 0; c < 3; ++c) dZ[c] = zb + z1 * Gc * u[c] * u[c];
+          Real S[6];
+#pragma unroll
+          for (int c = 0; c < 6; ++c) S[c] = node[(SN_S + c) * 32];
+          Real dP6[6];                                       // Pi - P^eq
+#pragma unroll
+          for (int c = 0; c < 3; ++c) dP6[c] = p.cPi + S[c] - dP - rho * u[c] * u[c];
+          dP6[3] = S[3] - rho * u[0] * u[1];
+          dP6[4] = S[4] - rho * u[0] * u[2];
+          dP6[5] = S[5] - rho * u[1] * u[2];
+          const Real qb[3] = {q3[0] - (u[0] * dP6[0] + u[1] * dP6[3] + u[2] * dP6[4]),
+                              q3[1] - (u[0] * dP6[3] + u[1] * dP6[1] + u[2] * dP6[5]),
+                              q3[2] - (u[0] * dP6[4] + u[1] * dP6[5] + u[2] * dP6[2])};
+          const Real rY = p.weak ? rho / node[SN_RHOSP * 32] : Real(1);
+          const Real c1 = om1 * T * rY, dw = om - om1;
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            const Real qeq = hk * j[c];
+            qt[c] = qeq * inv_theta;
+            mvec[c] = (om * qeq + dw * (qb[c] - qeq) + c1 * node[(SN_HYV + c) * 32]) * inv_theta;
+          }
+        }
+        if constexpr (EQ) {
+          if (active) {
+            EqRec<M> r;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) { r.u[c] = u[c]; r.usp[c] = node[(SN_USP + c) * 32]; }
+            r.dth = dth; r.dT = dT; r.drho = rho_dev; r.dE0 = dE0;
+            r.Gq = Gc * inv_theta; r.hq = hk * rho * inv_theta;
+#pragma unroll
+            for (int a = 0; a < M; ++a) {
+              const V d = reinterpret_cast<const V*>(sm + C::SP)[(SS_RD * LPN + a / 2) * LD + lane];
+              r.ra[a] = a % 2 ? d.y : d.x;
+            }
+            store_rec<M>(eq_rec_buf(side, N, p.rec_w, PAR), N, n, p.weak, r);
+          }
+        }
+        const Real w0 = Real(1) - theta, w1 = Real(0.5) * theta;          // Eq. (w0)
+        const Real r0 = Real(1) - p.thr, r1 = Real(0.5) * p.thr;
+        const Real d0 = -dth, d1 = Real(0.5) * dth;
+        Real s_g = Real(0);
+        static_for<0, 13>([&](auto I_) {
+          constexpr int i = decltype(I_)::value, o = Q - 1 - i;
+          constexpr int cx = cx_of(i), cy = cy_of(i), cz = cz_of(i);
+          long long node_i, node_o; int slot_i, slot_o;
+          aa_write_loc<WALL>(PAR, nbw, nw, i, node_i, slot_i);
+          aa_write_loc<WALL>(PAR, nbw, nw, o, node_o, slot_o);
+          const Real uc = dotc<Real, i>(u);
+          const Real cc = Real(0.5) * Real(c2_of(i));
+          const Real ucu = Gc * uc * uc * inv_theta;
+          const Real dEi = dE0 + cc * rho_dev + ucu;
+          const Real wx = cx ? w1 : w0, wy = cy ? w1 : w0, wz = cz ? w1 : w0;
+          const Real rx = cx ? r1 : r0, ry = cy ? r1 : r0;
+          const Real dx = cx ? d1 : d0, dy = cy ? d1 : d0, dzz = cz ? d1 : d0;
+          const Real wi = wx * wy * wz;
+          const Real dwi = dx * wy * wz + rx * dy * wz + rx * ry * dzz;
+          const Real eg = wi * dEi + dwi * energy_rest(p, M, c2_of(i)) + BdotZ<Real, i>(dZ);
+          s_g += eg + eg;
+          const Real fl = wi * dotc<Real, i>(mvec);
+          const Real gi = fg[(2 * i + 1) * 32], go = fg[(2 * o + 1) * 32];
+          const Real out_i = gi + om * (eg - gi) + fl;
+          const Real out_o = go + om * (eg - go) - fl;
+          if (active) {
+            const Real sq = EQ ? wi * dotc<Real, i>(qt) : Real(0);
+            codec_store<Store, Real>(p, at(M + 1, off(slot_i, node_i)), 0, M + 1, EQ ? out_i - (eg + sq) : out_i);
+            codec_store<Store, Real>(p, at(M + 1, off(slot_o, node_o)), 0, M + 1, EQ ? out_o - (eg - sq) : out_o);
+          }
+        });
+        long long nn; int slot;
+        aa_write_loc<WALL>(PAR, nbw, nw, 13, nn, slot);
+        const Real e13 = rhoE_dev - s_g;
+        const Real gr = fg[(2 * 13 + 1) * 32];
+        const Real out = gr + om * (e13 - gr);
+        if (active) codec_store<Store, Real>(p, at(M + 1, off(slot, nn)), 0, M + 1, EQ ? out - e13 : out);
+      }
+    }
+    __syncthreads();      // the next tile's moments take the place of this tile's
+  }
+}
+
+}  // namespace lbm
