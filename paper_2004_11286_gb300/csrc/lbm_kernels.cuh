@@ -227,6 +227,15 @@ diag_final_kernel(const double* __restrict__ partials, int nblocks, int nv, doub
 // ---------------------------------------------------------------------------
 // Host launchers.
 // ---------------------------------------------------------------------------
+// Grids of at most this many nodes take the stencil passes with a thread per
+// node and field: the row-blocked form leaves a 1024-node grid on one SM.
+// Measured (GB300, first / second pass, us): FP64 1024 nodes 10.6 / 6.3
+// against 40.1 / 22.9, 65,536 nodes 36 / 15 against 41 / 23, 262,144 nodes
+// 99 / 35 against 75 / 40; FP32 4096 nodes 7.1 / 6.4 against 8.2 / 6.5, 32,768
+// nodes 8.3 / 7.6 against 8.3 / 8.1, 65,536 nodes 10.3 / 8.8 against 9.7 / 8.5.
+template <class Real>
+constexpr long long kFieldStencilNodes = sizeof(Real) == 8 ? 131072 : 32768;
+
 inline unsigned grid_for(long long N, int block) { return (unsigned)((N + block - 1) / block); }
 
 template <int M, class Real, class Store>
@@ -264,20 +273,26 @@ struct Launch {
       collide_kernel<M, Real, Store, 1, CL, LD, WALL><<<grid_for(c.N, BS), BS, smem, c.stream>>>(
           P(c), (Store*)c.pops, side, c.err, c.mlp_img, c.mlp_stats, po);
   }
+  static int sm_count() {
+    static const int sms = [] {
+      int dev = 0, v = 1;
+      cudaGetDevice(&dev);
+      cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+      return v;
+    }();
+    return sms;
+  }
   template <int BND>
   static void split_launch(const LaunchCtx& c, int parity, Real* side) {
     using C = Split<M>;
     constexpr size_t smem = C::REALS * sizeof(Real);
-    static int resident = 0;                     // blocks the device holds at once
-    if (!resident) {
-      int dev = 0, sms = 1, per = 1;
-      cudaGetDevice(&dev);
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    static const int resident = [&] {            // blocks the device holds at once
+      int per = 1;
       cudaFuncSetAttribute(collide_split_kernel<M, Real, Store, 0, BND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       cudaFuncSetAttribute(collide_split_kernel<M, Real, Store, 1, BND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, collide_split_kernel<M, Real, Store, 0, BND>, C::THREADS, smem);
-      resident = sms * (per > 0 ? per : 1);
-    }
+      return sm_count() * (per > 0 ? per : 1);
+    }();
     PlaneOffsets po;
     for (int k = 0; k < (M + 2) * Q; ++k) po.off[k] = (long long)k * c.N * (long long)sizeof(Store);
     const int ntiles = (int)grid_for(c.N, 32);
@@ -294,36 +309,25 @@ struct Launch {
     // Walls normal to x (bounce-back), the opposed-jets frame: register
     // loads, exact closure (the host refuses both with the network closure).
     if constexpr (CL == 0 && kSplit<M, Real, Store>) {
-      if constexpr (EQ) {
+      const long long most = kSplitTilesPerSm<M, Real, Store> * 32LL * sm_count();
+      if (!P(c).tvar && (kSplitTilesPerSm<M, Real, Store> == 0 || c.N <= most)) {
         if (P(c).wall_x) split_launch<1>(c, parity, side);
+        else if (P(c).frame) split_launch<EQ ? 0 : 2>(c, parity, side);
         else split_launch<0>(c, parity, side);
-      } else {
-        if (P(c).tvar) collide_launch<0, 0>(c, parity, side);
-        else if (P(c).wall_x) split_launch<1>(c, parity, side);
-        else if (P(c).frame) split_launch<2>(c, parity, side);
-        else split_launch<0>(c, parity, side);
+        return;
       }
-      return;
+    }
+    if constexpr (CL == 0 && kSplit<M, Real, Store> && kSplitTilesPerSm<M, Real, Store> == 0) {
+      // only temperature-dependent heats get here (FP64, FP32, periodic)
+      if constexpr (!EQ) collide_launch<0, 0>(c, parity, side);
+    } else if constexpr (CL == 0) {
+      constexpr bool bulk = LBM_COLLIDE_BULK && M >= LBM_COLLIDE_BULK_MIN_M && std::is_same<Real, Store>::value;
+      if (P(c).wall_x) collide_launch<0, 0, 1>(c, parity, side);
+      else if (P(c).frame) collide_launch<0, 0, EQ ? 0 : 2>(c, parity, side);
+      else if (bulk && P(c).nx % collide_block<M, Real, 0, Store>() == 0) collide_launch<0, bulk>(c, parity, side);
+      else collide_launch<0, 0>(c, parity, side);
     } else {
-    if constexpr (CL == 0) {
-      if (P(c).wall_x) {
-        collide_launch<0, 0, 1>(c, parity, side);
-        return;
-      }
-      if constexpr (!EQ) {
-        if (P(c).frame) {
-          collide_launch<0, 0, 2>(c, parity, side);
-          return;
-        }
-      }
-    }
-    if constexpr (CL == 0 && LBM_COLLIDE_BULK && M >= LBM_COLLIDE_BULK_MIN_M && std::is_same<Real, Store>::value) {
-      if (P(c).nx % collide_block<M, Real, 0, Store>() == 0) {
-        collide_launch<0, 1>(c, parity, side);
-        return;
-      }
-    }
-    collide_launch<CL, 0>(c, parity, side);
+      collide_launch<CL, 0>(c, parity, side);
     }
   }
   static cudaError_t step(const LaunchCtx& c, int parity) {
@@ -344,13 +348,18 @@ struct Launch {
       frame_side_kernel<Real><<<fgrid, BLOCK_LIGHT, 0, c.stream>>>(P(c), side, 0);
     }
     if (c.ev) cudaEventRecord(c.ev[1], c.stream);
-    // Row-blocked stencils (ROWV nodes per thread) where rows split evenly.
+    // Row-blocked stencils (ROWV nodes per thread) where rows split evenly; a
+    // thread per node and field on grids of few nodes.
+    const bool few = c.N <= kFieldStencilNodes<Real>;
     const bool rows = P(c).nx % ROWV == 0 && !P(c).tvar;
-    if (rows) grad_GK_row_kernel<Real><<<grid_for(c.N / ROWV, BLOCK_LIGHT), BLOCK_LIGHT, 0, c.stream>>>(P(c), side);
+    const dim3 fg(grid_for(c.N, BLOCK_FIELD), 4), fx(fg.x, 3);
+    if (few) grad_GK_field_kernel<Real><<<fg, BLOCK_FIELD, 0, c.stream>>>(P(c), side);
+    else if (rows) grad_GK_row_kernel<Real><<<grid_for(c.N / ROWV, BLOCK_LIGHT), BLOCK_LIGHT, 0, c.stream>>>(P(c), side);
     else grad_GK_kernel<Real><<<grid_for(c.N, BLOCK_LIGHT), BLOCK_LIGHT, 0, c.stream>>>(P(c), side);
     if (frame) frame_side_kernel<Real><<<fgrid, BLOCK_LIGHT, 0, c.stream>>>(P(c), side, 1);
     if (c.ev) cudaEventRecord(c.ev[2], c.stream);
-    if (rows) grad_X_row_kernel<Real><<<grid_for(c.N / ROWV, BLOCK_LIGHT), BLOCK_LIGHT, 0, c.stream>>>(P(c), side);
+    if (few) grad_X_field_kernel<Real><<<fx, BLOCK_FIELD, 0, c.stream>>>(P(c), side);
+    else if (rows) grad_X_row_kernel<Real><<<grid_for(c.N / ROWV, BLOCK_LIGHT), BLOCK_LIGHT, 0, c.stream>>>(P(c), side);
     else grad_X_kernel<Real><<<grid_for(c.N, BLOCK_LIGHT), BLOCK_LIGHT, 0, c.stream>>>(P(c), side);
     if (frame) frame_side_kernel<Real><<<fgrid, BLOCK_LIGHT, 0, c.stream>>>(P(c), side, 2);
     if (c.ev) cudaEventRecord(c.ev[3], c.stream);

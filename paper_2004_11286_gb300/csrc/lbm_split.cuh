@@ -350,17 +350,23 @@ __device__ __forceinline__ void split_closure(const DevParams<Real>& p, Real* sm
   }
 }
 
-// Where the host takes this kernel (constant heats, exact closure): from four
-// species.  There a thread per node needs 255 registers and a stage of 690 to
-// 1080 bytes, which leaves 4 to 8 warps on an SM.  Measured (GB300), collide
-// here against a thread per node: eight species FP32 128^3 1.95 against 3.18
-// ms, BF16 192^3 8.0 against 15.7 ms; but two species FP32 256^3 6.7 against
-// 3.3 ms, three species FP32 45x75x101 0.186 against 0.129 ms.
-#ifndef LBM_SPLIT_MIN_M
-#define LBM_SPLIT_MIN_M 4
-#endif
+// Where the host takes this kernel (constant heats, exact closure).
+//   * From four species always.  There a thread per node needs 255 registers
+//     and a stage of 690 to 1080 bytes, which leaves 4 to 8 warps on an SM.
+//     Measured (GB300), collide here against a thread per node: eight species
+//     FP32 128^3 1.95 against 3.18 ms, BF16 192^3 8.0 against 15.7 ms, FP64 64^3
+//     4.3 against 13.2 ms.
+//   * With two or three species on grids of few tiles per SM, where the time
+//     is one node's latency: three species FP64 1024 nodes 59 against 121 us
+//     (16,384 nodes 156 against 132), FP32 1024 nodes 12.1 against 14.8 us
+//     (16,384 nodes 14.3 against 15.7, 32,768 nodes 22.4 against 16.6), BF16 1024
+//     nodes 14.2 against 22.4 us; two species FP64 1024 nodes 52 against 97 us,
+//     BF16 4096 nodes 15.7 against 18.3 us, but FP32 1024 nodes 12.0 against 10.3.
 template <int M, class Real, class Store>
-constexpr bool kSplit = M >= LBM_SPLIT_MIN_M;
+constexpr bool kSplit = M >= 3 || (M == 2 && (sizeof(Real) == 8 || sizeof(Store) == 2));
+// The largest number of tiles per SM taken (0: any).
+template <int M, class Real, class Store>
+constexpr int kSplitTilesPerSm = M >= 4 ? 0 : (sizeof(Real) == 8 ? 1 : 3);
 
 // Blocks per SM asked of the register allocator.
 #ifndef LBM_SPLIT_THREADS

@@ -422,6 +422,75 @@ __device__ __forceinline__ void grad_X_row(const DevParams<Real>& p, Real* __res
     }
 }
 
+// Small grids: a thread per node and field, so that few nodes still spread
+// over the SMs.  field 0..2: G_field; 3: K and the copy of theta.
+template <class Real>
+__device__ __forceinline__ void grad_GK_field(const DevParams<Real>& p, Real* __restrict__ side, long long n, int field) {
+  if (n >= p.N) return;
+  const long long N = p.N;
+  const Nbr nb = make_nbr(p, n);
+  if (field < 3) {
+    const Real* phi = side + (SP_PHI + field) * N;
+    Real d = Real(0);
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+      const int c = field == 0 ? cx_of(i) : (field == 1 ? cy_of(i) : cz_of(i));
+      if (c == 0) continue;
+      Real v = phi[nb.idx(cx_of(i), cy_of(i), cz_of(i))];
+      if (field == 0 && ((c < 0 && (nb.wall & 1u)) || (c > 0 && (nb.wall & 2u)))) v = -v;   // Phi_x is odd beyond a wall
+      d += (c * iso_w<Real>(i)) * v;
+    }
+    side[(SP_G + field) * N + n] = Real(3) * side[SP_COM * N + n] * d;
+    return;
+  }
+  const Real Tn = p.tvar ? side[SP_T * N + n] : Real(0);
+  Real dc[3] = {Real(0), Real(0), Real(0)};
+#pragma unroll
+  for (int i = 0; i < Q; ++i) {
+    if (i == 13) continue;
+    const long long nn = nb.idx(cx_of(i), cy_of(i), cz_of(i));
+    Real cp = side[SP_CP * N + nn];
+    if (p.tvar) cp += Tn * (side[SP_HC2 * N + nn] + Tn * side[SP_HC3 * N + nn]);
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+      if (c_of(i, c)) dc[c] += (c_of(i, c) * iso_w<Real>(i)) * cp;
+  }
+  const Real sv = Real(3) * side[SP_S * N + n];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) side[(SP_K + c) * N + n] = sv * dc[c];
+  side[SP_THR * N + n] = side[SP_TH * N + n];
+}
+template <class Real>
+__device__ __forceinline__ void grad_X_field(const DevParams<Real>& p, Real* __restrict__ side, long long n, int field) {
+  if (n >= p.N) return;
+  const long long N = p.N;
+  const Nbr nb = make_nbr(p, n);
+  const Real* g = side + (SP_G + field) * N;
+  Real d = Real(0);
+#pragma unroll
+  for (int i = 0; i < Q; ++i) {
+    const int c = field == 0 ? cx_of(i) : (field == 1 ? cy_of(i) : cz_of(i));
+    if (c) d += (c * iso_w<Real>(i)) * g[nb.idx(cx_of(i), cy_of(i), cz_of(i))];
+  }
+  side[(SP_X + field) * N + n] = Real(-3) * d;
+}
+constexpr int BLOCK_FIELD = 32;
+template <class Real>
+__global__ void __launch_bounds__(BLOCK_FIELD)
+grad_GK_field_kernel(const __grid_constant__ DevParams<Real> p, Real* __restrict__ side) {
+  if (blockIdx.y == 0) grad_GK_field<Real>(p, side, gtid(), 0);
+  else if (blockIdx.y == 1) grad_GK_field<Real>(p, side, gtid(), 1);
+  else if (blockIdx.y == 2) grad_GK_field<Real>(p, side, gtid(), 2);
+  else grad_GK_field<Real>(p, side, gtid(), 3);
+}
+template <class Real>
+__global__ void __launch_bounds__(BLOCK_FIELD)
+grad_X_field_kernel(const __grid_constant__ DevParams<Real> p, Real* __restrict__ side) {
+  if (blockIdx.y == 0) grad_X_field<Real>(p, side, gtid(), 0);
+  else if (blockIdx.y == 1) grad_X_field<Real>(p, side, gtid(), 1);
+  else grad_X_field<Real>(p, side, gtid(), 2);
+}
+
 // LBM_GK_MINB > 0 sets a minimum of resident blocks per SM (FP32); by
 // default the compiler chooses (64 registers, four blocks of 256).
 #ifndef LBM_GK_MINB

@@ -1,5 +1,6 @@
 """The collide whose warps share out a node's lattices, against the oracle:
-every species count it is built for, grids that end inside a 32-node tile or
+every species count it is built for (two and three on small grids; grids past
+that line, with a thread per node, are held to the same), grids that end inside a 32-node tile or
 fill none, walls, both couplings, and the FP64 re-solve of ill-conditioned
 systems (a condition bound of 1 sends every node there).
 
@@ -24,6 +25,11 @@ pytestmark = pytest.mark.gpu
     (4, "fp32", (3, 4, 5), {"fp64_cond_bound": 1.0}), (7, "fp32", (3, 4, 5), {"fp64_cond_bound": 1.0}),
     (8, "fp32", (3, 4, 5), {"fp64_cond_bound": 1.0, "coupling": "weak"}),
     (4, "fp32", (3, 4, 5), {"omega_fixed": 1.2, "omega1_fixed": 0.9}),
+    (2, "fp64", (3, 5, 7), {"coupling": "weak"}), (3, "fp32", (2, 3, 35), {"coupling": "weak"}), (3, "fp64", (1, 2, 40), {"walls_x": True}),
+    (3, "fp32", (3, 4, 5), {"fp64_cond_bound": 1.0}),
+    # past the small-grid lines: 6144 nodes in FP64, 15,600 in FP32
+    (2, "fp64", (12, 16, 32), {}), (3, "fp64", (12, 16, 32), {"walls_x": True}), (3, "fp64", (12, 17, 33), {"coupling": "weak"}),
+    (3, "fp32", (24, 25, 26), {}), (3, "fp32", (24, 25, 26), {"walls_x": True, "coupling": "weak"}),
 ])
 def test_split_collide(M, precision, shape, kw):
     wl = W.random_mixture(M=M, shape=shape, seed=20 + M, velocity=0.03)
