@@ -386,11 +386,8 @@ __device__ __forceinline__ void collide_node(const DevParams<Real>& p, Store* __
                                                       (cx > 0 ? nbk.xs[0] : nbk.xs[2]));
         const RowLoad<M> in(p, side, rin, snd, cy, cz);
         float2 v[NP];
-        float fv, gv, dth;
-        eq_shift_dir<M>(p, in.rec, refl, cx, cy, cz, v, fv, gv, dth);
-        const float th = p.thr + dth, w0 = 1.0f - th, w1 = 0.5f * th, sg = refl ? -1.0f : 1.0f;
-        gv += sg * w1 * (cy ? w1 : w0) * (cz ? w1 : w0) * (cx * in.k[0] + cy * in.k[1] + cz * in.k[2]);
-        if (cy == 0 && cz == 0) fv += sg * 0.5f * cx * in.x;
+        float fv, gv;
+        edge_terms<M>(p, in, refl, cx, cy, cz, v, fv, gv);
         const int at = tid - lane + k;
 #pragma unroll
         for (int a = 0; a < M; ++a) sps[(a * Q + i) * BS + at] = a % 2 ? v[a / 2].y : v[a / 2].x;
@@ -432,11 +429,11 @@ __device__ __forceinline__ void collide_node(const DevParams<Real>& p, Store* __
       }
 #pragma unroll
       for (int q = 0; q < NP; ++q) {
-        t.sp[2][q].x = __shfl_up_sync(0xffffffffu, t.sp[2][q].x, 1);
-        t.sp[0][q].x = __shfl_down_sync(0xffffffffu, t.sp[0][q].x, 1);
+        t.sp[q][2].x = __shfl_up_sync(0xffffffffu, t.sp[q][2].x, 1);
+        t.sp[q][0].x = __shfl_down_sync(0xffffffffu, t.sp[q][0].x, 1);
         if (2 * q + 1 < M) {
-          t.sp[2][q].y = __shfl_up_sync(0xffffffffu, t.sp[2][q].y, 1);
-          t.sp[0][q].y = __shfl_down_sync(0xffffffffu, t.sp[0][q].y, 1);
+          t.sp[q][2].y = __shfl_up_sync(0xffffffffu, t.sp[q][2].y, 1);
+          t.sp[q][0].y = __shfl_down_sync(0xffffffffu, t.sp[q][0].y, 1);
         }
       }
       t.f[2] = __shfl_up_sync(0xffffffffu, t.f[2], 1);
@@ -447,7 +444,7 @@ __device__ __forceinline__ void collide_node(const DevParams<Real>& p, Store* __
 #pragma unroll
         for (int a = 0; a < M; ++a) {
           const float s = sps[(a * Q + i0 + x) * BS + tid];
-          if (a % 2) t.sp[x][a / 2].y = s; else t.sp[x][a / 2].x = s;
+          if (a % 2) t.sp[a / 2][x].y = s; else t.sp[a / 2][x].x = s;
         }
         t.f[x] = sfg[(i0 + x) * BS + tid];
         t.g[x] = sfg[(Q + i0 + x) * BS + tid];
@@ -463,7 +460,7 @@ __device__ __forceinline__ void collide_node(const DevParams<Real>& p, Store* __
         for (int x = 0; x < 3; ++x) {
           v[x].x = codec_decode<Store, float>(p, raw[x][2 * q], 2 * q);
           v[x].y = 2 * q + 1 < M ? codec_decode<Store, float>(p, raw[x][2 * q + 1], 2 * q + 1) : 0.0f;
-          v[x] = add2(v[x], t.sp[x][q]);
+          v[x] = add2(v[x], t.sp[q][x]);
           sps[((2 * q) * Q + i0 + x) * BS + tid] = v[x].x;
           if (2 * q + 1 < M) sps[((2 * q + 1) * Q + i0 + x) * BS + tid] = v[x].y;
         }

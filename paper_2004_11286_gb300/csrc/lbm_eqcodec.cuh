@@ -286,102 +286,129 @@ __device__ __forceinline__ void eq_shift_dir(const DevParams<float>& p, const Re
 // lattice (as eq_shift_dir) and, on f and g, the deferred terms
 // c . X / 2 (faces) and w(theta) c . K.  The (y, z) factors, and all that
 // depends on the sender alone, are formed once for the three.
+// (y, z) factors of a row for the species: per axis Psi_c = a + be z.
+struct RowSpecies {
+  float by, bz, ay, az, x2, hx;
+  float T;
+  int k2;
+  __device__ __forceinline__ RowSpecies(float ux, float uy, float uz, float T_, int cy, int cz)
+      : by(cy ? 0.5f : -1.0f), bz(cz ? 0.5f : -1.0f), x2(ux * ux), hx(0.5f * ux), T(T_), k2(cy * cy + cz * cz) {
+    ay = by * uy * uy + 0.5f * cy * uy + (cy ? 0.0f : 1.0f);
+    az = bz * uz * uz + 0.5f * cz * uz + (cz ? 0.0f : 1.0f);
+  }
+};
+// Shifts of species a0, a1 with densities RL + d.
+__device__ __forceinline__ void row_species(const DevParams<float>& p, const RowSpecies& r, int a0, int a1, float2 d,
+                                            float2 (&out)[3]) {
+  const float2 z = mul2(make_float2(p.R_a[a0], p.R_a[a1]), bcast<float2>(r.T));
+  const float2 ra = add2(make_float2(p.RL[a0], p.RL[a1]), d);
+  const float2 yz = mul2(mul2(ra, fma2(bcast<float2>(r.by), z, bcast<float2>(r.ay))),
+                         fma2(bcast<float2>(r.bz), z, bcast<float2>(r.az)));
+  const float2 s = add2(bcast<float2>(r.x2), z), hs = mul2(bcast<float2>(0.5f), s);
+  const float2 r0 = make_float2(-p.bref[a0][r.k2], -p.bref[a1][r.k2]);
+  const float2 r1 = make_float2(-p.bref[a0][r.k2 + 1], -p.bref[a1][r.k2 + 1]);
+  out[0] = fma2(yz, sub2(hs, bcast<float2>(r.hx)), r1);
+  out[1] = fma2(yz, sub2(bcast<float2>(1.0f), s), r0);
+  out[2] = fma2(yz, add2(hs, bcast<float2>(r.hx)), r1);
+}
+// f and g: A, B the record's first two float4s, hq, K, and the component x of
+// X that a face velocity of the row needs.
+__device__ __forceinline__ void row_fg(const DevParams<float>& p, int M, float4 A, float4 B, float hq,
+                                       const float (&k)[3], float x, int cy, int cz, float (&f)[3], float (&g)[3]) {
+  const float dth = B.x, drho = B.y;
+  const float by = cy ? 0.5f : -1.0f, bz = cz ? 0.5f : -1.0f;
+  const int kyz = cy * cy + cz * cz;
+  const float x2 = A.x * A.x, hx = 0.5f * A.x;
+  const float r1 = 0.5f * p.thr, r0 = 1.0f - p.thr;
+  const float ry = cy ? r1 : r0, rz = cz ? r1 : r0, ryz = ry * rz;
+  const float wy = by * dth, wz = bz * dth, wx = 0.5f * dth;    // w_c(theta) - w_c(theta_r); x: c = 0 gives -dth
+  {
+    const float rho = p.RL[M] + drho;
+    const float dy = by * A.y * A.y + 0.5f * cy * A.y + wy, dz = bz * A.z * A.z + 0.5f * cz * A.z + wz;
+    const float az = rz + dz, ayz = (ry + dy) * az, fyz = dy * az + ry * dz;
+    const float hs = 0.5f * (x2 + dth), cf = 0.5f * x;
+    const float e1 = r1 * fyz, d1 = drho * (r1 * ryz);
+    f[0] = rho * ((hs - hx) * ayz + e1) + d1;
+    f[1] = rho * (r0 * fyz - (hs + hs) * ayz) + drho * (r0 * ryz);
+    f[2] = rho * ((hs + hx) * ayz + e1) + d1;
+    if (kyz == 0) { f[0] -= cf; f[2] += cf; }
+    if (kyz == 1) f[1] += (cy + cz) * cf;
+  }
+  const float oz = rz + wz, oyz = (ry + wy) * oz, dyz = wy * oz + ry * wz;
+  const float w1 = (r1 + wx) * oyz, w0 = (r0 - dth) * oyz;
+  const float c0 = (r0 * dyz - dth * oyz) * energy_rest(p, M, kyz), c1 = (wx * oyz + r1 * dyz) * energy_rest(p, M, kyz + 1);
+  const float uyz = cy * A.y + cz * A.z, kk = cy * k[1] + cz * k[2];
+  const float e0 = B.z + 0.5f * kyz * drho + kk, e1 = e0 + 0.5f * drho;
+  const float um = uyz - A.x, up = uyz + A.x;
+  g[0] = w1 * (e1 + um * (B.w * um + hq) - k[0]) + c1;
+  g[1] = w0 * (e0 + uyz * (B.w * uyz + hq)) + c0;
+  g[2] = w1 * (e1 + up * (B.w * up + hq) + k[0]) + c1;
+  if (kyz <= 1) {
+    const float theta = p.thr + dth, z1 = 1.0f - 3.0f * theta;
+    const float zb = 0.5f * (z1 * (drho * theta + p.RL[M] * dth) - 3.0f * dth * p.Pr), zG = z1 * B.w * theta;
+    if (kyz == 0) {
+      const float bx = 0.5f * (zb + zG * x2);
+      g[0] -= bx;
+      g[1] += 3.0f * zb + zG * (x2 + A.y * A.y + A.z * A.z);
+      g[2] -= bx;
+    } else {
+      g[1] -= 0.5f * (zb + zG * (cy ? A.y * A.y : A.z * A.z));
+    }
+  }
+}
 template <int M>
 struct RowTerms {
   static constexpr int NP = (M + 1) / 2;
-  float2 sp[3][NP];
+  float2 sp[NP][3];
   float f[3], g[3];
 };
-// What a sender's RowTerms are formed from, as loaded: its record, K, and the
-// component of X that a face velocity of the row needs.
-template <int M>
-struct RowLoad {
-  RecLoad<M> rec;
+// K and the component of X that a face velocity of the row needs.
+struct RowSide {
   float k[3], x;
-  __device__ __forceinline__ RowLoad(const DevParams<float>& p, const float* __restrict__ side,
-                                     const float* __restrict__ rin, long long snd, int cy, int cz)
-      : rec(rin, p.N, snd, p.weak) {
-    const long long N = p.N;
+  __device__ __forceinline__ RowSide(const float* __restrict__ side, long long N, long long snd, int cy, int cz) {
     k[0] = __ldg(side + (SP_K + 0) * N + snd);
     k[1] = cy ? __ldg(side + (SP_K + 1) * N + snd) : 0.0f;
     k[2] = cz ? __ldg(side + (SP_K + 2) * N + snd) : 0.0f;
     x = cy * cz == 0 ? __ldg(side + (SP_X + (cy ? 1 : (cz ? 2 : 0))) * N + snd) : 0.0f;
   }
 };
+// What a sender's RowTerms are formed from, as loaded.
+template <int M>
+struct RowLoad {
+  RecLoad<M> rec;
+  RowSide s;
+  __device__ __forceinline__ RowLoad(const DevParams<float>& p, const float* __restrict__ side,
+                                     const float* __restrict__ rin, long long snd, int cy, int cz)
+      : rec(rin, p.N, snd, p.weak), s(side, p.N, snd, cy, cz) {}
+};
 template <int M>
 __device__ __forceinline__ void row_terms(const DevParams<float>& p, const RowLoad<M>& in, int cy, int cz,
                                           RowTerms<M>& out) {
   constexpr int NT = RecLoad<M>::NT, NP = (M + 1) / 2;
-  const float4 A = in.rec.q[0], B = in.rec.q[1];
+  const float4 A = in.rec.q[0], W = p.weak ? in.rec.q[2 + NT] : A;
   float t[4 * NT];
 #pragma unroll
   for (int k = 0; k < NT; ++k) {
     const float4 c = in.rec.q[2 + k];
     t[4 * k] = c.x; t[4 * k + 1] = c.y; t[4 * k + 2] = c.z; t[4 * k + 3] = c.w;
   }
-  const float dth = B.x, drho = B.y;
-  const float by = cy ? 0.5f : -1.0f, bz = cz ? 0.5f : -1.0f, gy = 0.5f * cy, gz = 0.5f * cz;
-  const int kyz = cy * cy + cz * cz;
-  const float x2 = A.x * A.x, hx = 0.5f * A.x;
-  const float qy = by * A.y * A.y + gy * A.y, qz = bz * A.z * A.z + gz * A.z;
-  {
-    float sx2 = x2, shx = hx, sy = qy, sz = qz;
-    if (p.weak) {
-      const float4 w = in.rec.q[2 + NT];
-      sx2 = w.x * w.x; shx = 0.5f * w.x;
-      sy = by * w.y * w.y + gy * w.y; sz = bz * w.z * w.z + gz * w.z;
-    }
-    const float2 ay = bcast<float2>(sy + (cy ? 0.0f : 1.0f)), az = bcast<float2>(sz + (cz ? 0.0f : 1.0f));
-    const float2 T = bcast<float2>(p.Tr + A.w), px = bcast<float2>(shx), mx = bcast<float2>(-shx);
+  const RowSpecies r(W.x, W.y, W.z, p.Tr + A.w, cy, cz);
 #pragma unroll
-    for (int q = 0; q < NP; ++q) {
-      const int a0 = 2 * q, a1 = 2 * q + 1 < M ? 2 * q + 1 : 2 * q;
-      const float2 z = mul2(make_float2(p.R_a[a0], p.R_a[a1]), T);
-      const float2 ra = add2(make_float2(p.RL[a0], p.RL[a1]), make_float2(t[a0], t[2 * q + 1]));
-      const float2 yz = mul2(mul2(ra, fma2(bcast<float2>(by), z, ay)), fma2(bcast<float2>(bz), z, az));
-      const float2 s = add2(bcast<float2>(sx2), z), hs = mul2(bcast<float2>(0.5f), s);
-      const float2 r0 = make_float2(-p.bref[a0][kyz], -p.bref[a1][kyz]);
-      const float2 r1 = make_float2(-p.bref[a0][kyz + 1], -p.bref[a1][kyz + 1]);
-      out.sp[0][q] = fma2(yz, add2(hs, mx), r1);
-      out.sp[1][q] = fma2(yz, sub2(bcast<float2>(1.0f), s), r0);
-      out.sp[2][q] = fma2(yz, add2(hs, px), r1);
-    }
-  }
-  const float r1 = 0.5f * p.thr, r0 = 1.0f - p.thr;
-  const float ry = cy ? r1 : r0, rz = cz ? r1 : r0, ryz = ry * rz;
-  const float wy = by * dth, wz = bz * dth, wx = 0.5f * dth;    // w_c(theta) - w_c(theta_r); x: c = 0 gives -dth
-  {
-    const float rho = p.RL[M] + drho;
-    const float dy = qy + wy, dz = qz + wz, az = rz + dz, ayz = (ry + dy) * az, fyz = dy * az + ry * dz;
-    const float hs = 0.5f * (x2 + dth), cf = 0.5f * in.x;
-    const float e1 = r1 * fyz, d1 = drho * (r1 * ryz);
-    out.f[0] = rho * ((hs - hx) * ayz + e1) + d1;
-    out.f[1] = rho * (r0 * fyz - (hs + hs) * ayz) + drho * (r0 * ryz);
-    out.f[2] = rho * ((hs + hx) * ayz + e1) + d1;
-    if (kyz == 0) { out.f[0] -= cf; out.f[2] += cf; }
-    if (kyz == 1) out.f[1] += (cy + cz) * cf;
-  }
-  const float oz = rz + wz, oyz = (ry + wy) * oz, dyz = wy * oz + ry * wz;
-  const float w1 = (r1 + wx) * oyz, w0 = (r0 - dth) * oyz;
-  const float c0 = (r0 * dyz - dth * oyz) * energy_rest(p, M, kyz), c1 = (wx * oyz + r1 * dyz) * energy_rest(p, M, kyz + 1);
-  const float uyz = cy * A.y + cz * A.z, kk = cy * in.k[1] + cz * in.k[2];
-  const float e0 = B.z + 0.5f * kyz * drho + kk, e1 = e0 + 0.5f * drho;
-  const float um = uyz - A.x, up = uyz + A.x, hq = t[M];
-  out.g[0] = w1 * (e1 + um * (B.w * um + hq) - in.k[0]) + c1;
-  out.g[1] = w0 * (e0 + uyz * (B.w * uyz + hq)) + c0;
-  out.g[2] = w1 * (e1 + up * (B.w * up + hq) + in.k[0]) + c1;
-  if (kyz <= 1) {
-    const float theta = p.thr + dth, z1 = 1.0f - 3.0f * theta;
-    const float zb = 0.5f * (z1 * (drho * theta + p.RL[M] * dth) - 3.0f * dth * p.Pr), zG = z1 * B.w * theta;
-    if (kyz == 0) {
-      const float bx = 0.5f * (zb + zG * x2);
-      out.g[0] -= bx;
-      out.g[1] += 3.0f * zb + zG * (x2 + A.y * A.y + A.z * A.z);
-      out.g[2] -= bx;
-    } else {
-      out.g[1] -= 0.5f * (zb + zG * (cy ? A.y * A.y : A.z * A.z));
-    }
-  }
+  for (int q = 0; q < NP; ++q)
+    row_species(p, r, 2 * q, 2 * q + 1 < M ? 2 * q + 1 : 2 * q, make_float2(t[2 * q], t[2 * q + 1]), out.sp[q]);
+  row_fg(p, M, A, in.rec.q[1], t[M], in.s.k, in.s.x, cy, cz, out.f, out.g);
+}
+// The same for one velocity (c_x given) of one sender, c_x = -1 or 1: every
+// lattice's shift and deferred term, with the sender's signs reversed where
+// the population was reflected by a wall (refl).
+template <int M>
+__device__ __forceinline__ void edge_terms(const DevParams<float>& p, const RowLoad<M>& in, bool refl, int cx, int cy,
+                                           int cz, float2 (&sp)[(M + 1) / 2], float& f, float& g) {
+  float dth;
+  eq_shift_dir<M>(p, in.rec, refl, cx, cy, cz, sp, f, g, dth);
+  const float th = p.thr + dth, w0 = 1.0f - th, w1 = 0.5f * th, sg = refl ? -1.0f : 1.0f;
+  g += sg * w1 * (cy ? w1 : w0) * (cz ? w1 : w0) * (cx * in.s.k[0] + cy * in.s.k[1] + cz * in.s.k[2]);
+  if (cy == 0 && cz == 0) f += sg * 0.5f * cx * in.s.x;
 }
 
 // The record of a node from its coupled moments, in FP64 (initialisation

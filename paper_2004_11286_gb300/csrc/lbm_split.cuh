@@ -2,11 +2,12 @@
 // shared out over the warps of a block.
 //
 // A block takes tiles of 32 nodes, one per lane.  Per tile:
-//   1. the warps share out the 27 velocities: for each, the populations of
-//      every lattice are loaded, decoded, given the terms still due
-//      (lbm_stencil.cuh) and staged in shared memory.  The velocity is data of
-//      a loop, not unrolled: with 16-bit storage the unrolled decoding of the
-//      senders' equilibria overflows the instruction cache;
+//   1. the warps share out the velocities (16-bit storage: the nine rows of
+//      three, each in two parts): the populations of every lattice are
+//      loaded, decoded, given the terms still due (lbm_stencil.cuh,
+//      lbm_eqcodec.cuh) and staged in shared memory.  The velocity is data of a
+//      loop, not unrolled: unrolled, 16-bit decoding overflows the
+//      instruction cache;
 //   2. warp r < NP takes the species pair (2r, 2r + 1), its two species the
 //      lanes of paired FP32 instructions, warp NP takes f, warp NP + 1 takes
 //      g, and each sums its lattices' moments;
@@ -354,7 +355,7 @@ __device__ __forceinline__ void split_closure(const DevParams<Real>& p, Real* sm
 //   * From four species always.  There a thread per node needs 255 registers
 //     and a stage of 690 to 1080 bytes, which leaves 4 to 8 warps on an SM.
 //     Measured (GB300), collide here against a thread per node: eight species
-//     FP32 128^3 1.95 against 3.18 ms, BF16 192^3 8.0 against 15.7 ms, FP64 64^3
+//     FP32 128^3 1.95 against 3.18 ms, BF16 192^3 7.5 against 15.7 ms, FP64 64^3
 //     4.3 against 13.2 ms.
 //   * With two or three species on grids of few tiles per SM, where the time
 //     is one node's latency: three species FP64 1024 nodes 59 against 121 us
@@ -436,65 +437,171 @@ collide_split_kernel(const __grid_constant__ DevParams<Real> p, Store* __restric
     }
     const unsigned act = __ballot_sync(0xffffffffu, active);
     const Nbr nb = make_nbr(p, n);
-    // Byte offset of slot `slot` at node `nn` within a lattice; lattice L of it.
-    auto off = [&](int slot, long long nn) { return nn * (long long)sizeof(Store) + po.off[slot]; };
-    auto at = [&](int L, long long o) {
-      return reinterpret_cast<Store*>(reinterpret_cast<char*>(pops) + (long long)L * po.off[Q] + o);
-    };
+    // Lattice 0's slot `slot` at node `nn`; lattice L is po.off[L * Q] further.
+    auto slot_at = [&](int slot, long long nn) { return reinterpret_cast<char*>(pops + nn) + po.off[slot]; };
+    auto lat = [&](char* q, int L) { return reinterpret_cast<Store*>(q + po.off[L * Q]); };
 
-    // ---- 1. load: the velocities shared out over the warps -------------------
+    // ---- 1. load -------------------------------------------------------------
+    // 16-bit storage: rows shared out over the warps.  A row is the three
+    // velocities of one (c_y, c_z), in two parts: 0 its species but, from
+    // five, the last pair, 1 the rest.  What a population lacks is formed at
+    // its sender's x and handed to the neighbouring lane (lbm_eqcodec.cuh);
+    // needL / needR: the lane's sender at x - 1 / x + 1 is in no lane of the warp.
+    auto ysel = [&](const Nbr& b, int cy) { return cy == 0 ? b.ys[1] : (cy > 0 ? b.ys[0] : b.ys[2]); };   // of y - c_y
+    auto zsel = [&](const Nbr& b, int cz) { return cz == 0 ? b.zs[1] : (cz > 0 ? b.zs[0] : b.zs[2]); };
+    const bool needL = EQ && active && (lane == 0 || nb.xs[1] == 0);
+    const bool needR = EQ && active && (lane == 31 || (int)nb.xs[1] == p.nx - 1);
+    if constexpr (EQ) {
+      const float* const rin = eq_rec_buf(side, N, p.rec_w, 1 - PAR);
+      const unsigned long long need = (unsigned long long)__ballot_sync(0xffffffffu, needL) |
+                                      ((unsigned long long)__ballot_sync(0xffffffffu, needR) << 32);
+      const int cnt = 9 * __popcll(need);
 #pragma unroll 1
-    for (int i = role; i < Q; i += C::WARPS) {
-      const int cz = i / 9 - 1, cy = (i / 3) % 3 - 1, cx = i % 3 - 1;
-      const bool refl = WALL && arrives_from_wall_c(nb, cx);
-      const unsigned xs = cx == 0 ? nb.xs[1] : (cx > 0 ? nb.xs[0] : nb.xs[2]);
-      const unsigned ys = cy == 0 ? nb.ys[1] : (cy > 0 ? nb.ys[0] : nb.ys[2]);
-      const unsigned zs = cz == 0 ? nb.zs[1] : (cz > 0 ? nb.zs[0] : nb.zs[2]);
-      const long long snd = refl ? n : (long long)(xs + ys + zs);        // n - c_i, or n itself at a wall
-      const bool own = PAR == 0 || refl;                                 // aa_read_loc
-      const long long o = off(own ? i : Q - 1 - i, own ? n : snd);
-      Store raw[M + 2];
+      for (int e = tid; e < cnt; e += C::THREADS) {
+        unsigned long long rest = need;
+        for (int k = e / 9; k > 0; --k) rest &= rest - 1;
+        const int who = __ffsll((long long)rest) - 1, row = e % 9;
+        const int cx = who < 32 ? 1 : -1, cy = row % 3 - 1, cz = row / 3 - 1, k = who & 31;
+        const long long nk = (long long)tile * 32 + k;
+        const Nbr nbk = make_nbr(p, nk);
+        const bool refl = WALL && arrives_from_wall_c(nbk, cx);
+        const long long snd = refl ? nk : (long long)(zsel(nbk, cz) + ysel(nbk, cy) + (cx > 0 ? nbk.xs[0] : nbk.xs[2]));
+        const RowLoad<M> in(p, side, rin, snd, cy, cz);
+        float2 v[NP];
+        float fv, gv;
+        edge_terms<M>(p, in, refl, cx, cy, cz, v, fv, gv);
+        const int i = (cx + 1) + 3 * row;
 #pragma unroll
-      for (int L = 0; L < M + 2; ++L) raw[L] = *at(L, o);
-      V v[NP];
-      Real fv, gv, th = Real(0);
-      if constexpr (EQ) {
-        float dth;
-        const RecLoad<M> rl(eq_rec_buf(side, N, p.rec_w, 1 - PAR), N, snd, p.weak);
-        eq_shift_dir<M>(p, rl, refl, cx, cy, cz, v, fv, gv, dth);
-        th = p.thr + dth;
-      } else {
-        if (i != 13) th = side_ld(side + SP_THR * N + snd);
-#pragma unroll
-        for (int q = 0; q < NP; ++q) v[q] = bcast<V>(Real(0));
-        fv = gv = Real(0);
+        for (int q = 0; q < NP; ++q) stage[i * NP * 32 + q * 32 + k - lane] = v[q];
+        fg[2 * i * 32 + k - lane] = fv;
+        fg[(2 * i + 1) * 32 + k - lane] = gv;
       }
-      if (i != 13) {
-        // the deferred terms (incoming_corr_th)
-        Real kc = Real(0);
-        if (cx) { const Real k = side_ld(side + (SP_K + 0) * N + snd); kc += cx > 0 ? k : -k; }
-        if (cy) { const Real k = side_ld(side + (SP_K + 1) * N + snd); kc += cy > 0 ? k : -k; }
-        if (cz) { const Real k = side_ld(side + (SP_K + 2) * N + snd); kc += cz > 0 ? k : -k; }
-        const Real w0 = Real(1) - th, w1 = Real(0.5) * th;
-        const Real cg = (cx ? w1 : w0) * (cy ? w1 : w0) * (cz ? w1 : w0) * kc;
-        gv += refl ? -cg : cg;
-        if (cx * cx + cy * cy + cz * cz == 1) {
-          const Real X = side_ld(side + (SP_X + (cx ? 0 : (cy ? 1 : 2))) * N + snd);
-          const Real cf = (cx + cy + cz > 0 ? Real(0.5) : Real(-0.5)) * X;
-          fv += refl ? -cf : cf;
+      __syncthreads();
+    }
+    if constexpr (EQ) {
+      // Warps take the two parts in turn: WARPS may be even.
+      const float* const rin = eq_rec_buf(side, N, p.rec_w, 1 - PAR);
+#pragma unroll 1
+      for (int it = role, turn = 0; it < 18; it += C::WARPS, turn ^= 1) {
+        const int pair = it >> 1, part = C::WARPS % 2 == 0 ? (it & 1) ^ turn : it & 1;
+        const int row = pair, cy = row % 3 - 1, cz = row / 3 - 1, i0 = 3 * row;
+        const unsigned rb = ysel(nb, cy) + zsel(nb, cz);
+        const long long own = (long long)(rb + nb.xs[1]);                 // the sender at this x
+        char* src[3];
+#pragma unroll
+        for (int x = 0; x < 3; ++x) {
+          const bool here = PAR == 0 || (WALL && arrives_from_wall_c(nb, x - 1));        // aa_read_loc
+          src[x] = slot_at(here ? i0 + x : Q - 1 - i0 - x, here ? n : (long long)(rb + nb.xs[2 - x]));
+        }
+        const float4* rec = reinterpret_cast<const float4*>(rin) + own;
+        // pairs [q0, q0 + K) of the row
+        auto species = [&](auto Q0_, auto K_, const float4& A) {
+          constexpr int q0 = decltype(Q0_)::value, K = decltype(K_)::value;
+          Store raw[K][3][2];
+          float2 d[K];
+#pragma unroll
+          for (int k = 0; k < K; ++k) {
+            const int q = q0 + k;
+            d[k] = __ldg(reinterpret_cast<const float2*>(rec + (2 + q / 2) * N) + q % 2);
+#pragma unroll
+            for (int x = 0; x < 3; ++x) {
+              raw[k][x][0] = *lat(src[x], 2 * q);
+              if (2 * q + 1 < M) raw[k][x][1] = *lat(src[x], 2 * q + 1);
+            }
+          }
+          const float4 w = p.weak ? __ldg(rec + (2 + (1 + M + 3) / 4) * N) : A;
+          const RowSpecies r(w.x, w.y, w.z, p.Tr + A.w, cy, cz);
+#pragma unroll
+          for (int k = 0; k < K; ++k) {
+            const int q = q0 + k;
+            float2 t[3];
+            row_species(p, r, 2 * q, 2 * q + 1 < M ? 2 * q + 1 : 2 * q, d[k], t);
+            t[2].x = __shfl_up_sync(0xffffffffu, t[2].x, 1);
+            t[2].y = __shfl_up_sync(0xffffffffu, t[2].y, 1);
+            t[0].x = __shfl_down_sync(0xffffffffu, t[0].x, 1);
+            t[0].y = __shfl_down_sync(0xffffffffu, t[0].y, 1);
+            if (needL) t[2] = stage[((i0 + 2) * NP + q) * 32];
+            if (needR) t[0] = stage[(i0 * NP + q) * 32];
+#pragma unroll
+            for (int x = 0; x < 3; ++x) {
+              float2 v;
+              v.x = codec_decode<Store, float>(p, raw[k][x][0], 2 * q) + t[x].x;
+              v.y = 2 * q + 1 < M ? codec_decode<Store, float>(p, raw[k][x][1], 2 * q + 1) + t[x].y : 0.0f;
+              stage[((i0 + x) * NP + q) * 32] = v;
+            }
+          }
+        };
+        constexpr int Q1 = NP >= 3 ? NP - 1 : NP;          // pairs of part 0
+        using Zero = std::integral_constant<int, 0>;
+        using First = std::integral_constant<int, Q1>;
+        using Last = std::integral_constant<int, NP - Q1>;
+        const float4 A = __ldg(rec);
+        if (part == 0) {
+          species(Zero{}, First{}, A);
+        } else {
+          Store raw[3][2];
+#pragma unroll
+          for (int x = 0; x < 3; ++x) { raw[x][0] = *lat(src[x], M); raw[x][1] = *lat(src[x], M + 1); }
+          const float4 B = __ldg(rec + N);
+          const float hq = __ldg(reinterpret_cast<const float*>(rec + (2 + M / 4) * N) + M % 4);
+          const RowSide sd(side, N, own, cy, cz);
+          if constexpr (Last::value > 0) species(First{}, Last{}, A);
+          float f[3], g[3];
+          row_fg(p, M, A, B, hq, sd.k, sd.x, cy, cz, f, g);
+          f[2] = __shfl_up_sync(0xffffffffu, f[2], 1);
+          g[2] = __shfl_up_sync(0xffffffffu, g[2], 1);
+          f[0] = __shfl_down_sync(0xffffffffu, f[0], 1);
+          g[0] = __shfl_down_sync(0xffffffffu, g[0], 1);
+          if (needL) { f[2] = fg[2 * (i0 + 2) * 32]; g[2] = fg[(2 * (i0 + 2) + 1) * 32]; }
+          if (needR) { f[0] = fg[2 * i0 * 32]; g[0] = fg[(2 * i0 + 1) * 32]; }
+#pragma unroll
+          for (int x = 0; x < 3; ++x) {
+            fg[2 * (i0 + x) * 32] = codec_decode<Store, float>(p, raw[x][0], M) + f[x];
+            fg[(2 * (i0 + x) + 1) * 32] = codec_decode<Store, float>(p, raw[x][1], M + 1) + g[x];
+          }
         }
       }
+    } else {
+      // FP64 and FP32: the velocities in turn.  (Asynchronous copies of the whole
+      // tile into the stage with the deferred terms formed by rows meanwhile
+      // measured slower: eight species 128^3 FP32 2.07 against 1.95 ms.)
+#pragma unroll 1
+      for (int i = role; i < Q; i += C::WARPS) {
+        const int cz = i / 9 - 1, cy = (i / 3) % 3 - 1, cx = i % 3 - 1;
+        const bool refl = WALL && arrives_from_wall_c(nb, cx);
+        const unsigned xs = cx == 0 ? nb.xs[1] : (cx > 0 ? nb.xs[0] : nb.xs[2]);
+        const long long snd = refl ? n : (long long)(xs + ysel(nb, cy) + zsel(nb, cz));   // n - c_i, or n itself at a wall
+        const bool own = PAR == 0 || refl;                                                // aa_read_loc
+        char* const q = slot_at(own ? i : Q - 1 - i, own ? n : snd);
+        Real v[M + 2];
 #pragma unroll
-      for (int q = 0; q < NP; ++q) {
-        V d;
-        d.x = codec_decode<Store, Real>(p, raw[2 * q], 2 * q);
-        d.y = 2 * q + 1 < M ? codec_decode<Store, Real>(p, raw[2 * q + 1], 2 * q + 1) : Real(0);
-        d = EQ ? vadd(d, v[q]) : d;
-        if (2 * q + 1 >= M) d.y = Real(0);
-        stage[(i * NP + q) * 32] = d;
+        for (int L = 0; L < M + 2; ++L) v[L] = *lat(q, L);
+        if (i != 13) {
+          // the deferred terms (incoming_corr_th)
+          const Real th = side_ld(side + SP_THR * N + snd);
+          Real kc = Real(0);
+          if (cx) { const Real k = side_ld(side + (SP_K + 0) * N + snd); kc += cx > 0 ? k : -k; }
+          if (cy) { const Real k = side_ld(side + (SP_K + 1) * N + snd); kc += cy > 0 ? k : -k; }
+          if (cz) { const Real k = side_ld(side + (SP_K + 2) * N + snd); kc += cz > 0 ? k : -k; }
+          const Real w0 = Real(1) - th, w1 = Real(0.5) * th;
+          const Real cg = (cx ? w1 : w0) * (cy ? w1 : w0) * (cz ? w1 : w0) * kc;
+          v[M + 1] += refl ? -cg : cg;
+          if (cx * cx + cy * cy + cz * cz == 1) {
+            const Real X = side_ld(side + (SP_X + (cx ? 0 : (cy ? 1 : 2))) * N + snd);
+            const Real cf = (cx + cy + cz > 0 ? Real(0.5) : Real(-0.5)) * X;
+            v[M] += refl ? -cf : cf;
+          }
+        }
+#pragma unroll
+        for (int a = 0; a < M; a += 2) {
+          V d;
+          d.x = v[a];
+          d.y = a + 1 < M ? v[a + 1] : Real(0);
+          stage[(i * NP + a / 2) * 32] = d;
+        }
+        fg[2 * i * 32] = v[M];
+        fg[(2 * i + 1) * 32] = v[M + 1];
       }
-      fg[(2 * i) * 32] = codec_decode<Store, Real>(p, raw[M], M) + fv;
-      fg[(2 * i + 1) * 32] = codec_decode<Store, Real>(p, raw[M + 1], M + 1) + gv;
     }
     __syncthreads();
 
@@ -654,15 +761,16 @@ collide_split_kernel(const __grid_constant__ DevParams<Real> p, Store* __restric
           mm[k] = s;
         });
       };
+      char* const first = reinterpret_cast<char*>(pops) + (long long)a0 * po.off[Q];
       auto put = [&](auto I_, V val) {
         constexpr int i = decltype(I_)::value;
         long long nn; int slot;
         aa_write_loc<WALL>(PAR, nbw, nw, i, nn, slot);
-        const long long o = off(slot, nn);
+        char* const q = first + (nn * (long long)sizeof(Store) + po.off[slot]);
         const V out = vfma(cv, stage[(i * NP + role) * 32], val);
         if (active) {
-          codec_store<Store, Real>(p, at(a0, o), 0, a0, out.x);
-          if (two) codec_store<Store, Real>(p, at(a0 + 1, o), 0, a0 + 1, out.y);
+          codec_store<Store, Real>(p, reinterpret_cast<Store*>(q), 0, a0, out.x);
+          if (two) codec_store<Store, Real>(p, lat(q, 1), 0, a0 + 1, out.y);
         }
       };
       from_moments<Real, V>(crd, plane, put, [&](V val) { put(std::integral_constant<int, 13>{}, val); });
@@ -711,7 +819,7 @@ collide_split_kernel(const __grid_constant__ DevParams<Real> p, Store* __restric
           constexpr int i = decltype(I_)::value;
           long long nn; int slot;
           aa_write_loc<WALL>(PAR, nbw, nw, i, nn, slot);
-          if (active) codec_store<Store, Real>(p, at(M, off(slot, nn)), 0, M, cv * fg[2 * i * 32] + val);
+          if (active) codec_store<Store, Real>(p, lat(slot_at(slot, nn), M), 0, M, cv * fg[2 * i * 32] + val);
         };
         from_moments<Real, Real>(crd, plane, put, [&](Real val) { put(std::integral_constant<int, 13>{}, val); });
       } else {
@@ -790,8 +898,8 @@ collide_split_kernel(const __grid_constant__ DevParams<Real> p, Store* __restric
           const Real out_o = go + om * (eg - go) - fl;
           if (active) {
             const Real sq = EQ ? wi * dotc<Real, i>(qt) : Real(0);
-            codec_store<Store, Real>(p, at(M + 1, off(slot_i, node_i)), 0, M + 1, EQ ? out_i - (eg + sq) : out_i);
-            codec_store<Store, Real>(p, at(M + 1, off(slot_o, node_o)), 0, M + 1, EQ ? out_o - (eg - sq) : out_o);
+            codec_store<Store, Real>(p, lat(slot_at(slot_i, node_i), M + 1), 0, M + 1, EQ ? out_i - (eg + sq) : out_i);
+            codec_store<Store, Real>(p, lat(slot_at(slot_o, node_o), M + 1), 0, M + 1, EQ ? out_o - (eg - sq) : out_o);
           }
         });
         long long nn; int slot;
@@ -799,7 +907,7 @@ collide_split_kernel(const __grid_constant__ DevParams<Real> p, Store* __restric
         const Real e13 = rhoE_dev - s_g;
         const Real gr = fg[(2 * 13 + 1) * 32];
         const Real out = gr + om * (e13 - gr);
-        if (active) codec_store<Store, Real>(p, at(M + 1, off(slot, nn)), 0, M + 1, EQ ? out - e13 : out);
+        if (active) codec_store<Store, Real>(p, lat(slot_at(slot, nn), M + 1), 0, M + 1, EQ ? out - e13 : out);
       }
     }
     __syncthreads();      // the next tile's moments take the place of this tile's
