@@ -884,7 +884,7 @@ lbm_status lbm_mix_step(lbm_mix_t h, int nsteps) {
     lbm_status st = h->cuda(h->ks->step(c, (int)(h->steps & 1)), "step kernels");
     if (st != LBM_OK) return st;
     h->steps += 1;
-    h->launches += h->ks->launches_per_step + (h->p64.frame ? 4 : 0);
+    h->launches += h->ks->launches_per_step + (h->p64.frame ? 3 : 0);
   }
   return LBM_OK;
 }

@@ -341,12 +341,10 @@ struct Launch {
     }
     // opposed-jets frame: the populations and side fields of the frame nodes
     const bool frame = P(c).frame != 0;
-    const unsigned fgrid = frame ? grid_for(frame_count(P(c)), BLOCK_LIGHT) : 0u;
-    if (frame) {
-      frame_pops_kernel<M, Real, Store><<<fgrid, BLOCK_LIGHT, 0, c.stream>>>(P(c), (Store*)c.pops, c.jet, c.base,
-                                                                             parity);
-      frame_side_kernel<Real><<<fgrid, BLOCK_LIGHT, 0, c.stream>>>(P(c), side, 0);
-    }
+    const unsigned fgrid = frame ? grid_for(frame_count(P(c)), BLOCK_FRAME) : 0u;
+    if (frame)
+      frame_pops_kernel<M, Real, Store><<<dim3(fgrid, Q + 1), BLOCK_FRAME, 0, c.stream>>>(P(c), (Store*)c.pops, side, c.jet,
+                                                                                       c.base, parity);
     if (c.ev) cudaEventRecord(c.ev[1], c.stream);
     // Row-blocked stencils (ROWV nodes per thread) where rows split evenly; a
     // thread per node and field on grids of few nodes.
@@ -356,12 +354,12 @@ struct Launch {
     if (few) grad_GK_field_kernel<Real><<<fg, BLOCK_FIELD, 0, c.stream>>>(P(c), side);
     else if (rows) grad_GK_row_kernel<Real><<<grid_for(c.N / ROWV, BLOCK_LIGHT), BLOCK_LIGHT, 0, c.stream>>>(P(c), side);
     else grad_GK_kernel<Real><<<grid_for(c.N, BLOCK_LIGHT), BLOCK_LIGHT, 0, c.stream>>>(P(c), side);
-    if (frame) frame_side_kernel<Real><<<fgrid, BLOCK_LIGHT, 0, c.stream>>>(P(c), side, 1);
+    if (frame) frame_side_kernel<Real><<<fgrid, BLOCK_FRAME, 0, c.stream>>>(P(c), side, 1);
     if (c.ev) cudaEventRecord(c.ev[2], c.stream);
     if (few) grad_X_field_kernel<Real><<<fx, BLOCK_FIELD, 0, c.stream>>>(P(c), side);
     else if (rows) grad_X_row_kernel<Real><<<grid_for(c.N / ROWV, BLOCK_LIGHT), BLOCK_LIGHT, 0, c.stream>>>(P(c), side);
     else grad_X_kernel<Real><<<grid_for(c.N, BLOCK_LIGHT), BLOCK_LIGHT, 0, c.stream>>>(P(c), side);
-    if (frame) frame_side_kernel<Real><<<fgrid, BLOCK_LIGHT, 0, c.stream>>>(P(c), side, 2);
+    if (frame) frame_side_kernel<Real><<<fgrid, BLOCK_FRAME, 0, c.stream>>>(P(c), side, 2);
     if (c.ev) cudaEventRecord(c.ev[3], c.stream);
     return cudaGetLastError();
   }
