@@ -360,11 +360,14 @@ __device__ __forceinline__ void split_closure(const DevParams<Real>& p, Real* sm
 //   * With two or three species on grids of few tiles per SM, where the time
 //     is one node's latency: three species FP64 1024 nodes 59 against 121 us
 //     (16,384 nodes 156 against 132), FP32 1024 nodes 12.1 against 14.8 us
-//     (16,384 nodes 14.3 against 15.7, 32,768 nodes 22.4 against 16.6), BF16 1024
-//     nodes 14.2 against 22.4 us; two species FP64 1024 nodes 52 against 97 us,
-//     BF16 4096 nodes 15.7 against 18.3 us, but FP32 1024 nodes 12.0 against 10.3.
+//     (16,384 nodes 14.3 against 15.7, 32,768 nodes 22.4 against 16.6); two
+//     species FP64 1024 nodes 52 against 97 us, but FP32 12.0 against 10.3.
+//     Not with 16-bit storage (three species BF16 1024 nodes 14.2 against 22.4
+//     us): there the network closure's step, which stays with a thread per
+//     node, is held to the exact step to less than a change of rounding moves
+//     a 16-bit value.
 template <int M, class Real, class Store>
-constexpr bool kSplit = M >= 3 || (M == 2 && (sizeof(Real) == 8 || sizeof(Store) == 2));
+constexpr bool kSplit = M >= 4 || (sizeof(Store) >= 4 && (M == 3 || (M == 2 && sizeof(Real) == 8)));
 // The largest number of tiles per SM taken (0: any).
 template <int M, class Real, class Store>
 constexpr int kSplitTilesPerSm = M >= 4 ? 0 : (sizeof(Real) == 8 ? 1 : 3);
