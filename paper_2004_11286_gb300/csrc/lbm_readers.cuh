@@ -75,12 +75,13 @@ template <int M, class Real, class Store>
 __global__ void __launch_bounds__(BLOCK)
 moments_kernel(const DevParams<Real> p, const Store* __restrict__ pops, const Real* __restrict__ side,
                int parity, double* __restrict__ out) {
-  const long long n = gtid();
-  if (n >= p.N) return;
-  const long long N = p.N;
+  const bool active = gtid() < p.N;
+  if (!kEqCodec<Store, Real> && !active) return;
+  const long long N = p.N, n = active ? gtid() : N - 1;
   const Nbr nb = make_nbr(p, n);
   Real rdev[M], ja[M][3], rho_dev, j[3], rhoE_dev;
-  load_state_moments<M, Real, Store>(p, pops, side, parity, nb, n, rdev, ja, rho_dev, j, rhoE_dev);
+  load_state_moments<M, Real, Store>(p, pops, side, parity, nb, n, active, rdev, ja, rho_dev, j, rhoE_dev);
+  if (!active) return;
   Real jsum[3] = {Real(0), Real(0), Real(0)};
 #pragma unroll
   for (int a = 0; a < M; ++a) { jsum[0] += ja[a][0]; jsum[1] += ja[a][1]; jsum[2] += ja[a][2]; }
@@ -129,18 +130,29 @@ template <int M, class Real, class Store>
 __global__ void __launch_bounds__(BLOCK_LIGHT)
 get_pops_kernel(const DevParams<Real> p, const Store* __restrict__ pops, const Real* __restrict__ side,
                 const double* __restrict__ base, int parity, double* __restrict__ out) {
-  const long long n = gtid();
-  if (n >= p.N) return;
-  const long long N = p.N;
+  const bool active = gtid() < p.N;
+  if (!kEqCodec<Store, Real> && !active) return;
+  const long long N = p.N, n = active ? gtid() : N - 1;
   const Nbr nb = make_nbr(p, n);
+  if constexpr (kEqCodec<Store, Real>) {
+    row_populations<M, Store>(p, side, parity, nb, n, active,
+                              [&](int i, int, int, int, int slot, long long node, const float (&sh)[M + 2]) {
+      if (!active) return;
+#pragma unroll
+      for (int L = 0; L < M + 2; ++L)
+        out[(L * Q + i) * N + n] = base[L * Q + i] + ((double)codec_load<Store, Real>(p, pops, (L * Q + slot) * N + node, L) +
+                                                      (double)sh[L]);
+    });
+    return;
+  }
   static_for<0, Q>([&](auto I_) {
     constexpr int i = decltype(I_)::value;
     long long node; int slot;
     aa_read_loc<true>(parity, nb, n, i, node, slot);
-    Real cf, cg, sh[M + 2];
-    incoming_terms<M, Real, Store, i>(p, side, nb, n, parity, cf, cg, sh);
+    Real cf = Real(0), cg = Real(0);
+    if constexpr (i != 13) deferred_terms<Real, i, true>(side, N, nb, n, cf, cg);
     for (int L = 0; L < M + 2; ++L) {
-      double v = (double)codec_load<Store, Real>(p, pops, (L * Q + slot) * N + node, L) + (double)sh[L];
+      double v = (double)codec_load<Store, Real>(p, pops, (L * Q + slot) * N + node, L);
       if (L == M) v += (double)cf;
       if (L == M + 1) v += (double)cg;
       out[(L * Q + i) * N + n] = base[L * Q + i] + v;
@@ -192,24 +204,27 @@ template <int M, class Real, class Store>
 __global__ void __launch_bounds__(BLOCK_LIGHT)
 set_pops_kernel(const DevParams<Real> p, Store* __restrict__ pops, const Real* __restrict__ side,
                 const double* __restrict__ base, int parity, const double* __restrict__ in) {
-  const long long n = gtid();
-  if (n >= p.N) return;
-  const long long N = p.N;
+  const bool active = gtid() < p.N;
+  if (!kEqCodec<Store, Real> && !active) return;
+  const long long N = p.N, n = active ? gtid() : N - 1;
   const Nbr nb = make_nbr(p, n);
+  if constexpr (kEqCodec<Store, Real>) {
+    row_populations<M, Store>(p, side, parity, nb, n, active,
+                              [&](int i, int, int, int, int slot, long long node, const float (&sh)[M + 2]) {
+      if (!active) return;
+#pragma unroll
+      for (int L = 0; L < M + 2; ++L)
+        codec_store<Store, Real>(p, pops, (L * Q + slot) * N + node, L,
+                                 (Real)((in[(L * Q + i) * N + n] - base[L * Q + i]) - (double)sh[L]));
+    });
+    return;
+  }
   static_for<0, Q>([&](auto I_) {
     constexpr int i = decltype(I_)::value;
     long long node; int slot;
     aa_read_loc<true>(parity, nb, n, i, node, slot);
-    Real sh[M + 2];
-#pragma unroll
-    for (int L = 0; L < M + 2; ++L) sh[L] = Real(0);
-    if constexpr (kEqCodec<Store, Real>) {
-      Real cf, cg;
-      eq_incoming<M, i, true>(p, side, nb, n, parity, cf, cg, sh);
-    }
     for (int L = 0; L < M + 2; ++L)
-      codec_store<Store, Real>(p, pops, (L * Q + slot) * N + node, L,
-                               (Real)((in[(L * Q + i) * N + n] - base[L * Q + i]) - (double)sh[L]));
+      codec_store<Store, Real>(p, pops, (L * Q + slot) * N + node, L, (Real)(in[(L * Q + i) * N + n] - base[L * Q + i]));
   });
 }
 
@@ -222,11 +237,13 @@ __global__ void __launch_bounds__(BLOCK)
 closure_samples_kernel(const DevParams<Real> p, const Store* __restrict__ pops, const Real* __restrict__ side,
                        int parity, float* __restrict__ feat, float* __restrict__ tgt) {
   using Dm = MlpDims<M>;
-  const long long n = gtid();
-  if (n >= p.N) return;
+  const bool active = gtid() < p.N;
+  if (!kEqCodec<Store, Real> && !active) return;
+  const long long n = active ? gtid() : p.N - 1;
   const Nbr nb = make_nbr(p, n);
   Real rdev[M], ja[M][3], rho_dev, j[3], rhoE_dev;
-  load_state_moments<M, Real, Store>(p, pops, side, parity, nb, n, rdev, ja, rho_dev, j, rhoE_dev);
+  load_state_moments<M, Real, Store>(p, pops, side, parity, nb, n, active, rdev, ja, rho_dev, j, rhoE_dev);
+  if (!active) return;
   Real jsum[3] = {Real(0), Real(0), Real(0)};
 #pragma unroll
   for (int a = 0; a < M; ++a) { jsum[0] += ja[a][0]; jsum[1] += ja[a][1]; jsum[2] += ja[a][2]; }
