@@ -1063,6 +1063,7 @@ __global__ void __launch_bounds__(collide_block<M, Real, CL, Store>(), collide_m
 collide_kernel(const __grid_constant__ DevParams<Real> p, Store* __restrict__ pops, Real* __restrict__ side,
                unsigned* __restrict__ err, const unsigned char* __restrict__ mlp_img,
                unsigned long long* __restrict__ mlp_stats, const __grid_constant__ PlaneOffsets po) {
+  wait_previous();
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   collide_node<M, Real, Store, PAR, CL, LD, WALL == 1, LBM_PLANE_OFFSETS != 0, WALL == 2>(
       p, pops, side, err, mlp_img, mlp_stats, gtid(), smem_raw, po.off);

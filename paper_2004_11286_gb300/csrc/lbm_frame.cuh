@@ -91,7 +91,8 @@ __device__ __forceinline__ void frame_side_node(const DevParams<Real>& p, Real* 
 
 template <class Real>
 __global__ void __launch_bounds__(BLOCK_FRAME)
-frame_side_kernel(const DevParams<Real> p, Real* __restrict__ side, int stage) {
+frame_side_kernel(const __grid_constant__ DevParams<Real> p, Real* __restrict__ side, int stage) {
+  wait_previous();
   const long long t = gtid();
   const long long per = frame_count(p) / p.nz;
   if (t >= per * p.nz) return;
@@ -112,8 +113,9 @@ frame_side_kernel(const DevParams<Real> p, Real* __restrict__ side, int stage) {
 // 200 x 400 jets, FP32): collide and frame 59 against 116 us.
 template <int M, class Real, class Store>
 __global__ void __launch_bounds__(BLOCK_FRAME)
-frame_pops_kernel(const DevParams<Real> p, Store* __restrict__ pops, Real* __restrict__ side,
+frame_pops_kernel(const __grid_constant__ DevParams<Real> p, Store* __restrict__ pops, Real* __restrict__ side,
                   const double* __restrict__ jet, const double* __restrict__ base, int parity) {
+  wait_previous();
   const long long t = gtid();
   const long long per = frame_count(p) / p.nz;
   if (t >= per * p.nz) return;

@@ -430,6 +430,7 @@ collide_split_kernel(const __grid_constant__ DevParams<Real> p, Store* __restric
     }
   }
 
+  wait_previous();
   for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const long long n_raw = (long long)tile * 32 + lane;
     bool active = n_raw < N;

@@ -561,6 +561,7 @@ constexpr int BLOCK_FIELD = 32;
 template <class Real>
 __global__ void __launch_bounds__(BLOCK_FIELD)
 grad_GK_field_kernel(const __grid_constant__ DevParams<Real> p, Real* __restrict__ side) {
+  wait_previous();
   if (blockIdx.y == 0) grad_GK_field<Real>(p, side, gtid(), 0);
   else if (blockIdx.y == 1) grad_GK_field<Real>(p, side, gtid(), 1);
   else if (blockIdx.y == 2) grad_GK_field<Real>(p, side, gtid(), 2);
@@ -569,6 +570,7 @@ grad_GK_field_kernel(const __grid_constant__ DevParams<Real> p, Real* __restrict
 template <class Real>
 __global__ void __launch_bounds__(BLOCK_FIELD)
 grad_X_field_kernel(const __grid_constant__ DevParams<Real> p, Real* __restrict__ side) {
+  wait_previous();
   if (blockIdx.y == 0) grad_X_field<Real>(p, side, gtid(), 0);
   else if (blockIdx.y == 1) grad_X_field<Real>(p, side, gtid(), 1);
   else grad_X_field<Real>(p, side, gtid(), 2);
@@ -587,6 +589,7 @@ __launch_bounds__(BLOCK_LIGHT, sizeof(Real) == 4 ? LBM_GK_MINB : 1)
 __launch_bounds__(BLOCK_LIGHT)
 #endif
 grad_GK_row_kernel(const __grid_constant__ DevParams<Real> p, Real* __restrict__ side) {
+  wait_previous();
   const long long t = gtid();
   const bool in = ROWV * t < p.N;
   grad_GK_row<Real>(p, side, (unsigned)(in ? ROWV * t : p.N - ROWV), in);
@@ -594,6 +597,7 @@ grad_GK_row_kernel(const __grid_constant__ DevParams<Real> p, Real* __restrict__
 template <class Real>
 __global__ void __launch_bounds__(BLOCK_LIGHT)
 grad_X_row_kernel(const __grid_constant__ DevParams<Real> p, Real* __restrict__ side) {
+  wait_previous();
   const long long t = gtid();
   const bool in = ROWV * t < p.N;
   grad_X_row<Real>(p, side, (unsigned)(in ? ROWV * t : p.N - ROWV), in);
@@ -602,11 +606,13 @@ grad_X_row_kernel(const __grid_constant__ DevParams<Real> p, Real* __restrict__ 
 template <class Real>
 __global__ void __launch_bounds__(BLOCK_LIGHT)
 grad_GK_kernel(const __grid_constant__ DevParams<Real> p, Real* __restrict__ side) {
+  wait_previous();
   grad_GK_node<Real>(p, side, gtid(), p.tvar != 0);
 }
 template <class Real>
 __global__ void __launch_bounds__(BLOCK_LIGHT)
 grad_X_kernel(const __grid_constant__ DevParams<Real> p, Real* __restrict__ side) {
+  wait_previous();
   grad_X_node<Real>(p, side, gtid());
 }
 
