@@ -335,14 +335,18 @@ struct Launch {
         return;
       }
     }
+    constexpr bool bulk = CL == 0 && LBM_COLLIDE_BULK && M >= LBM_COLLIDE_BULK_MIN_M && std::is_same<Real, Store>::value;
+    const bool segments = bulk && P(c).nx % collide_block<M, Real, 0, Store>() == 0;
     if constexpr (CL == 0 && kSplit<M, Real, Store> && kSplitTilesPerSm<M, Real, Store> == 0) {
       // only temperature-dependent heats get here (FP64, FP32, periodic)
-      if constexpr (!EQ) collide_launch<0, 0>(c, parity, side);
+      if constexpr (!EQ) {
+        if (segments) collide_launch<0, bulk>(c, parity, side);
+        else collide_launch<0, 0>(c, parity, side);
+      }
     } else if constexpr (CL == 0) {
-      constexpr bool bulk = LBM_COLLIDE_BULK && M >= LBM_COLLIDE_BULK_MIN_M && std::is_same<Real, Store>::value;
       if (P(c).wall_x) collide_launch<0, 0, 1>(c, parity, side);
       else if (P(c).frame) collide_launch<0, 0, EQ ? 0 : 2>(c, parity, side);
-      else if (bulk && P(c).nx % collide_block<M, Real, 0, Store>() == 0) collide_launch<0, bulk>(c, parity, side);
+      else if (segments) collide_launch<0, bulk>(c, parity, side);
       else collide_launch<0, 0>(c, parity, side);
     } else {
       collide_launch<CL, 0>(c, parity, side);

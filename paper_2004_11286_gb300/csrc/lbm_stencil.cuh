@@ -57,9 +57,8 @@ __device__ __forceinline__ Real side_ld(const Real* p) {
 }
 
 // The deferred terms of the population that `sender` sent in direction I,
-// for a sender whose theta is th (with FACE = false, only the
-// energy lattice's).
-template <class Real, int I, bool FACE = true>
+// for a sender whose theta is th.
+template <class Real, int I>
 __device__ __forceinline__ void incoming_corr_th(const Real* __restrict__ side, long long N, long long sender,
                                                  Real th, Real& cf, Real& cg) {
   constexpr int cx = cx_of(I), cy = cy_of(I), cz = cz_of(I);
@@ -71,7 +70,7 @@ __device__ __forceinline__ void incoming_corr_th(const Real* __restrict__ side, 
   const Real w = (cx ? w1 : w0) * (cy ? w1 : w0) * (cz ? w1 : w0);   // Eq. (weights)
   cg = w * kc;
   cf = Real(0);
-  if constexpr (FACE && c2_of(I) == 1) {
+  if constexpr (c2_of(I) == 1) {
     constexpr int a = cx ? 0 : (cy ? 1 : 2);
     constexpr int sg = cx + cy + cz;
     cf = (sg > 0 ? Real(0.5) : Real(-0.5)) * side_ld(side + (SP_X + a) * N + sender);
