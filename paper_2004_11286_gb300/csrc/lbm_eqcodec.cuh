@@ -71,21 +71,21 @@ template <int M>
 __device__ __forceinline__ EqRec<M> load_rec(const float* __restrict__ buf, long long N, long long node, int weak) {
   const float4* q = reinterpret_cast<const float4*>(buf) + node;
   EqRec<M> r;
-  const float4 a = __ldg(q), b = __ldg(q + N);
+  const float4 a = q[0], b = q[N];
   r.u[0] = a.x; r.u[1] = a.y; r.u[2] = a.z; r.dT = a.w;
   r.dth = b.x; r.drho = b.y; r.dE0 = b.z; r.Gq = b.w;
   constexpr int NT = (1 + M + 3) / 4;
   float t[4 * NT];
 #pragma unroll
   for (int k = 0; k < NT; ++k) {
-    const float4 c = __ldg(q + (2 + k) * N);
+    const float4 c = q[(2 + k) * N];
     t[4 * k] = c.x; t[4 * k + 1] = c.y; t[4 * k + 2] = c.z; t[4 * k + 3] = c.w;
   }
 #pragma unroll
   for (int s = 0; s < M; ++s) r.ra[s] = t[s];
   r.hq = t[M];
   if (weak) {
-    const float4 d = __ldg(q + (2 + NT) * N);
+    const float4 d = q[(2 + NT) * N];
     r.usp[0] = d.x; r.usp[1] = d.y; r.usp[2] = d.z;
   } else {
     r.usp[0] = r.u[0]; r.usp[1] = r.u[1]; r.usp[2] = r.u[2];
@@ -210,8 +210,8 @@ struct RecLoad {
   __device__ __forceinline__ RecLoad(const float* __restrict__ buf, long long N, long long node, int weak) {
     const float4* r = reinterpret_cast<const float4*>(buf) + node;
 #pragma unroll
-    for (int k = 0; k < 2 + NT; ++k) q[k] = __ldg(r + k * N);
-    q[2 + NT] = weak ? __ldg(r + (2 + NT) * N) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    for (int k = 0; k < 2 + NT; ++k) q[k] = r[k * N];
+    q[2 + NT] = weak ? r[(2 + NT) * N] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   }
 };
 
@@ -366,10 +366,10 @@ struct RowTerms {
 struct RowSide {
   float k[3], x;
   __device__ __forceinline__ RowSide(const float* __restrict__ side, long long N, long long snd, int cy, int cz) {
-    k[0] = __ldg(side + (SP_K + 0) * N + snd);
-    k[1] = cy ? __ldg(side + (SP_K + 1) * N + snd) : 0.0f;
-    k[2] = cz ? __ldg(side + (SP_K + 2) * N + snd) : 0.0f;
-    x = cy * cz == 0 ? __ldg(side + (SP_X + (cy ? 1 : (cz ? 2 : 0))) * N + snd) : 0.0f;
+    k[0] = side[(SP_K + 0) * N + snd];
+    k[1] = cy ? side[(SP_K + 1) * N + snd] : 0.0f;
+    k[2] = cz ? side[(SP_K + 2) * N + snd] : 0.0f;
+    x = cy * cz == 0 ? side[(SP_X + (cy ? 1 : (cz ? 2 : 0))) * N + snd] : 0.0f;
   }
 };
 // What a sender's RowTerms are formed from, as loaded.

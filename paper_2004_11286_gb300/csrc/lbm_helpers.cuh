@@ -19,12 +19,18 @@ __device__ __forceinline__ long long gtid() {
 }
 
 // Step kernels are launched with programmatic stream serialization
-// (launch_next): their blocks may start while the last blocks of the kernel
-// before them finish.  Nothing that kernel writes is read, and nothing it reads
-// is written, before this wait, which returns once it has completed (at
-// once where there is nothing to wait for).  No kernel triggers its successor
-// early: successors whose blocks were resident from the start took SMs from
-// the blocks still to come (1024-node FP64 step 79 against 62 us).
+// (launch_next).  None triggers its successor, so a kernel's blocks may start
+// once every block of the kernel before it has exited, while that kernel's
+// writes may still be on their way: what overlaps is the launch and the set-up
+// ahead of this wait.  Nothing the kernel before writes is read, and nothing it
+// reads is written, before the wait, which returns once that kernel has
+// completed and its writes are visible (at once where there is nothing to wait
+// for).  The planes a step kernel reads are therefore not constant from its
+// first block on, and it reads them by ordinary loads, which the wait orders:
+// the non-coherent path (__ldg) is for memory that no one writes while the
+// kernel lives.  An early trigger lost: successors whose blocks were resident
+// from the start took SMs from the blocks still to come (1024-node FP64 step
+// 79 against 62 us).
 __device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // ---------------------------------------------------------------------------

@@ -236,9 +236,10 @@ diag_final_kernel(const double* __restrict__ partials, int nblocks, int nv, doub
 template <class Real>
 constexpr long long kFieldStencilNodes = sizeof(Real) == 8 ? 131072 : 32768;
 
-// A kernel of the step, behind another one on the stream: it may start while
-// that one drains (every kernel launched so calls wait_previous before it
-// touches memory), which hides its launch and its set-up.  Measured (GB300, us a
+// A kernel of the step, behind another one on the stream: its blocks may start
+// when the last block of that one has exited, before its completion has been
+// signalled (every kernel launched so calls wait_previous before it touches
+// memory), which hides the launch and the set-up.  Measured (GB300, us a
 // step): 96-node walled FP32 tube 9.4 against 15.9, 1024-node FP64 62 against
 // 70, 200 x 400 jets 65 against 77, 45x75x101 ternary FP32 141 against 149,
 // 128^3 two-species FP32 455 against 463.

@@ -506,14 +506,14 @@ collide_split_kernel(const __grid_constant__ DevParams<Real> p, Store* __restric
 #pragma unroll
           for (int k = 0; k < K; ++k) {
             const int q = q0 + k;
-            d[k] = __ldg(reinterpret_cast<const float2*>(rec + (2 + q / 2) * N) + q % 2);
+            d[k] = reinterpret_cast<const float2*>(rec + (2 + q / 2) * N)[q % 2];
 #pragma unroll
             for (int x = 0; x < 3; ++x) {
               raw[k][x][0] = *lat(src[x], 2 * q);
               if (2 * q + 1 < M) raw[k][x][1] = *lat(src[x], 2 * q + 1);
             }
           }
-          const float4 w = p.weak ? __ldg(rec + (2 + (1 + M + 3) / 4) * N) : A;
+          const float4 w = p.weak ? rec[(2 + (1 + M + 3) / 4) * N] : A;
           const RowSpecies r(w.x, w.y, w.z, p.Tr + A.w, cy, cz);
 #pragma unroll
           for (int k = 0; k < K; ++k) {
@@ -539,15 +539,15 @@ collide_split_kernel(const __grid_constant__ DevParams<Real> p, Store* __restric
         using Zero = std::integral_constant<int, 0>;
         using First = std::integral_constant<int, Q1>;
         using Last = std::integral_constant<int, NP - Q1>;
-        const float4 A = __ldg(rec);
+        const float4 A = *rec;
         if (part == 0) {
           species(Zero{}, First{}, A);
         } else {
           Store raw[3][2];
 #pragma unroll
           for (int x = 0; x < 3; ++x) { raw[x][0] = *lat(src[x], M); raw[x][1] = *lat(src[x], M + 1); }
-          const float4 B = __ldg(rec + N);
-          const float hq = __ldg(reinterpret_cast<const float*>(rec + (2 + M / 4) * N) + M % 4);
+          const float4 B = rec[N];
+          const float hq = reinterpret_cast<const float*>(rec + (2 + M / 4) * N)[M % 4];
           const RowSide sd(side, N, own, cy, cz);
           if constexpr (Last::value > 0) species(First{}, Last{}, A);
           float f[3], g[3];
@@ -582,16 +582,16 @@ collide_split_kernel(const __grid_constant__ DevParams<Real> p, Store* __restric
         for (int L = 0; L < M + 2; ++L) v[L] = *lat(q, L);
         if (i != 13) {
           // the deferred terms (incoming_corr_th)
-          const Real th = side_ld(side + SP_THR * N + snd);
+          const Real th = side[SP_THR * N + snd];
           Real kc = Real(0);
-          if (cx) { const Real k = side_ld(side + (SP_K + 0) * N + snd); kc += cx > 0 ? k : -k; }
-          if (cy) { const Real k = side_ld(side + (SP_K + 1) * N + snd); kc += cy > 0 ? k : -k; }
-          if (cz) { const Real k = side_ld(side + (SP_K + 2) * N + snd); kc += cz > 0 ? k : -k; }
+          if (cx) { const Real k = side[(SP_K + 0) * N + snd]; kc += cx > 0 ? k : -k; }
+          if (cy) { const Real k = side[(SP_K + 1) * N + snd]; kc += cy > 0 ? k : -k; }
+          if (cz) { const Real k = side[(SP_K + 2) * N + snd]; kc += cz > 0 ? k : -k; }
           const Real w0 = Real(1) - th, w1 = Real(0.5) * th;
           const Real cg = (cx ? w1 : w0) * (cy ? w1 : w0) * (cz ? w1 : w0) * kc;
           v[M + 1] += refl ? -cg : cg;
           if (cx * cx + cy * cy + cz * cz == 1) {
-            const Real X = side_ld(side + (SP_X + (cx ? 0 : (cy ? 1 : 2))) * N + snd);
+            const Real X = side[(SP_X + (cx ? 0 : (cy ? 1 : 2))) * N + snd];
             const Real cf = (cx + cy + cz > 0 ? Real(0.5) : Real(-0.5)) * X;
             v[M] += refl ? -cf : cf;
           }

@@ -42,20 +42,6 @@ __device__ __forceinline__ void store4(Real* __restrict__ f, const Real* v) {
   }
 }
 
-// Read-only gathers of the deferred terms through the non-coherent data path
-// (LBM_SIDE_LDG = 1; the collide never writes the planes it gathers from).
-#ifndef LBM_SIDE_LDG
-#define LBM_SIDE_LDG 1
-#endif
-template <class Real>
-__device__ __forceinline__ Real side_ld(const Real* p) {
-#if LBM_SIDE_LDG
-  return __ldg(p);
-#else
-  return *p;
-#endif
-}
-
 // The deferred terms of the population that `sender` sent in direction I,
 // for a sender whose theta is th.
 template <class Real, int I>
@@ -63,9 +49,9 @@ __device__ __forceinline__ void incoming_corr_th(const Real* __restrict__ side, 
                                                  Real th, Real& cf, Real& cg) {
   constexpr int cx = cx_of(I), cy = cy_of(I), cz = cz_of(I);
   Real kc = Real(0);
-  if constexpr (cx != 0) kc += (cx > 0 ? side_ld(side + (SP_K + 0) * N + sender) : -side_ld(side + (SP_K + 0) * N + sender));
-  if constexpr (cy != 0) kc += (cy > 0 ? side_ld(side + (SP_K + 1) * N + sender) : -side_ld(side + (SP_K + 1) * N + sender));
-  if constexpr (cz != 0) kc += (cz > 0 ? side_ld(side + (SP_K + 2) * N + sender) : -side_ld(side + (SP_K + 2) * N + sender));
+  if constexpr (cx != 0) kc += (cx > 0 ? side[(SP_K + 0) * N + sender] : -side[(SP_K + 0) * N + sender]);
+  if constexpr (cy != 0) kc += (cy > 0 ? side[(SP_K + 1) * N + sender] : -side[(SP_K + 1) * N + sender]);
+  if constexpr (cz != 0) kc += (cz > 0 ? side[(SP_K + 2) * N + sender] : -side[(SP_K + 2) * N + sender]);
   const Real w0 = Real(1) - th, w1 = Real(0.5) * th;
   const Real w = (cx ? w1 : w0) * (cy ? w1 : w0) * (cz ? w1 : w0);   // Eq. (weights)
   cg = w * kc;
@@ -73,13 +59,13 @@ __device__ __forceinline__ void incoming_corr_th(const Real* __restrict__ side, 
   if constexpr (c2_of(I) == 1) {
     constexpr int a = cx ? 0 : (cy ? 1 : 2);
     constexpr int sg = cx + cy + cz;
-    cf = (sg > 0 ? Real(0.5) : Real(-0.5)) * side_ld(side + (SP_X + a) * N + sender);
+    cf = (sg > 0 ? Real(0.5) : Real(-0.5)) * side[(SP_X + a) * N + sender];
   }
 }
 template <class Real, int I>
 __device__ __forceinline__ void incoming_corr(const Real* __restrict__ side, long long N, long long sender,
                                               Real& cf, Real& cg) {
-  incoming_corr_th<Real, I>(side, N, sender, side_ld(side + SP_THR * N + sender), cf, cg);
+  incoming_corr_th<Real, I>(side, N, sender, side[SP_THR * N + sender], cf, cg);
 }
 
 // Reduced-precision storage: the record of the node that sent the population
