@@ -189,7 +189,9 @@ __device__ __forceinline__ void collide_node(const DevParams<Real>& p, Store* __
   constexpr bool EQ = kEqCodec<Store, Real>;
   static_assert(!LD || std::is_same<Store, Real>::value, "bulk loads stage the stored type");
   static_assert(!(LD && WALL), "walls use the register-load path");
-  // Stage, thread-private columns: species [M*27][BS] (SpT), then f, g [2*27][BS] (Real).
+  // Stage, a column per thread: species [M*27][BS] (SpT), then f, g [2*27][BS]
+  // (Real).  Threads use their own columns, except the bulk row loads and, with
+  // 16-bit storage, the values formed ahead for other lanes of the warp.
   SpT* const sps = reinterpret_cast<SpT*>(smem_raw);
   Real* const sfg = reinterpret_cast<Real*>(smem_raw + (size_t)M * Q * BS * sizeof(SpT));
   Real* const sm = reinterpret_cast<Real*>(smem_raw);   // the whole stage when SpT == Real
@@ -363,6 +365,7 @@ __device__ __forceinline__ void collide_node(const DevParams<Real>& p, Store* __
     const int lane = tid & 31;
     const bool needL = active && (lane == 0 || nb.xs[1] == 0);
     const bool needR = active && (lane == 31 || (int)nb.xs[1] == p.nx - 1);
+    __syncwarp();      // a block that walks tiles: the columns written below were read for the tile before
     for (unsigned long long need = (unsigned long long)__ballot_sync(0xffffffffu, needL) |
                                    ((unsigned long long)__ballot_sync(0xffffffffu, needR) << 32);
          need != 0;) {
