@@ -19,6 +19,7 @@
 #include "lbm_batch.cuh"
 #include "lbm_readers.cuh"
 #include "lbm_frame.cuh"
+#include "lbm_per_device.h"
 
 namespace lbm {
 
@@ -261,6 +262,17 @@ inline void launch_next(void (*kernel)(P...), dim3 grid, unsigned block, size_t 
   cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
+inline int current_device() {
+  int dev = 0;
+  cudaGetDevice(&dev);
+  return dev;
+}
+// Lets a kernel take `bytes` of dynamic shared memory on the current device.
+template <class K>
+inline bool allow_smem(K* kernel, size_t bytes) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess;
+}
+
 inline unsigned grid_for(long long N, int block) { return (unsigned)((N + block - 1) / block); }
 
 template <int M, class Real, class Store>
@@ -281,39 +293,39 @@ struct Launch {
   static void collide_launch(const LaunchCtx& c, int parity, Real* side) {
     constexpr int BS = collide_block<M, Real, CL, Store>();
     constexpr size_t smem = collide_smem<M, Real, CL, LD, Store>();
-    static bool attr = false;
-    if (!attr) {
-      cudaFuncSetAttribute(collide_kernel<M, Real, Store, 0, CL, LD, WALL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)smem);
-      cudaFuncSetAttribute(collide_kernel<M, Real, Store, 1, CL, LD, WALL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)smem);
-      attr = true;
-    }
+    static PerDevice ready;
+    ready.get(current_device(), [] {
+      return (int)(allow_smem(collide_kernel<M, Real, Store, 0, CL, LD, WALL>, smem) &&
+                   allow_smem(collide_kernel<M, Real, Store, 1, CL, LD, WALL>, smem));
+    });
     PlaneOffsets po;
     for (int k = 0; k < (M + 2) * Q; ++k) po.off[k] = (long long)k * c.N * (long long)sizeof(Store);
     launch_next(parity == 0 ? collide_kernel<M, Real, Store, 0, CL, LD, WALL> : collide_kernel<M, Real, Store, 1, CL, LD, WALL>,
                 dim3(grid_for(c.N, BS)), BS, smem, c.stream, P(c), (Store*)c.pops, side, c.err, c.mlp_img, c.mlp_stats, po);
   }
   static int sm_count() {
-    static const int sms = [] {
-      int dev = 0, v = 1;
-      cudaGetDevice(&dev);
-      cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
-      return v;
-    }();
-    return sms;
+    static PerDevice sms;
+    const int dev = current_device();
+    const int v = sms.get(dev, [&] {
+      int n = 0;
+      cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+      return n;
+    });
+    return v > 0 ? v : 1;
   }
   template <int BND>
   static void split_launch(const LaunchCtx& c, int parity, Real* side) {
     using C = Split<M>;
     constexpr size_t smem = C::REALS * sizeof(Real);
-    static const int resident = [&] {            // blocks the device holds at once
+    static PerDevice blocks;
+    const int found = blocks.get(current_device(), [] {      // blocks the device holds at once
+      if (!allow_smem(collide_split_kernel<M, Real, Store, 0, BND>, smem) ||
+          !allow_smem(collide_split_kernel<M, Real, Store, 1, BND>, smem)) return 0;
       int per = 1;
-      cudaFuncSetAttribute(collide_split_kernel<M, Real, Store, 0, BND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      cudaFuncSetAttribute(collide_split_kernel<M, Real, Store, 1, BND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, collide_split_kernel<M, Real, Store, 0, BND>, C::THREADS, smem);
       return sm_count() * (per > 0 ? per : 1);
-    }();
+    });
+    const int resident = found > 0 ? found : sm_count();
     PlaneOffsets po;
     for (int k = 0; k < (M + 2) * Q; ++k) po.off[k] = (long long)k * c.N * (long long)sizeof(Store);
     const int ntiles = (int)grid_for(c.N, 32);
@@ -413,11 +425,8 @@ struct Launch {
   }
   static cudaError_t mlp_forward(const LaunchCtx& c, const float* feat, float* out, long long n) {
     constexpr int smem = mlp_smem<M, 1>();
-    static bool attr = false;
-    if (!attr) {
-      cudaFuncSetAttribute(mlp_forward_kernel<M>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-      attr = true;
-    }
+    static PerDevice ready;
+    ready.get(current_device(), [] { return (int)allow_smem(mlp_forward_kernel<M>, smem); });
     if (n > 0)
       mlp_forward_kernel<M><<<grid_for(n, MLP_TILE), MLP_TILE, smem, c.stream>>>(c.mlp_img, feat, out, n, c.err);
     return cudaGetLastError();
