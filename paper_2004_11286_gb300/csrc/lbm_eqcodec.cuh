@@ -66,26 +66,26 @@ struct EqRec {
   float usp[3];
 };
 
-// buf: a record buffer of N nodes (eq_rec_buf).
+// buf: a record buffer of N nodes (eq_rec_buf).  For the readers of the state.
 template <int M>
 __device__ __forceinline__ EqRec<M> load_rec(const float* __restrict__ buf, long long N, long long node, int weak) {
   const float4* q = reinterpret_cast<const float4*>(buf) + node;
   EqRec<M> r;
-  const float4 a = q[0], b = q[N];
+  const float4 a = ld<true>(q), b = ld<true>(q + N);
   r.u[0] = a.x; r.u[1] = a.y; r.u[2] = a.z; r.dT = a.w;
   r.dth = b.x; r.drho = b.y; r.dE0 = b.z; r.Gq = b.w;
   constexpr int NT = (1 + M + 3) / 4;
   float t[4 * NT];
 #pragma unroll
   for (int k = 0; k < NT; ++k) {
-    const float4 c = q[(2 + k) * N];
+    const float4 c = ld<true>(q + (2 + k) * N);
     t[4 * k] = c.x; t[4 * k + 1] = c.y; t[4 * k + 2] = c.z; t[4 * k + 3] = c.w;
   }
 #pragma unroll
   for (int s = 0; s < M; ++s) r.ra[s] = t[s];
   r.hq = t[M];
   if (weak) {
-    const float4 d = q[(2 + NT) * N];
+    const float4 d = ld<true>(q + (2 + NT) * N);
     r.usp[0] = d.x; r.usp[1] = d.y; r.usp[2] = d.z;
   } else {
     r.usp[0] = r.u[0]; r.usp[1] = r.u[1]; r.usp[2] = r.u[2];
@@ -203,15 +203,15 @@ __device__ __forceinline__ void eq_shift(const DevParams<float>& p, const EqRec<
 }
 
 // A record as loaded (the species velocity only under weak coupling).
-template <int M>
+template <int M, bool NC>
 struct RecLoad {
   static constexpr int NT = (1 + M + 3) / 4;
   float4 q[3 + NT];
   __device__ __forceinline__ RecLoad(const float* __restrict__ buf, long long N, long long node, int weak) {
     const float4* r = reinterpret_cast<const float4*>(buf) + node;
 #pragma unroll
-    for (int k = 0; k < 2 + NT; ++k) q[k] = r[k * N];
-    q[2 + NT] = weak ? r[(2 + NT) * N] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    for (int k = 0; k < 2 + NT; ++k) q[k] = ld<NC>(r + k * N);
+    q[2 + NT] = weak ? ld<NC>(r + (2 + NT) * N) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   }
 };
 
@@ -220,11 +220,11 @@ struct RecLoad {
 // velocity as data): per axis the product-form factor is r + da, r the rest
 // factor at theta_r and da = be (x^2 + dz) + ga x, with (be, ga) = (1/2, c/2),
 // or (-1, 0) for c = 0.  sp: species pairs; dth: the sender's theta - theta_r.
-template <int M>
-__device__ __forceinline__ void eq_shift_dir(const DevParams<float>& p, const RecLoad<M>& rec, bool refl, int cx,
+template <int M, bool NC>
+__device__ __forceinline__ void eq_shift_dir(const DevParams<float>& p, const RecLoad<M, NC>& rec, bool refl, int cx,
                                              int cy, int cz, float2 (&sp)[(M + 1) / 2], float& sf, float& sg,
                                              float& dth) {
-  constexpr int NT = RecLoad<M>::NT, NP = (M + 1) / 2;
+  constexpr int NT = RecLoad<M, NC>::NT, NP = (M + 1) / 2;
   const float4 A = rec.q[0], B = rec.q[1];
   float t[4 * NT];
 #pragma unroll
@@ -363,28 +363,29 @@ struct RowTerms {
   float f[3], g[3];
 };
 // K and the component of X that a face velocity of the row needs.
+template <bool NC>
 struct RowSide {
   float k[3], x;
   __device__ __forceinline__ RowSide(const float* __restrict__ side, long long N, long long snd, int cy, int cz) {
-    k[0] = side[(SP_K + 0) * N + snd];
-    k[1] = cy ? side[(SP_K + 1) * N + snd] : 0.0f;
-    k[2] = cz ? side[(SP_K + 2) * N + snd] : 0.0f;
-    x = cy * cz == 0 ? side[(SP_X + (cy ? 1 : (cz ? 2 : 0))) * N + snd] : 0.0f;
+    k[0] = ld<NC>(side + (SP_K + 0) * N + snd);
+    k[1] = cy ? ld<NC>(side + (SP_K + 1) * N + snd) : 0.0f;
+    k[2] = cz ? ld<NC>(side + (SP_K + 2) * N + snd) : 0.0f;
+    x = cy * cz == 0 ? ld<NC>(side + (SP_X + (cy ? 1 : (cz ? 2 : 0))) * N + snd) : 0.0f;
   }
 };
 // What a sender's RowTerms are formed from, as loaded.
-template <int M>
+template <int M, bool NC = false>
 struct RowLoad {
-  RecLoad<M> rec;
-  RowSide s;
+  RecLoad<M, NC> rec;
+  RowSide<NC> s;
   __device__ __forceinline__ RowLoad(const DevParams<float>& p, const float* __restrict__ side,
                                      const float* __restrict__ rin, long long snd, int cy, int cz)
       : rec(rin, p.N, snd, p.weak), s(side, p.N, snd, cy, cz) {}
 };
-template <int M>
-__device__ __forceinline__ void row_terms(const DevParams<float>& p, const RowLoad<M>& in, int cy, int cz,
+template <int M, bool NC>
+__device__ __forceinline__ void row_terms(const DevParams<float>& p, const RowLoad<M, NC>& in, int cy, int cz,
                                           RowTerms<M>& out) {
-  constexpr int NT = RecLoad<M>::NT, NP = (M + 1) / 2;
+  constexpr int NT = RecLoad<M, NC>::NT, NP = (M + 1) / 2;
   const float4 A = in.rec.q[0], W = p.weak ? in.rec.q[2 + NT] : A;
   float t[4 * NT];
 #pragma unroll
@@ -401,11 +402,11 @@ __device__ __forceinline__ void row_terms(const DevParams<float>& p, const RowLo
 // The same for one velocity (c_x given) of one sender, c_x = -1 or 1: every
 // lattice's shift and deferred term, with the sender's signs reversed where
 // the population was reflected by a wall (refl).
-template <int M>
-__device__ __forceinline__ void edge_terms(const DevParams<float>& p, const RowLoad<M>& in, bool refl, int cx, int cy,
+template <int M, bool NC>
+__device__ __forceinline__ void edge_terms(const DevParams<float>& p, const RowLoad<M, NC>& in, bool refl, int cx, int cy,
                                            int cz, float2 (&sp)[(M + 1) / 2], float& f, float& g) {
   float dth;
-  eq_shift_dir<M>(p, in.rec, refl, cx, cy, cz, sp, f, g, dth);
+  eq_shift_dir<M, NC>(p, in.rec, refl, cx, cy, cz, sp, f, g, dth);
   const float th = p.thr + dth, w0 = 1.0f - th, w1 = 0.5f * th, sg = refl ? -1.0f : 1.0f;
   g += sg * w1 * (cy ? w1 : w0) * (cz ? w1 : w0) * (cx * in.s.k[0] + cy * in.s.k[1] + cz * in.s.k[2]);
   if (cy == 0 && cz == 0) f += sg * 0.5f * cx * in.s.x;

@@ -32,6 +32,13 @@ __device__ __forceinline__ long long gtid() {
 // from the start took SMs from the blocks still to come (1024-node FP64 step
 // 79 against 62 us).
 __device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// The readers of the state (NC) are launched plainly and write none of it; with
+// ordinary loads the observables of 256^3 two-species BF16 took 5.1 against
+// 4.2 ms, the collide there 5.07 against 4.95 ms.
+template <bool NC, class T>
+__device__ __forceinline__ T ld(const T* p) {
+  if constexpr (NC) return __ldg(p); else return *p;
+}
 
 // ---------------------------------------------------------------------------
 // Energy-lattice ansatz coefficients, Eqs. (gansatz), (grad), (RcorrectionPrime):

@@ -150,7 +150,7 @@ get_pops_kernel(const DevParams<Real> p, const Store* __restrict__ pops, const R
     long long node; int slot;
     aa_read_loc<true>(parity, nb, n, i, node, slot);
     Real cf = Real(0), cg = Real(0);
-    if constexpr (i != 13) deferred_terms<Real, i, true>(side, N, nb, n, cf, cg);
+    if constexpr (i != 13) deferred_terms<Real, i, true, true>(side, N, nb, n, cf, cg);
     for (int L = 0; L < M + 2; ++L) {
       double v = (double)codec_load<Store, Real>(p, pops, (L * Q + slot) * N + node, L);
       if (L == M) v += (double)cf;

@@ -548,7 +548,7 @@ collide_split_kernel(const __grid_constant__ DevParams<Real> p, Store* __restric
           for (int x = 0; x < 3; ++x) { raw[x][0] = *lat(src[x], M); raw[x][1] = *lat(src[x], M + 1); }
           const float4 B = rec[N];
           const float hq = reinterpret_cast<const float*>(rec + (2 + M / 4) * N)[M % 4];
-          const RowSide sd(side, N, own, cy, cz);
+          const RowSide<false> sd(side, N, own, cy, cz);
           if constexpr (Last::value > 0) species(First{}, Last{}, A);
           float f[3], g[3];
           row_fg(p, M, A, B, hq, sd.k, sd.x, cy, cz, f, g);

@@ -44,14 +44,14 @@ __device__ __forceinline__ void store4(Real* __restrict__ f, const Real* v) {
 
 // The deferred terms of the population that `sender` sent in direction I,
 // for a sender whose theta is th.
-template <class Real, int I>
+template <class Real, int I, bool NC>
 __device__ __forceinline__ void incoming_corr_th(const Real* __restrict__ side, long long N, long long sender,
                                                  Real th, Real& cf, Real& cg) {
   constexpr int cx = cx_of(I), cy = cy_of(I), cz = cz_of(I);
   Real kc = Real(0);
-  if constexpr (cx != 0) kc += (cx > 0 ? side[(SP_K + 0) * N + sender] : -side[(SP_K + 0) * N + sender]);
-  if constexpr (cy != 0) kc += (cy > 0 ? side[(SP_K + 1) * N + sender] : -side[(SP_K + 1) * N + sender]);
-  if constexpr (cz != 0) kc += (cz > 0 ? side[(SP_K + 2) * N + sender] : -side[(SP_K + 2) * N + sender]);
+  if constexpr (cx != 0) kc += (cx > 0 ? ld<NC>(side + (SP_K + 0) * N + sender) : -ld<NC>(side + (SP_K + 0) * N + sender));
+  if constexpr (cy != 0) kc += (cy > 0 ? ld<NC>(side + (SP_K + 1) * N + sender) : -ld<NC>(side + (SP_K + 1) * N + sender));
+  if constexpr (cz != 0) kc += (cz > 0 ? ld<NC>(side + (SP_K + 2) * N + sender) : -ld<NC>(side + (SP_K + 2) * N + sender));
   const Real w0 = Real(1) - th, w1 = Real(0.5) * th;
   const Real w = (cx ? w1 : w0) * (cy ? w1 : w0) * (cz ? w1 : w0);   // Eq. (weights)
   cg = w * kc;
@@ -59,13 +59,13 @@ __device__ __forceinline__ void incoming_corr_th(const Real* __restrict__ side, 
   if constexpr (c2_of(I) == 1) {
     constexpr int a = cx ? 0 : (cy ? 1 : 2);
     constexpr int sg = cx + cy + cz;
-    cf = (sg > 0 ? Real(0.5) : Real(-0.5)) * side[(SP_X + a) * N + sender];
+    cf = (sg > 0 ? Real(0.5) : Real(-0.5)) * ld<NC>(side + (SP_X + a) * N + sender);
   }
 }
-template <class Real, int I>
+template <class Real, int I, bool NC = false>
 __device__ __forceinline__ void incoming_corr(const Real* __restrict__ side, long long N, long long sender,
                                               Real& cf, Real& cg) {
-  incoming_corr_th<Real, I>(side, N, sender, side[SP_THR * N + sender], cf, cg);
+  incoming_corr_th<Real, I, NC>(side, N, sender, ld<NC>(side + SP_THR * N + sender), cf, cg);
 }
 
 // Reduced-precision storage: the record of the node that sent the population
@@ -73,7 +73,8 @@ __device__ __forceinline__ void incoming_corr(const Real* __restrict__ side, lon
 // that population (lbm_eqcodec.cuh) and its deferred terms.  The sender is
 // n - c_I; with walls, a population arriving from beyond a wall is n's own
 // population of direction opp(I) reflected, so it was stored with n's shift
-// for opp(I) and carries n's terms for I negated.
+// for opp(I) and carries n's terms for I negated.  For the readers of the state
+// and its initialisation.
 template <int M, int I, bool WALL>
 __device__ __forceinline__ void eq_incoming(const DevParams<float>& p, const float* __restrict__ side,
                                             const Nbr& nb, long long n, int parity, float& cf, float& cg,
@@ -91,7 +92,7 @@ __device__ __forceinline__ void eq_incoming(const DevParams<float>& p, const flo
   else eq_shift<M, I>(p, r, sh);
   cf = 0.0f; cg = 0.0f;
   if constexpr (I != 13) {
-    incoming_corr_th<float, I>(side, N, snd, p.thr + r.dth, cf, cg);
+    incoming_corr_th<float, I, true>(side, N, snd, p.thr + r.dth, cf, cg);
     if (WALL && refl) { cf = -cf; cg = -cg; }
   }
 }
@@ -100,18 +101,18 @@ __device__ __forceinline__ void eq_incoming(const DevParams<float>& p, const flo
 // With walls (WALL), one arriving from beyond a wall is the node's own
 // population of direction opp(I) reflected, so its terms are the node's own
 // for opp(I): those of I at the node, negated (w_opp(I) = w_I, c_opp(I) = -c_I).
-template <class Real, int I, bool WALL>
+template <class Real, int I, bool WALL, bool NC = false>
 __device__ __forceinline__ void deferred_terms(const Real* __restrict__ side, long long N, const Nbr& nb,
                                                long long n, Real& cf, Real& cg) {
   if constexpr (WALL) {
     if (arrives_from_wall(nb, I)) {
-      incoming_corr<Real, I>(side, N, n, cf, cg);
+      incoming_corr<Real, I, NC>(side, N, n, cf, cg);
       cf = -cf;
       cg = -cg;
       return;
     }
   }
-  incoming_corr<Real, I>(side, N, nb.idx(-cx_of(I), -cy_of(I), -cz_of(I)), cf, cg);
+  incoming_corr<Real, I, NC>(side, N, nb.idx(-cx_of(I), -cy_of(I), -cz_of(I)), cf, cg);
 }
 
 // The decoding terms of the population arriving at n in direction I for the
@@ -128,7 +129,7 @@ __device__ __forceinline__ void incoming_terms(const DevParams<Real>& p, const R
   } else {
 #pragma unroll
     for (int L = 0; L < M + 2; ++L) sh[L] = Real(0);
-    if constexpr (I != 13) deferred_terms<Real, I, true>(side, p.N, nb, n, cf, cg);
+    if constexpr (I != 13) deferred_terms<Real, I, true, true>(side, p.N, nb, n, cf, cg);
   }
 }
 
@@ -156,7 +157,7 @@ __device__ __forceinline__ void row_populations(const DevParams<float>& p, const
     const unsigned rb = (cy == 0 ? nb.ys[1] : (cy > 0 ? nb.ys[0] : nb.ys[2])) +
                         (cz == 0 ? nb.zs[1] : (cz > 0 ? nb.zs[0] : nb.zs[2]));
     RowTerms<M> t;
-    row_terms<M>(p, RowLoad<M>(p, side, rin, (long long)(rb + nb.xs[1]), cy, cz), cy, cz, t);
+    row_terms<M>(p, RowLoad<M, true>(p, side, rin, (long long)(rb + nb.xs[1]), cy, cz), cy, cz, t);
 #pragma unroll
     for (int q = 0; q < NP; ++q) {
       t.sp[q][2].x = __shfl_up_sync(0xffffffffu, t.sp[q][2].x, 1);
@@ -177,7 +178,7 @@ __device__ __forceinline__ void row_populations(const DevParams<float>& p, const
       const bool refl = arrives_from_wall_c(nb, cx);
       float2 sp[NP];
       float fv, gv;
-      edge_terms<M>(p, RowLoad<M>(p, side, rin, refl ? n : (long long)(rb + (cx > 0 ? nb.xs[0] : nb.xs[2])), cy, cz), refl,
+      edge_terms<M>(p, RowLoad<M, true>(p, side, rin, refl ? n : (long long)(rb + (cx > 0 ? nb.xs[0] : nb.xs[2])), cy, cz), refl,
                     cx, cy, cz, sp, fv, gv);
 #pragma unroll
       for (int q = 0; q < NP; ++q) { if (cx > 0) t.sp[q][2] = sp[q]; else t.sp[q][0] = sp[q]; }
