@@ -11,6 +11,7 @@
 #include "lbm_device.cuh"
 #include "lbm_eqcodec.cuh"
 #include "lbm_dispatch.h"
+#include "lbm_halo.h"
 #include "lbm_train.h"
 
 namespace {
@@ -998,12 +999,15 @@ static lbm_status halo_check(lbm_mix_t h, int face, int ghost) {
   return h->ready();
 }
 
+static lbm::HaloLayout halo_layout(lbm_mix_t h, int ghost) {
+  return lbm::halo_layout((size_t)(h->M + 2) * 27, (size_t)ghost * (size_t)h->p64.nx * (size_t)h->p64.ny,
+                          store_elem_bytes(h->prec), lbm::NSIDE, side_elem_bytes(h->prec), 2 * (size_t)h->p64.rec_w);
+}
+
 lbm_status lbm_mix_halo_bytes(lbm_mix_t h, int ghost, size_t* bytes) {
   if (!h || !bytes) return LBM_ERR_ARG;
   if (ghost < 1) return h->fail(LBM_ERR_ARG, "ghost must be >= 1");
-  const size_t plane = (size_t)h->p64.nx * (size_t)h->p64.ny;
-  *bytes = (size_t)ghost * plane * ((size_t)(h->M + 2) * 27 * store_elem_bytes(h->prec) +
-                                    (size_t)lbm::NSIDE * side_elem_bytes(h->prec) + 2 * (size_t)h->p64.rec_w * 4);
+  *bytes = halo_layout(h, ghost).bytes;
   return LBM_OK;
 }
 
@@ -1017,17 +1021,18 @@ static lbm_status halo_move(lbm_mix_t h, int face, int ghost, void* buf, int unp
   const long long seg = (long long)ghost * plane;
   const size_t es = store_elem_bytes(h->prec), ss = side_elem_bytes(h->prec);
   const long long nf = (long long)(h->M + 2) * 27;
+  const lbm::HaloLayout lay = halo_layout(h, ghost);
   char* b = (char*)buf;
   cudaError_t e;
   if (es == 8) e = halo_copy<double>(h->pops, b, nf, N, z0 * plane, seg, unpack, h->stream);
   else if (es == 4) e = halo_copy<float>(h->pops, b, nf, N, z0 * plane, seg, unpack, h->stream);
   else e = halo_copy<unsigned short>(h->pops, b, nf, N, z0 * plane, seg, unpack, h->stream);
-  b += (size_t)nf * seg * es;
+  b = (char*)buf + lay.side;
   if (e == cudaSuccess) {
     if (ss == 8) e = halo_copy<double>(h->scratch, b, lbm::NSIDE, N, z0 * plane, seg, unpack, h->stream);
     else e = halo_copy<float>(h->scratch, b, lbm::NSIDE, N, z0 * plane, seg, unpack, h->stream);
   }
-  b += (size_t)lbm::NSIDE * seg * ss;
+  b = (char*)buf + lay.rec;
   const long long rw = h->p64.rec_w;
   if (e == cudaSuccess && rw > 0)
     e = halo_copy<float>((float*)h->scratch + lbm::eq_rec_offset(N), b, 2 * (rw / 4), 4 * N, z0 * plane * 4, seg * 4, unpack,
