@@ -130,7 +130,7 @@ __device__ __forceinline__ float eq_shift_f(const DevParams<float>& p, int M, co
 // (energy_rest), so the bracket's deviation is w_I dE_I + (w_I - W_I) (E_I - dE_I).
 template <class Real>
 __device__ __forceinline__ Real energy_rest(const DevParams<Real>& p, int M, int k2) {
-  return p.RL[M + 1] - Real(1.5) * p.RL[M] * p.thr + Real(0.5) * Real(k2) * p.RL[M];
+  return fma1(Real(0.5) * Real(k2), p.RL[M], fma1(Real(-1.5) * p.RL[M], p.thr, p.RL[M + 1]));
 }
 template <int I>
 __device__ __forceinline__ float eq_shift_g(const DevParams<float>& p, int M, const float (&u)[3], float dth,
@@ -215,86 +215,25 @@ struct RecLoad {
   }
 };
 
-// Equilibrium shifts of every lattice for one velocity (cx, cy, cz) given at
-// run time, from the sender's record (eq_shift of lbm_eqcodec.cuh with the
-// velocity as data): per axis the product-form factor is r + da, r the rest
-// factor at theta_r and da = be (x^2 + dz) + ga x, with (be, ga) = (1/2, c/2),
-// or (-1, 0) for c = 0.  sp: species pairs; dth: the sender's theta - theta_r.
-template <int M, bool NC>
-__device__ __forceinline__ void eq_shift_dir(const DevParams<float>& p, const RecLoad<M, NC>& rec, bool refl, int cx,
-                                             int cy, int cz, float2 (&sp)[(M + 1) / 2], float& sf, float& sg,
-                                             float& dth) {
-  constexpr int NT = RecLoad<M, NC>::NT, NP = (M + 1) / 2;
-  const float4 A = rec.q[0], B = rec.q[1];
-  float t[4 * NT];
-#pragma unroll
-  for (int k = 0; k < NT; ++k) {
-    const float4 c = rec.q[2 + k];
-    t[4 * k] = c.x; t[4 * k + 1] = c.y; t[4 * k + 2] = c.z; t[4 * k + 3] = c.w;
-  }
-  const float sgn = refl ? -1.0f : 1.0f;          // f^eq of the opposite velocity is that of -u
-  float u[3] = {sgn * A.x, sgn * A.y, sgn * A.z};
-  dth = B.x;
-  const float bx = cx ? 0.5f : -1.0f, by = cy ? 0.5f : -1.0f, bz = cz ? 0.5f : -1.0f;
-  const float gx = 0.5f * cx, gy = 0.5f * cy, gz = 0.5f * cz;
-  const int k2 = cx * cx + cy * cy + cz * cz;
-  // mixture velocity: da = q + be dth with q = be x^2 + ga x
-  const float x2[3] = {u[0] * u[0], u[1] * u[1], u[2] * u[2]};
-  const float qx = bx * x2[0] + gx * u[0], qy = by * x2[1] + gy * u[1], qz = bz * x2[2] + gz * u[2];
-  {
-    float vx = qx, vy = qy, vz = qz;
-    if (p.weak) {
-      const float4 w = rec.q[2 + NT];
-      const float s0 = sgn * w.x, s1 = sgn * w.y, s2 = sgn * w.z;
-      vx = bx * s0 * s0 + gx * s0; vy = by * s1 * s1 + gy * s1; vz = bz * s2 * s2 + gz * s2;
-    }
-    const float2 ax = bcast<float2>(vx + (cx ? 0.0f : 1.0f)), ay = bcast<float2>(vy + (cy ? 0.0f : 1.0f)),
-                 az = bcast<float2>(vz + (cz ? 0.0f : 1.0f));
-    const float2 T = bcast<float2>(p.Tr + A.w);
-#pragma unroll
-    for (int q = 0; q < NP; ++q) {
-      const int a0 = 2 * q, a1 = 2 * q + 1 < M ? 2 * q + 1 : 2 * q;
-      const float2 z = mul2(make_float2(p.R_a[a0], p.R_a[a1]), T);
-      const float2 f = mul2(mul2(fma2(bcast<float2>(bx), z, ax), fma2(bcast<float2>(by), z, ay)),
-                            fma2(bcast<float2>(bz), z, az));
-      const float2 ra = add2(make_float2(p.RL[a0], p.RL[a1]), make_float2(t[a0], t[2 * q + 1]));
-      sp[q] = fma2(ra, f, make_float2(-p.bref[a0][k2], -p.bref[a1][k2]));
-    }
-  }
-  const float r1 = 0.5f * p.thr, r0 = 1.0f - p.thr;
-  const float rx = cx ? r1 : r0, ry = cy ? r1 : r0, rz = cz ? r1 : r0;
-  const float rho = p.RL[M] + B.y, rr = rx * ry * rz;
-  const float wx = bx * dth, wy = by * dth, wz = bz * dth;      // w_c(theta) - w_c(theta_r)
-  {
-    const float dx = qx + wx, dy = qy + wy, dz = qz + wz, az = rz + dz;
-    sf = rho * (dx * ((ry + dy) * az) + rx * (dy * az + ry * dz)) + B.y * rr;
-  }
-  const float uc = cx * u[0] + cy * u[1] + cz * u[2];
-  const float dEi = B.z + 0.5f * k2 * B.y + B.w * uc * uc;
-  const float oz = rz + wz, oyz = (ry + wy) * oz;
-  sg = (rx + wx) * oyz * (dEi + t[M] * uc) + (wx * oyz + rx * (wy * oz + ry * wz)) * energy_rest(p, M, k2);
-  if (k2 <= 1) {
-    const float theta = p.thr + dth, z1 = 1.0f - 3.0f * theta;
-    const float zb = 0.5f * (z1 * (B.y * theta + p.RL[M] * dth) - 3.0f * dth * p.Pr), zG = z1 * B.w * theta;
-    if (k2 == 0) sg += 3.0f * zb + zG * (x2[0] + x2[1] + x2[2]);
-    else sg -= 0.5f * (zb + zG * (cx ? x2[0] : (cy ? x2[1] : x2[2])));
-  }
-}
-
 // What one sender adds to the populations it sent along the three velocities
 // (c_x = -1, 0, 1; c_y; c_z) of a row: the equilibrium shifts of every
-// lattice (as eq_shift_dir) and, on f and g, the deferred terms
+// lattice (the values of eq_shift) and, on f and g, the deferred terms
 // c . X / 2 (faces) and w(theta) c . K.  The (y, z) factors, and all that
 // depends on the sender alone, are formed once for the three.
+// Which lane forms a sender's terms depends on where the receiver falls in its
+// warp, so every operation's rounding is fixed here (paired instructions, and
+// the scalar operations of lbm_helpers.cuh that the compiler does not
+// contract): the same sender gives the same bits wherever its terms are
+// formed, and a node's result does not depend on its place in a warp.
 // (y, z) factors of a row for the species: per axis Psi_c = a + be z.
 struct RowSpecies {
   float by, bz, ay, az, x2, hx;
   float T;
   int k2;
   __device__ __forceinline__ RowSpecies(float ux, float uy, float uz, float T_, int cy, int cz)
-      : by(cy ? 0.5f : -1.0f), bz(cz ? 0.5f : -1.0f), x2(ux * ux), hx(0.5f * ux), T(T_), k2(cy * cy + cz * cz) {
-    ay = by * uy * uy + 0.5f * cy * uy + (cy ? 0.0f : 1.0f);
-    az = bz * uz * uz + 0.5f * cz * uz + (cz ? 0.0f : 1.0f);
+      : by(cy ? 0.5f : -1.0f), bz(cz ? 0.5f : -1.0f), x2(mul1(ux, ux)), hx(mul1(0.5f, ux)), T(T_), k2(cy * cy + cz * cz) {
+    ay = fma1(mul1(by, uy), uy, fma1(0.5f * cy, uy, cy ? 0.0f : 1.0f));
+    az = fma1(mul1(bz, uz), uz, fma1(0.5f * cz, uz, cz ? 0.0f : 1.0f));
   }
 };
 // Shifts of species a0, a1 with densities RL + d.
@@ -316,43 +255,47 @@ __device__ __forceinline__ void row_species(const DevParams<float>& p, const Row
 __device__ __forceinline__ void row_fg(const DevParams<float>& p, int M, float4 A, float4 B, float hq,
                                        const float (&k)[3], float x, int cy, int cz, float (&f)[3], float (&g)[3]) {
   const float dth = B.x, drho = B.y;
-  const float by = cy ? 0.5f : -1.0f, bz = cz ? 0.5f : -1.0f;
+  const float by = cy ? 0.5f : -1.0f, bz = cz ? 0.5f : -1.0f, sy = (float)cy, sz = (float)cz;
   const int kyz = cy * cy + cz * cz;
-  const float x2 = A.x * A.x, hx = 0.5f * A.x;
-  const float r1 = 0.5f * p.thr, r0 = 1.0f - p.thr;
-  const float ry = cy ? r1 : r0, rz = cz ? r1 : r0, ryz = ry * rz;
-  const float wy = by * dth, wz = bz * dth, wx = 0.5f * dth;    // w_c(theta) - w_c(theta_r); x: c = 0 gives -dth
+  const float x2 = mul1(A.x, A.x), hx = mul1(0.5f, A.x);
+  const float r1 = mul1(0.5f, p.thr), r0 = sub1(1.0f, p.thr);
+  const float ry = cy ? r1 : r0, rz = cz ? r1 : r0, ryz = mul1(ry, rz);
+  const float wy = mul1(by, dth), wz = mul1(bz, dth), wx = mul1(0.5f, dth);    // w_c(theta) - w_c(theta_r); x: c = 0 gives -dth
   {
-    const float rho = p.RL[M] + drho;
-    const float dy = by * A.y * A.y + 0.5f * cy * A.y + wy, dz = bz * A.z * A.z + 0.5f * cz * A.z + wz;
-    const float az = rz + dz, ayz = (ry + dy) * az, fyz = dy * az + ry * dz;
-    const float hs = 0.5f * (x2 + dth), cf = 0.5f * x;
-    const float e1 = r1 * fyz, d1 = drho * (r1 * ryz);
-    f[0] = rho * ((hs - hx) * ayz + e1) + d1;
-    f[1] = rho * (r0 * fyz - (hs + hs) * ayz) + drho * (r0 * ryz);
-    f[2] = rho * ((hs + hx) * ayz + e1) + d1;
-    if (kyz == 0) { f[0] -= cf; f[2] += cf; }
-    if (kyz == 1) f[1] += (cy + cz) * cf;
+    const float rho = add1(p.RL[M], drho);
+    const float dy = fma1(mul1(by, A.y), A.y, fma1(mul1(0.5f, sy), A.y, wy));
+    const float dz = fma1(mul1(bz, A.z), A.z, fma1(mul1(0.5f, sz), A.z, wz));
+    const float az = add1(rz, dz), ayz = mul1(add1(ry, dy), az), fyz = fma1(dy, az, mul1(ry, dz));
+    const float hs = mul1(0.5f, fma1(A.x, A.x, dth)), cf = mul1(0.5f, x);
+    const float e1 = mul1(r1, fyz), d1 = mul1(drho, mul1(r1, ryz));
+    f[0] = fma1(rho, fma1(sub1(hs, hx), ayz, e1), d1);
+    f[1] = fma1(rho, fma1(mul1(-2.0f, hs), ayz, mul1(r0, fyz)), mul1(drho, mul1(r0, ryz)));
+    f[2] = fma1(rho, fma1(add1(hs, hx), ayz, e1), d1);
+    if (kyz == 0) { f[0] = sub1(f[0], cf); f[2] = add1(f[2], cf); }
+    if (kyz == 1) f[1] = fma1(add1(sy, sz), cf, f[1]);
   }
-  const float oz = rz + wz, oyz = (ry + wy) * oz, dyz = wy * oz + ry * wz;
-  const float w1 = (r1 + wx) * oyz, w0 = (r0 - dth) * oyz;
-  const float c0 = (r0 * dyz - dth * oyz) * energy_rest(p, M, kyz), c1 = (wx * oyz + r1 * dyz) * energy_rest(p, M, kyz + 1);
-  const float uyz = cy * A.y + cz * A.z, kk = cy * k[1] + cz * k[2];
-  const float e0 = B.z + 0.5f * kyz * drho + kk, e1 = e0 + 0.5f * drho;
-  const float um = uyz - A.x, up = uyz + A.x;
-  g[0] = w1 * (e1 + um * (B.w * um + hq) - k[0]) + c1;
-  g[1] = w0 * (e0 + uyz * (B.w * uyz + hq)) + c0;
-  g[2] = w1 * (e1 + up * (B.w * up + hq) + k[0]) + c1;
+  const float oz = add1(rz, wz), oyz = mul1(add1(ry, wy), oz), dyz = fma1(wy, oz, mul1(ry, wz));
+  const float w1 = mul1(add1(r1, wx), oyz), w0 = mul1(sub1(r0, dth), oyz);
+  const float c0 = mul1(fma1(-dth, oyz, mul1(r0, dyz)), energy_rest(p, M, kyz));
+  const float c1 = mul1(fma1(wx, oyz, mul1(r1, dyz)), energy_rest(p, M, kyz + 1));
+  const float uyz = fma1(sy, A.y, mul1(sz, A.z)), kk = fma1(sy, k[1], mul1(sz, k[2]));
+  const float e0 = add1(fma1(mul1(0.5f, (float)kyz), drho, B.z), kk), e1 = fma1(0.5f, drho, e0);
+  const float um = sub1(uyz, A.x), up = add1(uyz, A.x);
+  g[0] = fma1(w1, sub1(fma1(um, fma1(B.w, um, hq), e1), k[0]), c1);
+  g[1] = fma1(w0, fma1(uyz, fma1(B.w, uyz, hq), e0), c0);
+  g[2] = fma1(w1, add1(fma1(up, fma1(B.w, up, hq), e1), k[0]), c1);
   if (kyz <= 1) {
-    const float theta = p.thr + dth, z1 = 1.0f - 3.0f * theta;
-    const float zb = 0.5f * (z1 * (drho * theta + p.RL[M] * dth) - 3.0f * dth * p.Pr), zG = z1 * B.w * theta;
+    const float theta = add1(p.thr, dth), z1 = fma1(-3.0f, theta, 1.0f);
+    const float zb = mul1(0.5f, fma1(z1, fma1(drho, theta, mul1(p.RL[M], dth)), mul1(mul1(-3.0f, dth), p.Pr)));
+    const float zG = mul1(mul1(z1, B.w), theta);
     if (kyz == 0) {
-      const float bx = 0.5f * (zb + zG * x2);
-      g[0] -= bx;
-      g[1] += 3.0f * zb + zG * (x2 + A.y * A.y + A.z * A.z);
-      g[2] -= bx;
+      const float bx = mul1(0.5f, fma1(zG, x2, zb)), u2 = fma1(A.x, A.x, fma1(A.y, A.y, mul1(A.z, A.z)));
+      g[0] = sub1(g[0], bx);
+      g[1] = add1(g[1], fma1(zG, u2, mul1(3.0f, zb)));
+      g[2] = sub1(g[2], bx);
     } else {
-      g[1] -= 0.5f * (zb + zG * (cy ? A.y * A.y : A.z * A.z));
+      const float c = cy ? A.y : A.z;
+      g[1] = fma1(-0.5f, fma1(zG, mul1(c, c), zb), g[1]);
     }
   }
 }
@@ -393,23 +336,34 @@ __device__ __forceinline__ void row_terms(const DevParams<float>& p, const RowLo
     const float4 c = in.rec.q[2 + k];
     t[4 * k] = c.x; t[4 * k + 1] = c.y; t[4 * k + 2] = c.z; t[4 * k + 3] = c.w;
   }
-  const RowSpecies r(W.x, W.y, W.z, p.Tr + A.w, cy, cz);
+  const RowSpecies r(W.x, W.y, W.z, add1(p.Tr, A.w), cy, cz);
 #pragma unroll
   for (int q = 0; q < NP; ++q)
     row_species(p, r, 2 * q, 2 * q + 1 < M ? 2 * q + 1 : 2 * q, make_float2(t[2 * q], t[2 * q + 1]), out.sp[q]);
   row_fg(p, M, A, in.rec.q[1], t[M], in.s.k, in.s.x, cy, cz, out.f, out.g);
 }
-// The same for one velocity (c_x given) of one sender, c_x = -1 or 1: every
-// lattice's shift and deferred term, with the sender's signs reversed where
-// the population was reflected by a wall (refl).
+// The same for one velocity (c_x = -1 or 1 given) of one sender.  refl: the
+// population is the node's own of the opposite velocity, reflected by a wall;
+// f^eq of the opposite velocity is that of -u, and the deferred terms change
+// sign, so the row is formed with the sender's vectors reversed.
 template <int M, bool NC>
-__device__ __forceinline__ void edge_terms(const DevParams<float>& p, const RowLoad<M, NC>& in, bool refl, int cx, int cy,
+__device__ __forceinline__ void edge_terms(const DevParams<float>& p, RowLoad<M, NC> in, bool refl, int cx, int cy,
                                            int cz, float2 (&sp)[(M + 1) / 2], float& f, float& g) {
-  float dth;
-  eq_shift_dir<M, NC>(p, in.rec, refl, cx, cy, cz, sp, f, g, dth);
-  const float th = p.thr + dth, w0 = 1.0f - th, w1 = 0.5f * th, sg = refl ? -1.0f : 1.0f;
-  g += sg * w1 * (cy ? w1 : w0) * (cz ? w1 : w0) * (cx * in.s.k[0] + cy * in.s.k[1] + cz * in.s.k[2]);
-  if (cy == 0 && cz == 0) f += sg * 0.5f * cx * in.s.x;
+  if (refl) {
+    float4& A = in.rec.q[0];
+    float4& W = in.rec.q[2 + RecLoad<M, NC>::NT];
+    A.x = -A.x; A.y = -A.y; A.z = -A.z;
+    W.x = -W.x; W.y = -W.y; W.z = -W.z;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) in.s.k[c] = -in.s.k[c];
+    in.s.x = -in.s.x;
+  }
+  RowTerms<M> t;
+  row_terms<M>(p, in, cy, cz, t);
+#pragma unroll
+  for (int q = 0; q < RowTerms<M>::NP; ++q) sp[q] = cx > 0 ? t.sp[q][2] : t.sp[q][0];
+  f = cx > 0 ? t.f[2] : t.f[0];
+  g = cx > 0 ? t.g[2] : t.g[0];
 }
 
 // The record of a node from its coupled moments, in FP64 (initialisation

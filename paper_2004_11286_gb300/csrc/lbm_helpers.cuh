@@ -208,6 +208,17 @@ __device__ __forceinline__ float2 sub2(float2 a, float2 b) {
   return d;
 }
 
+// Scalar arithmetic with the rounding of each operation fixed: the compiler
+// contracts a product and a sum into one operation only where fma1 is written.
+__device__ __forceinline__ float mul1(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float add1(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float sub1(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float fma1(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double mul1(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ double add1(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ double sub1(double a, double b) { return __dsub_rn(a, b); }
+__device__ __forceinline__ double fma1(double a, double b, double c) { return __fma_rn(a, b, c); }
+
 // Two species' values of one quantity.
 template <class Real> struct Pair;
 template <> struct Pair<float> { using T = float2; };

@@ -514,7 +514,7 @@ collide_split_kernel(const __grid_constant__ DevParams<Real> p, Store* __restric
             }
           }
           const float4 w = p.weak ? rec[(2 + (1 + M + 3) / 4) * N] : A;
-          const RowSpecies r(w.x, w.y, w.z, p.Tr + A.w, cy, cz);
+          const RowSpecies r(w.x, w.y, w.z, add1(p.Tr, A.w), cy, cz);
 #pragma unroll
           for (int k = 0; k < K; ++k) {
             const int q = q0 + k;
