@@ -251,9 +251,12 @@ __device__ __forceinline__ void row_species(const DevParams<float>& p, const Row
   out[2] = fma2(yz, add2(hs, bcast<float2>(r.hx)), r1);
 }
 // f and g: A, B the record's first two float4s, hq, K, and the component x of
-// X that a face velocity of the row needs.
+// X that a face velocity of the row needs.  SEP: the deferred terms apart, in
+// cf and cg (for the readers that add the parts in FP64).
+template <bool SEP>
 __device__ __forceinline__ void row_fg(const DevParams<float>& p, int M, float4 A, float4 B, float hq,
-                                       const float (&k)[3], float x, int cy, int cz, float (&f)[3], float (&g)[3]) {
+                                       const float (&k)[3], float x, int cy, int cz, float (&f)[3], float (&g)[3],
+                                       float* cf_out, float* cg_out) {
   const float dth = B.x, drho = B.y;
   const float by = cy ? 0.5f : -1.0f, bz = cz ? 0.5f : -1.0f, sy = (float)cy, sz = (float)cz;
   const int kyz = cy * cy + cz * cz;
@@ -271,19 +274,31 @@ __device__ __forceinline__ void row_fg(const DevParams<float>& p, int M, float4 
     f[0] = fma1(rho, fma1(sub1(hs, hx), ayz, e1), d1);
     f[1] = fma1(rho, fma1(mul1(-2.0f, hs), ayz, mul1(r0, fyz)), mul1(drho, mul1(r0, ryz)));
     f[2] = fma1(rho, fma1(add1(hs, hx), ayz, e1), d1);
-    if (kyz == 0) { f[0] = sub1(f[0], cf); f[2] = add1(f[2], cf); }
-    if (kyz == 1) f[1] = fma1(add1(sy, sz), cf, f[1]);
+    if constexpr (SEP) {
+      cf_out[0] = kyz == 0 ? -cf : 0.0f;
+      cf_out[1] = kyz == 1 ? mul1(add1(sy, sz), cf) : 0.0f;
+      cf_out[2] = kyz == 0 ? cf : 0.0f;
+    } else {
+      if (kyz == 0) { f[0] = sub1(f[0], cf); f[2] = add1(f[2], cf); }
+      if (kyz == 1) f[1] = fma1(add1(sy, sz), cf, f[1]);
+    }
   }
   const float oz = add1(rz, wz), oyz = mul1(add1(ry, wy), oz), dyz = fma1(wy, oz, mul1(ry, wz));
   const float w1 = mul1(add1(r1, wx), oyz), w0 = mul1(sub1(r0, dth), oyz);
   const float c0 = mul1(fma1(-dth, oyz, mul1(r0, dyz)), energy_rest(p, M, kyz));
   const float c1 = mul1(fma1(wx, oyz, mul1(r1, dyz)), energy_rest(p, M, kyz + 1));
   const float uyz = fma1(sy, A.y, mul1(sz, A.z)), kk = fma1(sy, k[1], mul1(sz, k[2]));
-  const float e0 = add1(fma1(mul1(0.5f, (float)kyz), drho, B.z), kk), e1 = fma1(0.5f, drho, e0);
+  const float es = fma1(mul1(0.5f, (float)kyz), drho, B.z), e0 = SEP ? es : add1(es, kk), e1 = fma1(0.5f, drho, e0);
   const float um = sub1(uyz, A.x), up = add1(uyz, A.x);
-  g[0] = fma1(w1, sub1(fma1(um, fma1(B.w, um, hq), e1), k[0]), c1);
+  const float b0 = fma1(um, fma1(B.w, um, hq), e1), b2 = fma1(up, fma1(B.w, up, hq), e1);
+  g[0] = fma1(w1, SEP ? b0 : sub1(b0, k[0]), c1);
   g[1] = fma1(w0, fma1(uyz, fma1(B.w, uyz, hq), e0), c0);
-  g[2] = fma1(w1, add1(fma1(up, fma1(B.w, up, hq), e1), k[0]), c1);
+  g[2] = fma1(w1, SEP ? b2 : add1(b2, k[0]), c1);
+  if constexpr (SEP) {
+    cg_out[0] = mul1(w1, sub1(kk, k[0]));
+    cg_out[1] = mul1(w0, kk);
+    cg_out[2] = mul1(w1, add1(kk, k[0]));
+  }
   if (kyz <= 1) {
     const float theta = add1(p.thr, dth), z1 = fma1(-3.0f, theta, 1.0f);
     const float zb = mul1(0.5f, fma1(z1, fma1(drho, theta, mul1(p.RL[M], dth)), mul1(mul1(-3.0f, dth), p.Pr)));
@@ -299,11 +314,12 @@ __device__ __forceinline__ void row_fg(const DevParams<float>& p, int M, float4 
     }
   }
 }
-template <int M>
+template <int M, bool SEP = false>
 struct RowTerms {
   static constexpr int NP = (M + 1) / 2;
   float2 sp[NP][3];
   float f[3], g[3];
+  float cf[SEP ? 3 : 1], cg[SEP ? 3 : 1];
 };
 // K and the component of X that a face velocity of the row needs.
 template <bool NC>
@@ -325,9 +341,9 @@ struct RowLoad {
                                      const float* __restrict__ rin, long long snd, int cy, int cz)
       : rec(rin, p.N, snd, p.weak), s(side, p.N, snd, cy, cz) {}
 };
-template <int M, bool NC>
+template <int M, bool NC, bool SEP>
 __device__ __forceinline__ void row_terms(const DevParams<float>& p, const RowLoad<M, NC>& in, int cy, int cz,
-                                          RowTerms<M>& out) {
+                                          RowTerms<M, SEP>& out) {
   constexpr int NT = RecLoad<M, NC>::NT, NP = (M + 1) / 2;
   const float4 A = in.rec.q[0], W = p.weak ? in.rec.q[2 + NT] : A;
   float t[4 * NT];
@@ -340,15 +356,16 @@ __device__ __forceinline__ void row_terms(const DevParams<float>& p, const RowLo
 #pragma unroll
   for (int q = 0; q < NP; ++q)
     row_species(p, r, 2 * q, 2 * q + 1 < M ? 2 * q + 1 : 2 * q, make_float2(t[2 * q], t[2 * q + 1]), out.sp[q]);
-  row_fg(p, M, A, in.rec.q[1], t[M], in.s.k, in.s.x, cy, cz, out.f, out.g);
+  row_fg<SEP>(p, M, A, in.rec.q[1], t[M], in.s.k, in.s.x, cy, cz, out.f, out.g, out.cf, out.cg);
 }
 // The same for one velocity (c_x = -1 or 1 given) of one sender.  refl: the
 // population is the node's own of the opposite velocity, reflected by a wall;
 // f^eq of the opposite velocity is that of -u, and the deferred terms change
 // sign, so the row is formed with the sender's vectors reversed.
-template <int M, bool NC>
+template <int M, bool NC, bool SEP = false>
 __device__ __forceinline__ void edge_terms(const DevParams<float>& p, RowLoad<M, NC> in, bool refl, int cx, int cy,
-                                           int cz, float2 (&sp)[(M + 1) / 2], float& f, float& g) {
+                                           int cz, float2 (&sp)[(M + 1) / 2], float& f, float& g,
+                                           float* cf = nullptr, float* cg = nullptr) {
   if (refl) {
     float4& A = in.rec.q[0];
     float4& W = in.rec.q[2 + RecLoad<M, NC>::NT];
@@ -358,12 +375,16 @@ __device__ __forceinline__ void edge_terms(const DevParams<float>& p, RowLoad<M,
     for (int c = 0; c < 3; ++c) in.s.k[c] = -in.s.k[c];
     in.s.x = -in.s.x;
   }
-  RowTerms<M> t;
+  RowTerms<M, SEP> t;
   row_terms<M>(p, in, cy, cz, t);
 #pragma unroll
   for (int q = 0; q < RowTerms<M>::NP; ++q) sp[q] = cx > 0 ? t.sp[q][2] : t.sp[q][0];
   f = cx > 0 ? t.f[2] : t.f[0];
   g = cx > 0 ? t.g[2] : t.g[0];
+  if constexpr (SEP) {
+    *cf = cx > 0 ? t.cf[2] : t.cf[0];
+    *cg = cx > 0 ? t.cg[2] : t.cg[0];
+  }
 }
 
 // The record of a node from its coupled moments, in FP64 (initialisation

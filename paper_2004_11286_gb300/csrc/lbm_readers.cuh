@@ -135,13 +135,17 @@ get_pops_kernel(const DevParams<Real> p, const Store* __restrict__ pops, const R
   const long long N = p.N, n = active ? gtid() : N - 1;
   const Nbr nb = make_nbr(p, n);
   if constexpr (kEqCodec<Store, Real>) {
-    row_populations<M, Store>(p, side, parity, nb, n, active,
-                              [&](int i, int, int, int, int slot, long long node, const float (&sh)[M + 2]) {
+    row_populations<M, Store, true>(p, side, parity, nb, n, active,
+                                    [&](int i, int, int, int, int slot, long long node, const float (&sh)[M + 2], float cf,
+                                        float cg) {
       if (!active) return;
 #pragma unroll
-      for (int L = 0; L < M + 2; ++L)
-        out[(L * Q + i) * N + n] = base[L * Q + i] + ((double)codec_load<Store, Real>(p, pops, (L * Q + slot) * N + node, L) +
-                                                      (double)sh[L]);
+      for (int L = 0; L < M + 2; ++L) {
+        double v = (double)codec_load<Store, Real>(p, pops, (L * Q + slot) * N + node, L) + (double)sh[L];
+        if (L == M) v += (double)cf;
+        if (L == M + 1) v += (double)cg;
+        out[(L * Q + i) * N + n] = base[L * Q + i] + v;
+      }
     });
     return;
   }
@@ -209,8 +213,9 @@ set_pops_kernel(const DevParams<Real> p, Store* __restrict__ pops, const Real* _
   const long long N = p.N, n = active ? gtid() : N - 1;
   const Nbr nb = make_nbr(p, n);
   if constexpr (kEqCodec<Store, Real>) {
-    row_populations<M, Store>(p, side, parity, nb, n, active,
-                              [&](int i, int, int, int, int slot, long long node, const float (&sh)[M + 2]) {
+    row_populations<M, Store, true>(p, side, parity, nb, n, active,
+                                    [&](int i, int, int, int, int slot, long long node, const float (&sh)[M + 2], float,
+                                        float) {
       if (!active) return;
 #pragma unroll
       for (int L = 0; L < M + 2; ++L)

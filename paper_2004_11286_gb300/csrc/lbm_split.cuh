@@ -551,7 +551,7 @@ collide_split_kernel(const __grid_constant__ DevParams<Real> p, Store* __restric
           const RowSide<false> sd(side, N, own, cy, cz);
           if constexpr (Last::value > 0) species(First{}, Last{}, A);
           float f[3], g[3];
-          row_fg(p, M, A, B, hq, sd.k, sd.x, cy, cz, f, g);
+          row_fg<false>(p, M, A, B, hq, sd.k, sd.x, cy, cz, f, g, nullptr, nullptr);
           f[2] = __shfl_up_sync(0xffffffffu, f[2], 1);
           g[2] = __shfl_up_sync(0xffffffffu, g[2], 1);
           f[0] = __shfl_down_sync(0xffffffffu, f[0], 1);

@@ -134,16 +134,17 @@ __device__ __forceinline__ void incoming_terms(const DevParams<Real>& p, const R
 }
 
 // 16-bit storage, for the readers of the state: every population arriving at
-// node n, a (c_y, c_z) row at a time, as f(i, cx, cy, cz, slot, node, sh) with
-// the AA place it is stored in and sh what it lacks (shifts of every lattice,
-// with the deferred terms of f and g).  As in the collide, a row's terms are
+// node n, a (c_y, c_z) row at a time, as f(i, cx, cy, cz, slot, node, sh, cf, cg)
+// with the AA place it is stored in and what it lacks: the shifts sh of every
+// lattice and the deferred terms of f and g, added to sh or (SEP) apart in cf
+// and cg.  As in the collide, a row's terms are
 // formed once at the lane's x and exchanged between lanes; a lane whose sender
 // is in no lane of the warp forms it itself.  All lanes of a warp call it;
 // those past the grid with active = false and the last node.  Measured (GB300):
 // observables of the 192^3 eight-species BF16 state 4.4 against 9.3 ms with
 // every population's terms formed from its own gathered record, restart copies
 // of 96^3 FP16 0.77 against 0.92 ms, two-species 256^3 BF16 4.2 ms either way.
-template <int M, class Store, class F>
+template <int M, class Store, bool SEP, class F>
 __device__ __forceinline__ void row_populations(const DevParams<float>& p, const float* __restrict__ side, int parity,
                                                 const Nbr& nb, long long n, bool active, F&& f) {
   constexpr int NP = (M + 1) / 2;
@@ -156,7 +157,7 @@ __device__ __forceinline__ void row_populations(const DevParams<float>& p, const
     const int cy = row % 3 - 1, cz = row / 3 - 1;
     const unsigned rb = (cy == 0 ? nb.ys[1] : (cy > 0 ? nb.ys[0] : nb.ys[2])) +
                         (cz == 0 ? nb.zs[1] : (cz > 0 ? nb.zs[0] : nb.zs[2]));
-    RowTerms<M> t;
+    RowTerms<M, SEP> t;
     row_terms<M>(p, RowLoad<M, true>(p, side, rin, (long long)(rb + nb.xs[1]), cy, cz), cy, cz, t);
 #pragma unroll
     for (int q = 0; q < NP; ++q) {
@@ -171,18 +172,27 @@ __device__ __forceinline__ void row_populations(const DevParams<float>& p, const
     t.g[2] = __shfl_up_sync(0xffffffffu, t.g[2], 1);
     t.f[0] = __shfl_down_sync(0xffffffffu, t.f[0], 1);
     t.g[0] = __shfl_down_sync(0xffffffffu, t.g[0], 1);
+    if constexpr (SEP) {
+      t.cf[2] = __shfl_up_sync(0xffffffffu, t.cf[2], 1);
+      t.cg[2] = __shfl_up_sync(0xffffffffu, t.cg[2], 1);
+      t.cf[0] = __shfl_down_sync(0xffffffffu, t.cf[0], 1);
+      t.cg[0] = __shfl_down_sync(0xffffffffu, t.cg[0], 1);
+    }
     // the lane's first need, then (rows of one node) a second
     for (int k = 0; k < 2; ++k) {
       if (k == 0 ? !(needL || needR) : !(needL && needR)) continue;
       const int cx = k == 0 && needL ? 1 : -1;
       const bool refl = arrives_from_wall_c(nb, cx);
       float2 sp[NP];
-      float fv, gv;
-      edge_terms<M>(p, RowLoad<M, true>(p, side, rin, refl ? n : (long long)(rb + (cx > 0 ? nb.xs[0] : nb.xs[2])), cy, cz), refl,
-                    cx, cy, cz, sp, fv, gv);
+      float fv, gv, cfv, cgv;
+      edge_terms<M, true, SEP>(p, RowLoad<M, true>(p, side, rin, refl ? n : (long long)(rb + (cx > 0 ? nb.xs[0] : nb.xs[2])), cy, cz), refl,
+                    cx, cy, cz, sp, fv, gv, &cfv, &cgv);
 #pragma unroll
       for (int q = 0; q < NP; ++q) { if (cx > 0) t.sp[q][2] = sp[q]; else t.sp[q][0] = sp[q]; }
       if (cx > 0) { t.f[2] = fv; t.g[2] = gv; } else { t.f[0] = fv; t.g[0] = gv; }
+      if constexpr (SEP) {
+        if (cx > 0) { t.cf[2] = cfv; t.cg[2] = cgv; } else { t.cf[0] = cfv; t.cg[0] = cgv; }
+      }
     }
 #pragma unroll
     for (int x = 0; x < 3; ++x) {
@@ -193,7 +203,8 @@ __device__ __forceinline__ void row_populations(const DevParams<float>& p, const
       for (int a = 0; a < M; ++a) sh[a] = a % 2 ? t.sp[a / 2][x].y : t.sp[a / 2][x].x;
       sh[M] = t.f[x];
       sh[M + 1] = t.g[x];
-      f(i, x - 1, cy, cz, own ? i : Q - 1 - i, own ? n : (long long)(rb + nb.xs[2 - x]), sh);
+      f(i, x - 1, cy, cz, own ? i : Q - 1 - i, own ? n : (long long)(rb + nb.xs[2 - x]), sh,
+        SEP ? t.cf[SEP ? x : 0] : 0.0f, SEP ? t.cg[SEP ? x : 0] : 0.0f);
     }
   }
 }
@@ -211,8 +222,9 @@ __device__ __forceinline__ void load_state_moments(const DevParams<Real>& p, con
   for (int a = 0; a < M; ++a) { rdev[a] = Real(0); ja[a][0] = ja[a][1] = ja[a][2] = Real(0); }
   rho_dev = Real(0); j[0] = j[1] = j[2] = Real(0); rhoE_dev = Real(0);
   if constexpr (kEqCodec<Store, Real>) {
-    row_populations<M, Store>(p, side, parity, nb, n, active,
-                              [&](int, int cx, int cy, int cz, int slot, long long node, const float (&sh)[M + 2]) {
+    row_populations<M, Store, false>(p, side, parity, nb, n, active,
+                                     [&](int, int cx, int cy, int cz, int slot, long long node, const float (&sh)[M + 2],
+                                         float, float) {
       const Store* q = pops + ((long long)slot * N + node);
       const float fx = (float)cx, fy = (float)cy, fz = (float)cz;
 #pragma unroll
