@@ -40,7 +40,9 @@ grad_GK_batch_kernel(const BatchGeom* __restrict__ geom, void* const* __restrict
   for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
     const int2 tl = tiles[t];
     const BatchGeom g = geom[tl.x];
-    grad_GK_node<Real>(g, static_cast<Real*>(side[tl.x]), (long long)tl.y + threadIdx.x);
+    Real* const s = static_cast<Real*>(side[tl.x]);
+    if (g.nx % ROWV == 0) grad_GK_node<Real, true>(g, s, (long long)tl.y + threadIdx.x);
+    else grad_GK_node<Real, false>(g, s, (long long)tl.y + threadIdx.x);
   }
 }
 
@@ -51,7 +53,9 @@ grad_X_batch_kernel(const BatchGeom* __restrict__ geom, void* const* __restrict_
   for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
     const int2 tl = tiles[t];
     const BatchGeom g = geom[tl.x];
-    grad_X_node<Real>(g, static_cast<Real*>(side[tl.x]), (long long)tl.y + threadIdx.x);
+    Real* const s = static_cast<Real*>(side[tl.x]);
+    if (g.nx % ROWV == 0) grad_X_node<Real, true>(g, s, (long long)tl.y + threadIdx.x);
+    else grad_X_node<Real, false>(g, s, (long long)tl.y + threadIdx.x);
   }
 }
 

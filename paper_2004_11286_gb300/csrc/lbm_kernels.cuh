@@ -386,12 +386,12 @@ struct Launch {
     const bool few = c.N <= kFieldStencilNodes<Real>;
     const bool rows = P(c).nx % ROWV == 0 && !P(c).tvar;
     const dim3 fg(grid_for(c.N, BLOCK_FIELD), 4), fx(fg.x, 3);
-    if (few) launch_next(grad_GK_field_kernel<Real>, fg, BLOCK_FIELD, 0, c.stream, P(c), side);
+    if (few) launch_next(rows ? grad_GK_field_kernel<Real, true> : grad_GK_field_kernel<Real, false>, fg, BLOCK_FIELD, 0, c.stream, P(c), side);
     else if (rows) launch_next(grad_GK_row_kernel<Real>, dim3(grid_for(c.N / ROWV, BLOCK_LIGHT)), BLOCK_LIGHT, 0, c.stream, P(c), side);
     else launch_next(grad_GK_kernel<Real>, dim3(grid_for(c.N, BLOCK_LIGHT)), BLOCK_LIGHT, 0, c.stream, P(c), side);
     if (frame) launch_next(frame_side_kernel<Real>, dim3(fgrid), BLOCK_FRAME, 0, c.stream, P(c), side, 1);
     if (c.ev) cudaEventRecord(c.ev[2], c.stream);
-    if (few) launch_next(grad_X_field_kernel<Real>, fx, BLOCK_FIELD, 0, c.stream, P(c), side);
+    if (few) launch_next(rows ? grad_X_field_kernel<Real, true> : grad_X_field_kernel<Real, false>, fx, BLOCK_FIELD, 0, c.stream, P(c), side);
     else if (rows) launch_next(grad_X_row_kernel<Real>, dim3(grid_for(c.N / ROWV, BLOCK_LIGHT)), BLOCK_LIGHT, 0, c.stream, P(c), side);
     else launch_next(grad_X_kernel<Real>, dim3(grid_for(c.N, BLOCK_LIGHT)), BLOCK_LIGHT, 0, c.stream, P(c), side);
     if (frame) launch_next(frame_side_kernel<Real>, dim3(fgrid), BLOCK_FRAME, 0, c.stream, P(c), side, 2);

@@ -270,83 +270,123 @@ __device__ __forceinline__ void load_state_moments(const DevParams<Real>& p, con
 // With temperature-dependent heats (tvar) the enthalpy field differentiated
 // is H-like: Phi_1 + T_n Phi_2 + T_n^2 Phi_3 of the neighbours with this
 // node's T_n, so that K = s sum_k T^(k-1) grad Phi_k = (s / T) sum_a H_a grad Y_a.
-template <class Real, class G>
-__device__ __forceinline__ void grad_GK_node(const G& p, Real* __restrict__ side, long long n, bool tvar = false) {
-  if (n >= p.N) return;
-  const long long N = p.N;
-  const Nbr nb = make_nbr(p, n);
-  Real d[3] = {Real(0), Real(0), Real(0)}, dc[3] = {Real(0), Real(0), Real(0)};
-  const Real Tn = tvar ? side[SP_T * N + n] : Real(0);
-#pragma unroll
-  for (int i = 0; i < Q; ++i) {
-    const int cx = cx_of(i), cy = cy_of(i), cz = cz_of(i);
-    if (i == 13) continue;
-    const long long nn = nb.idx(cx, cy, cz);
-    const Real w = iso_w<Real>(i);
-    Real cp = side[SP_CP * N + nn];
-    if (tvar) cp += Tn * (side[SP_HC2 * N + nn] + Tn * side[SP_HC3 * N + nn]);
-    // beyond a wall the mirror image of Phi_x is odd, the other fields even
-    const bool mirror = (cx < 0 && (nb.wall & 1u)) || (cx > 0 && (nb.wall & 2u));
-    if (cx) {
-      const Real phx = side[(SP_PHI + 0) * N + nn];
-      d[0] += (cx * w) * (mirror ? -phx : phx);
-      dc[0] += (cx * w) * cp;
-    }
-    if (cy) { d[1] += (cy * w) * side[(SP_PHI + 1) * N + nn]; dc[1] += (cy * w) * cp; }
-    if (cz) { d[2] += (cz * w) * side[(SP_PHI + 2) * N + nn]; dc[2] += (cz * w) * cp; }
-  }
-  const Real co = Real(3) * side[SP_COM * N + n], sv = Real(3) * side[SP_S * N + n];
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    side[(SP_G + c) * N + n] = co * d[c];
-    side[(SP_K + c) * N + n] = sv * dc[c];
-  }
-  side[SP_THR * N + n] = side[SP_TH * N + n];
-}
-
-// Stencil pass 2: X_alpha = -d_alpha G_alpha (Eq. Xalpha).
-template <class Real, class G>
-__device__ __forceinline__ void grad_X_node(const G& p, Real* __restrict__ side, long long n) {
-  if (n >= p.N) return;
-  const long long N = p.N;
-  const Nbr nb = make_nbr(p, n);
-  Real d[3] = {Real(0), Real(0), Real(0)};
-#pragma unroll
-  for (int i = 0; i < Q; ++i) {
-    const int cx = cx_of(i), cy = cy_of(i), cz = cz_of(i);
-    if (i == 13) continue;
-    const long long nn = nb.idx(cx, cy, cz);
-    const Real w = iso_w<Real>(i);
-    if (cx) d[0] += (cx * w) * side[(SP_G + 0) * N + nn];
-    if (cy) d[1] += (cy * w) * side[(SP_G + 1) * N + nn];
-    if (cz) d[2] += (cz * w) * side[(SP_G + 2) * N + nn];
-  }
-#pragma unroll
-  for (int c = 0; c < 3; ++c) side[(SP_X + c) * N + n] = Real(-3) * d[c];
-}
-
-// ---------------------------------------------------------------------------
-// Row-blocked stencil passes (grids with nx a multiple of ROWV): one thread
-// computes ROWV consecutive nodes of a row.  The D3Q27 weights factor per
-// axis, w_i = w(c_ix) w(c_iy) w(c_iz) with w(0) = 2/3, w(+-1) = 1/6, so the
-// isotropic gradient separates over the nine neighbour rows (c_y, c_z):
-//   d_x phi = (1/72) sum_{cy,cz} W(cy) W(cz) [phi(x+1) - phi(x-1)]
-//   d_y phi = (1/72) sum_{cz} W(cz) [s(+1, cz) - s(-1, cz)]
-//   d_z phi = (1/72) sum_{cy} W(cy) [s(cy, +1) - s(cy, -1)]
-// with W(0) = 4, W(+-1) = 1 and s = phi(x-1) + 4 phi(x) + phi(x+1) on the
-// row.  Each row is read once as ROWV + 2 values (x0-1 .. x0+ROWV) shared by
-// the thread's nodes: the middle ones as 16-byte vector loads, the two ends
-// as scalar loads or (SHFL) from the neighbouring lanes, which hold them as
-// their own middle values, except at warp and row edges.  Every lane of a
-// warp takes part in the shuffles; lanes past the grid compute on the last
-// nodes and store nothing.
-// ---------------------------------------------------------------------------
+// The passes exist as four nodes of a row per thread, a node per thread, and a
+// thread per node and field.  Which of them a grid takes depends on its number
+// of nodes; the sums a node gets do not.  They run over the nine neighbour rows
+// (c_y, c_z), c_z outermost, and add a row's three values in one of two forms:
+//   ROWS (rows of a multiple of ROWV nodes, constant heats): the D3Q27 weights
+//     factor per axis, w_i = w(c_ix) w(c_iy) w(c_iz) with w(0) = 2/3, w(+-1) = 1/6,
+//     so the isotropic gradient separates,
+//       d_x phi = (1/72) sum_{cy,cz} W(cy) W(cz) [phi(x+1) - phi(x-1)]
+//       d_y phi = (1/72) sum_{cz} W(cz) [s(+1, cz) - s(-1, cz)]
+//       d_z phi = (1/72) sum_{cy} W(cy) [s(cy, +1) - s(cy, -1)]
+//     with W(0) = 4, W(+-1) = 1 and s = phi(x-1) + 4 phi(x) + phi(x+1) on the row
+//     (products with powers of two: exact, so the sums round the same whether
+//     or not the compiler contracts them; with explicit fused operations the
+//     four-node first pass took 140 registers in place of 64 and, at 256^3, 363
+//     us in place of 212);
+//   else velocity by velocity, grad = 3 sum_i w_i c_i phi(x + c_i), by fused
+//     operations.
+// Slabs of a grid and the batched domains thus agree with the undivided grid
+// and the single domain bit for bit, whatever passes those take.
 #ifndef LBM_STENCIL_ROW
 #define LBM_STENCIL_ROW 4
 #endif
 constexpr int ROWV = LBM_STENCIL_ROW;
 static_assert(ROWV == 4 || ROWV == 8, "row blocking of 4 or 8 nodes");
 
+// Adds row (cy, cz), its values lo, mid, hi at x-1, x, x+1, to the sum d of the A-derivative.
+template <class Real, int A, bool ROWS>
+__device__ __forceinline__ Real row_term(Real lo, Real mid, Real hi, int cy, int cz, Real d) {
+  if constexpr (ROWS) {
+    const Real Wy = cy ? Real(1) : Real(4), Wz = cz ? Real(1) : Real(4);
+    const Real W = A == 0 ? Wy * Wz : (A == 1 ? cy * Wz : cz * Wy);
+    const Real s = A == 0 ? hi - lo : lo + Real(4) * mid + hi;
+    return d + W * s;
+  } else {
+    const int i = 3 * (cy + 1) + 9 * (cz + 1);
+    const Real w1 = iso_w<Real>(i), w0 = iso_w<Real>(i + 1), c = A == 0 ? Real(1) : (A == 1 ? Real(cy) : Real(cz));
+    if constexpr (A == 0) return fma(w1, hi, fma(-w1, lo, d));
+    return fma(c * w1, hi, fma(c * w0, mid, fma(c * w1, lo, d)));
+  }
+}
+// The factors of the sums: G = c_omega grad Phi, K = s grad C_p; X = -div.
+template <class Real, bool ROWS>
+__device__ __forceinline__ Real scaled_gradient(Real c, Real d) {
+  return ROWS ? c * (d * (Real(1) / Real(72))) : Real(3) * c * d;
+}
+template <class Real, bool ROWS>
+__device__ __forceinline__ Real minus_gradient(Real d) {
+  return d * (ROWS ? Real(-1) / Real(72) : Real(-3));
+}
+
+template <class Real, bool ROWS, class G>
+__device__ __forceinline__ void grad_GK_node(const G& p, Real* __restrict__ side, long long n, bool tvar = false) {
+  if (n >= p.N) return;
+  const long long N = p.N;
+  const Nbr nb = make_nbr(p, n);
+  Real d[3] = {Real(0), Real(0), Real(0)}, dc[3] = {Real(0), Real(0), Real(0)};
+  const Real Tn = tvar ? side[SP_T * N + n] : Real(0);
+  auto phi = [&](int c, long long nn) { return side[(SP_PHI + c) * N + nn]; };
+  auto cp = [&](long long nn) {
+    Real v = side[SP_CP * N + nn];
+    if (tvar) v = fma1(Tn, fma1(Tn, side[SP_HC3 * N + nn], side[SP_HC2 * N + nn]), v);
+    return v;
+  };
+#pragma unroll
+  for (int cz = -1; cz <= 1; ++cz)
+#pragma unroll
+    for (int cy = -1; cy <= 1; ++cy) {
+      const long long lo = nb.idx(-1, cy, cz), mid = nb.idx(0, cy, cz), hi = nb.idx(1, cy, cz);
+      // beyond a wall the mirror image of Phi_x is odd, the other fields even
+      const Real plo = phi(0, lo), phi_hi = phi(0, hi);
+      d[0] = row_term<Real, 0, ROWS>((nb.wall & 1u) ? -plo : plo, Real(0), (nb.wall & 2u) ? -phi_hi : phi_hi, cy, cz, d[0]);
+      if (cy) d[1] = row_term<Real, 1, ROWS>(phi(1, lo), phi(1, mid), phi(1, hi), cy, cz, d[1]);
+      if (cz) d[2] = row_term<Real, 2, ROWS>(phi(2, lo), phi(2, mid), phi(2, hi), cy, cz, d[2]);
+      const Real clo = cp(lo), chi = cp(hi), cm = cy || cz ? cp(mid) : Real(0);
+      dc[0] = row_term<Real, 0, ROWS>(clo, cm, chi, cy, cz, dc[0]);
+      if (cy) dc[1] = row_term<Real, 1, ROWS>(clo, cm, chi, cy, cz, dc[1]);
+      if (cz) dc[2] = row_term<Real, 2, ROWS>(clo, cm, chi, cy, cz, dc[2]);
+    }
+  const Real co = side[SP_COM * N + n], sv = side[SP_S * N + n];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    side[(SP_G + c) * N + n] = scaled_gradient<Real, ROWS>(co, d[c]);
+    side[(SP_K + c) * N + n] = scaled_gradient<Real, ROWS>(sv, dc[c]);
+  }
+  side[SP_THR * N + n] = side[SP_TH * N + n];
+}
+
+// Stencil pass 2: X_alpha = -d_alpha G_alpha (Eq. Xalpha).
+template <class Real, bool ROWS, class G>
+__device__ __forceinline__ void grad_X_node(const G& p, Real* __restrict__ side, long long n) {
+  if (n >= p.N) return;
+  const long long N = p.N;
+  const Nbr nb = make_nbr(p, n);
+  Real d[3] = {Real(0), Real(0), Real(0)};
+  auto g = [&](int c, long long nn) { return side[(SP_G + c) * N + nn]; };
+#pragma unroll
+  for (int cz = -1; cz <= 1; ++cz)
+#pragma unroll
+    for (int cy = -1; cy <= 1; ++cy) {
+      const long long lo = nb.idx(-1, cy, cz), mid = nb.idx(0, cy, cz), hi = nb.idx(1, cy, cz);
+      d[0] = row_term<Real, 0, ROWS>(g(0, lo), Real(0), g(0, hi), cy, cz, d[0]);
+      if (cy) d[1] = row_term<Real, 1, ROWS>(g(1, lo), g(1, mid), g(1, hi), cy, cz, d[1]);
+      if (cz) d[2] = row_term<Real, 2, ROWS>(g(2, lo), g(2, mid), g(2, hi), cy, cz, d[2]);
+    }
+#pragma unroll
+  for (int c = 0; c < 3; ++c) side[(SP_X + c) * N + n] = minus_gradient<Real, ROWS>(d[c]);
+}
+
+// ---------------------------------------------------------------------------
+// Row-blocked stencil passes (grids with nx a multiple of ROWV): one thread
+// computes ROWV consecutive nodes of a row.  Each row is read once as ROWV + 2
+// values (x0-1 .. x0+ROWV) shared by the thread's nodes: the middle ones as
+// 16-byte vector loads, the two ends as scalar loads or (SHFL) from the
+// neighbouring lanes, which hold them as their own middle values, except at
+// warp and row edges.  Every lane of a warp takes part in the shuffles; lanes
+// past the grid compute on the last nodes and store nothing.
+// ---------------------------------------------------------------------------
 // Row coordinates of the nodes n0 .. n0+ROWV-1 (x0 = n0 mod nx, a multiple of ROWV).
 struct RowV {
   unsigned x0, xm, xp;       // first x, its left neighbour, the right neighbour of the last node (periodic)
@@ -408,16 +448,8 @@ __device__ __forceinline__ void load_row(const Real* __restrict__ f, const RowV&
 // Adds row (cy, cz) of a field to the a-derivative accumulators d[ROWV] (a = 0, 1, 2).
 template <class Real, int A>
 __device__ __forceinline__ void row_derivative(const Real (&v)[ROWV + 2], int cy, int cz, Real (&d)[ROWV]) {
-  const Real Wy = cy ? Real(1) : Real(4), Wz = cz ? Real(1) : Real(4);
 #pragma unroll
-  for (int j = 0; j < ROWV; ++j) {
-    if constexpr (A == 0) d[j] += (Wy * Wz) * (v[j + 2] - v[j]);
-    else {
-      const Real s = v[j] + Real(4) * v[j + 1] + v[j + 2];
-      if constexpr (A == 1) d[j] += (cy * Wz) * s;
-      else d[j] += (cz * Wy) * s;
-    }
-  }
+  for (int j = 0; j < ROWV; ++j) d[j] = row_term<Real, A, true>(v[j], v[j + 1], v[j + 2], cy, cz, d[j]);
 }
 
 // Pass 1 on ROWV nodes: G_a = c_omega d_a Phi_a, K = s grad C_p, theta copied.
@@ -448,7 +480,6 @@ __device__ __forceinline__ void grad_GK_row(const DevParams<Real>& p, Real* __re
     }
   if (!store) return;
   const unsigned own = r.row(0, 0) + r.x0;
-  const Real k72 = Real(1) / Real(72);
 #pragma unroll
   for (int q = 0; q < ROWV; q += 4) {
     Real co[4], sv[4], th[4];
@@ -459,7 +490,10 @@ __device__ __forceinline__ void grad_GK_row(const DevParams<Real>& p, Real* __re
     for (int a = 0; a < 3; ++a) {
       Real g[4], k[4];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) { g[j] = co[j] * (dp[a][q + j] * k72); k[j] = sv[j] * (dc[a][q + j] * k72); }
+      for (int j = 0; j < 4; ++j) {
+        g[j] = scaled_gradient<Real, true>(co[j], dp[a][q + j]);
+        k[j] = scaled_gradient<Real, true>(sv[j], dc[a][q + j]);
+      }
       store4<Real>(side + (SP_G + a) * N + own + q, g);
       store4<Real>(side + (SP_K + a) * N + own + q, k);
     }
@@ -491,87 +525,90 @@ __device__ __forceinline__ void grad_X_row(const DevParams<Real>& p, Real* __res
     }
   if (!store) return;
   const unsigned own = r.row(0, 0) + r.x0;
-  const Real k72 = Real(-1) / Real(72);
 #pragma unroll
   for (int a = 0; a < 3; ++a)
 #pragma unroll
     for (int q = 0; q < ROWV; q += 4) {
       Real x[4];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) x[j] = d[a][q + j] * k72;
+      for (int j = 0; j < 4; ++j) x[j] = minus_gradient<Real, true>(d[a][q + j]);
       store4<Real>(side + (SP_X + a) * N + own + q, x);
     }
 }
 
 // Small grids: a thread per node and field, so that few nodes still spread
-// over the SMs.  field 0..2: G_field; 3: K and the copy of theta.
-template <class Real>
-__device__ __forceinline__ void grad_GK_field(const DevParams<Real>& p, Real* __restrict__ side, long long n, int field) {
+// over the SMs.  F = 0..2: G_F; 3: K and the copy of theta.
+template <class Real, bool ROWS, int F>
+__device__ __forceinline__ void grad_GK_field(const DevParams<Real>& p, Real* __restrict__ side, long long n) {
   if (n >= p.N) return;
   const long long N = p.N;
   const Nbr nb = make_nbr(p, n);
-  if (field < 3) {
-    const Real* phi = side + (SP_PHI + field) * N;
-    Real d = Real(0);
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-      const int c = field == 0 ? cx_of(i) : (field == 1 ? cy_of(i) : cz_of(i));
-      if (c == 0) continue;
-      Real v = phi[nb.idx(cx_of(i), cy_of(i), cz_of(i))];
-      if (field == 0 && ((c < 0 && (nb.wall & 1u)) || (c > 0 && (nb.wall & 2u)))) v = -v;   // Phi_x is odd beyond a wall
-      d += (c * iso_w<Real>(i)) * v;
+  const Real Tn = F == 3 && p.tvar ? side[SP_T * N + n] : Real(0);
+  auto value = [&](int cx, int cy, int cz) {
+    const long long nn = nb.idx(cx, cy, cz);
+    if constexpr (F < 3) {
+      const Real v = side[(SP_PHI + F) * N + nn];
+      return F == 0 && ((cx < 0 && (nb.wall & 1u)) || (cx > 0 && (nb.wall & 2u))) ? -v : v;   // Phi_x is odd beyond a wall
+    } else {
+      Real v = side[SP_CP * N + nn];
+      if (p.tvar) v = fma1(Tn, fma1(Tn, side[SP_HC3 * N + nn], side[SP_HC2 * N + nn]), v);
+      return v;
     }
-    side[(SP_G + field) * N + n] = Real(3) * side[SP_COM * N + n] * d;
-    return;
+  };
+  Real d[3] = {Real(0), Real(0), Real(0)};
+#pragma unroll
+  for (int cz = -1; cz <= 1; ++cz)
+#pragma unroll
+    for (int cy = -1; cy <= 1; ++cy) {
+      if ((F == 1 && cy == 0) || (F == 2 && cz == 0)) continue;
+      const Real lo = value(-1, cy, cz), hi = value(1, cy, cz);
+      const Real mid = F == 0 || (cy == 0 && cz == 0) ? Real(0) : value(0, cy, cz);
+      if (F == 0 || F == 3) d[0] = row_term<Real, 0, ROWS>(lo, mid, hi, cy, cz, d[0]);
+      if (F == 1 || (F == 3 && cy)) d[1] = row_term<Real, 1, ROWS>(lo, mid, hi, cy, cz, d[1]);
+      if (F == 2 || (F == 3 && cz)) d[2] = row_term<Real, 2, ROWS>(lo, mid, hi, cy, cz, d[2]);
+    }
+  if constexpr (F < 3) {
+    side[(SP_G + F) * N + n] = scaled_gradient<Real, ROWS>(side[SP_COM * N + n], d[F]);
+  } else {
+    const Real sv = side[SP_S * N + n];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) side[(SP_K + c) * N + n] = scaled_gradient<Real, ROWS>(sv, d[c]);
+    side[SP_THR * N + n] = side[SP_TH * N + n];
   }
-  const Real Tn = p.tvar ? side[SP_T * N + n] : Real(0);
-  Real dc[3] = {Real(0), Real(0), Real(0)};
-#pragma unroll
-  for (int i = 0; i < Q; ++i) {
-    if (i == 13) continue;
-    const long long nn = nb.idx(cx_of(i), cy_of(i), cz_of(i));
-    Real cp = side[SP_CP * N + nn];
-    if (p.tvar) cp += Tn * (side[SP_HC2 * N + nn] + Tn * side[SP_HC3 * N + nn]);
-#pragma unroll
-    for (int c = 0; c < 3; ++c)
-      if (c_of(i, c)) dc[c] += (c_of(i, c) * iso_w<Real>(i)) * cp;
-  }
-  const Real sv = Real(3) * side[SP_S * N + n];
-#pragma unroll
-  for (int c = 0; c < 3; ++c) side[(SP_K + c) * N + n] = sv * dc[c];
-  side[SP_THR * N + n] = side[SP_TH * N + n];
 }
-template <class Real>
-__device__ __forceinline__ void grad_X_field(const DevParams<Real>& p, Real* __restrict__ side, long long n, int field) {
+template <class Real, bool ROWS, int F>
+__device__ __forceinline__ void grad_X_field(const DevParams<Real>& p, Real* __restrict__ side, long long n) {
   if (n >= p.N) return;
   const long long N = p.N;
   const Nbr nb = make_nbr(p, n);
-  const Real* g = side + (SP_G + field) * N;
+  auto g = [&](int cx, int cy, int cz) { return side[(SP_G + F) * N + nb.idx(cx, cy, cz)]; };
   Real d = Real(0);
 #pragma unroll
-  for (int i = 0; i < Q; ++i) {
-    const int c = field == 0 ? cx_of(i) : (field == 1 ? cy_of(i) : cz_of(i));
-    if (c) d += (c * iso_w<Real>(i)) * g[nb.idx(cx_of(i), cy_of(i), cz_of(i))];
-  }
-  side[(SP_X + field) * N + n] = Real(-3) * d;
+  for (int cz = -1; cz <= 1; ++cz)
+#pragma unroll
+    for (int cy = -1; cy <= 1; ++cy) {
+      if ((F == 1 && cy == 0) || (F == 2 && cz == 0)) continue;
+      d = row_term<Real, F, ROWS>(g(-1, cy, cz), F == 0 ? Real(0) : g(0, cy, cz), g(1, cy, cz), cy, cz, d);
+    }
+  side[(SP_X + F) * N + n] = minus_gradient<Real, ROWS>(d);
 }
 constexpr int BLOCK_FIELD = 32;
-template <class Real>
+template <class Real, bool ROWS>
 __global__ void __launch_bounds__(BLOCK_FIELD)
 grad_GK_field_kernel(const __grid_constant__ DevParams<Real> p, Real* __restrict__ side) {
   wait_previous();
-  if (blockIdx.y == 0) grad_GK_field<Real>(p, side, gtid(), 0);
-  else if (blockIdx.y == 1) grad_GK_field<Real>(p, side, gtid(), 1);
-  else if (blockIdx.y == 2) grad_GK_field<Real>(p, side, gtid(), 2);
-  else grad_GK_field<Real>(p, side, gtid(), 3);
+  if (blockIdx.y == 0) grad_GK_field<Real, ROWS, 0>(p, side, gtid());
+  else if (blockIdx.y == 1) grad_GK_field<Real, ROWS, 1>(p, side, gtid());
+  else if (blockIdx.y == 2) grad_GK_field<Real, ROWS, 2>(p, side, gtid());
+  else grad_GK_field<Real, ROWS, 3>(p, side, gtid());
 }
-template <class Real>
+template <class Real, bool ROWS>
 __global__ void __launch_bounds__(BLOCK_FIELD)
 grad_X_field_kernel(const __grid_constant__ DevParams<Real> p, Real* __restrict__ side) {
   wait_previous();
-  if (blockIdx.y == 0) grad_X_field<Real>(p, side, gtid(), 0);
-  else if (blockIdx.y == 1) grad_X_field<Real>(p, side, gtid(), 1);
-  else grad_X_field<Real>(p, side, gtid(), 2);
+  if (blockIdx.y == 0) grad_X_field<Real, ROWS, 0>(p, side, gtid());
+  else if (blockIdx.y == 1) grad_X_field<Real, ROWS, 1>(p, side, gtid());
+  else grad_X_field<Real, ROWS, 2>(p, side, gtid());
 }
 
 // LBM_GK_MINB > 0 sets a minimum of resident blocks per SM (FP32); by
@@ -605,13 +642,13 @@ template <class Real>
 __global__ void __launch_bounds__(BLOCK_LIGHT)
 grad_GK_kernel(const __grid_constant__ DevParams<Real> p, Real* __restrict__ side) {
   wait_previous();
-  grad_GK_node<Real>(p, side, gtid(), p.tvar != 0);
+  grad_GK_node<Real, false>(p, side, gtid(), p.tvar != 0);
 }
 template <class Real>
 __global__ void __launch_bounds__(BLOCK_LIGHT)
 grad_X_kernel(const __grid_constant__ DevParams<Real> p, Real* __restrict__ side) {
   wait_previous();
-  grad_X_node<Real>(p, side, gtid());
+  grad_X_node<Real, false>(p, side, gtid());
 }
 
 }  // namespace lbm
