@@ -235,7 +235,8 @@ LBM_API lbm_status lbm_mix_set_reference(lbm_mix_t h, const double* Y, double T,
  * with 16-bit storage, both equilibrium-record buffers.  One step reads
  * across at most three planes (the collision's neighbours, then the two
  * stencil passes of the non-local terms of Eq. Xalpha), so with ghost >= 3
- * the interior evolves exactly as the same planes of the undivided grid.
+ * and lbm_mix_set_grid_nodes the interior evolves exactly as the same planes
+ * of the undivided grid.
  *   lbm_mix_halo_bytes:  bytes of one face's buffer;
  *   lbm_mix_halo_pack:   copies the `ghost` interior planes next to face
  *                        0 (-z: planes ghost..2 ghost-1) or 1 (+z: planes
@@ -246,7 +247,15 @@ LBM_API lbm_status lbm_mix_set_reference(lbm_mix_t h, const double* Y, double T,
  * k-1's face 1 (slab indices periodic).  The buffer is caller-owned device
  * memory, on this device or reachable from it (another GPU's buffer through
  * peer access, or a receive buffer of a collective); ordered on the handle's
- * stream.  LBM_ERR_ARG for a bad face, ghost or grid. */
+ * stream.  LBM_ERR_ARG for a bad face, ghost or grid.
+ *   lbm_mix_set_grid_nodes: the nodes of the whole (undivided) grid, the same
+ *                        on every slab.  The step chooses between collide
+ *                        kernels by grid size, and these differ in rounding:
+ *                        a slab that knows the whole grid takes the kernel the
+ *                        undivided grid takes.  0 (the default): the handle's
+ *                        own nodes.  At any time; LBM_ERR_ARG if negative,
+ *                        LBM_ERR_STATE for a domain of a batch. */
+LBM_API lbm_status lbm_mix_set_grid_nodes(lbm_mix_t h, long long nodes);
 LBM_API lbm_status lbm_mix_halo_bytes(lbm_mix_t h, int ghost, size_t* bytes);
 LBM_API lbm_status lbm_mix_halo_pack(lbm_mix_t h, int face, int ghost, void* buf);
 LBM_API lbm_status lbm_mix_halo_unpack(lbm_mix_t h, int face, int ghost, const void* buf);

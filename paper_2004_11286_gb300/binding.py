@@ -62,6 +62,7 @@ SIGNATURES = {
     "lbm_mix_halo_bytes": (ct.c_int, [ct.c_void_p, ct.c_int, ct.POINTER(ct.c_size_t)]),
     "lbm_mix_halo_pack": (ct.c_int, [ct.c_void_p, ct.c_int, ct.c_int, ct.c_void_p]),
     "lbm_mix_halo_unpack": (ct.c_int, [ct.c_void_p, ct.c_int, ct.c_int, ct.c_void_p]),
+    "lbm_mix_set_grid_nodes": (ct.c_int, [ct.c_void_p, ct.c_longlong]),
     "lbm_mix_step_count": (ct.c_longlong, [ct.c_void_p]),
     "lbm_mix_launch_count": (ct.c_longlong, [ct.c_void_p]),
     "lbm_mix_enable_kernel_timing": (ct.c_int, [ct.c_void_p, ct.c_int]),
@@ -306,6 +307,10 @@ class LbmMix:
         if y.size != self.M:
             raise ValueError("Y must have M entries")
         self._check(self.lib.lbm_mix_set_reference(self.h, y.ctypes.data_as(_DP), float(T), float(rho)))
+
+    def set_grid_nodes(self, nodes: int):
+        """The nodes of the whole grid this handle is a slab of (0: its own)."""
+        self._check(self.lib.lbm_mix_set_grid_nodes(self.h, int(nodes)))
 
     def halo_bytes(self, ghost: int) -> int:
         b = ct.c_size_t()

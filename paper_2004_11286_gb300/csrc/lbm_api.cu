@@ -182,6 +182,8 @@ void lbm_set_thread_error(const std::string& msg) { g_create_error = msg; }
 struct lbm_mix {
   int M = 0, prec = 0, device = 0;
   long long N = 0;
+  long long grid_nodes = 0;    // of the whole grid where this one is a slab of it (0: its own)
+  bool batched = false;        // a domain of a batch
   cudaStream_t stream = nullptr;
   const lbm::KernelSet* ks = nullptr;
   lbm::DevParams<double> p64{};
@@ -227,7 +229,7 @@ struct lbm_mix {
   }
   lbm::LaunchCtx ctx() {
     lbm::LaunchCtx c;
-    c.N = N; c.stream = stream; c.pops = pops; c.side = scratch; c.err = d_err;
+    c.N = N; c.grid_nodes = grid_nodes > 0 ? grid_nodes : N; c.stream = stream; c.pops = pops; c.side = scratch; c.err = d_err;
     c.partials = d_partials; c.p64 = &p64; c.p32 = &p32; c.base = d_base; c.ev = nullptr;
     c.closure = closure; c.mlp_img = d_img; c.mlp_stats = d_stats;
     c.jet = d_jet;
@@ -1052,6 +1054,14 @@ lbm_status lbm_mix_halo_unpack(lbm_mix_t h, int face, int ghost, const void* buf
   return halo_move(h, face, ghost, const_cast<void*>(buf), 1);
 }
 
+lbm_status lbm_mix_set_grid_nodes(lbm_mix_t h, long long nodes) {
+  if (!h) return LBM_ERR_ARG;
+  if (nodes < 0) return h->fail(LBM_ERR_ARG, "nodes must be >= 0");
+  if (h->batched) return h->fail(LBM_ERR_STATE, "a domain of a batch is its own grid");
+  h->grid_nodes = nodes;
+  return LBM_OK;
+}
+
 lbm_status lbm_mix_synchronize(lbm_mix_t h) {
   if (!h) return LBM_ERR_ARG;
   return h->check_flag();
@@ -1240,6 +1250,7 @@ lbm_status lbm_mix_batch_create(const lbm_mix_params* params, int ndomains, void
       g_create_error = "domain " + std::to_string(d) + ": " + g_create_error;
       return cleanup(st);
     }
+    h->batched = true;
     b->dom.push_back(h);
   }
   b->ks = b->dom[0]->ks;

@@ -10,6 +10,7 @@ template <class Real> struct DevParams;
 
 struct LaunchCtx {
   long long N;
+  long long grid_nodes;   // nodes of the whole grid, of which these N may be a slab: what the kernel choice goes by
   cudaStream_t stream;
   void* pops;
   void* side;

@@ -341,7 +341,7 @@ struct Launch {
     // loads, exact closure (the host refuses both with the network closure).
     if constexpr (CL == 0 && kSplit<M, Real, Store>) {
       const long long most = kSplitTilesPerSm<M, Real, Store> * 32LL * sm_count();
-      if (!P(c).tvar && (kSplitTilesPerSm<M, Real, Store> == 0 || c.N <= most)) {
+      if (!P(c).tvar && (kSplitTilesPerSm<M, Real, Store> == 0 || c.grid_nodes <= most)) {
         if (P(c).wall_x) split_launch<1>(c, parity, side);
         else if (P(c).frame) split_launch<EQ ? 0 : 2>(c, parity, side);
         else split_launch<0>(c, parity, side);

@@ -368,7 +368,9 @@ __device__ __forceinline__ void split_closure(const DevParams<Real>& p, Real* sm
 //     a 16-bit value.
 template <int M, class Real, class Store>
 constexpr bool kSplit = M >= 4 || (sizeof(Store) >= 4 && (M == 3 || (M == 2 && sizeof(Real) == 8)));
-// The largest number of tiles per SM taken (0: any).
+// The largest number of tiles per SM taken (0: any), of the whole grid where
+// the handle holds a slab of it (LaunchCtx::grid_nodes): the two collides differ
+// in rounding, and a slab agrees with the undivided grid bit for bit.
 template <int M, class Real, class Store>
 constexpr int kSplitTilesPerSm = M >= 4 ? 0 : (sizeof(Real) == 8 ? 1 : 3);
 

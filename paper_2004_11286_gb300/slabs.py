@@ -7,9 +7,10 @@ counts.  Each slab is a handle (``binding.LbmMix``) on its own planes plus
 shares one reference rest state (``LbmMix.set_reference``).  After every
 step each ghost region is refreshed from the neighbouring slab's boundary
 planes (``LbmMix.halo_pack`` / ``halo_unpack``: population slots, side fields,
-equilibrium records).  One step reads across at most three planes, so with
-ghost = 3 each slab's interior evolves exactly as the same planes of the
-undivided grid.
+equilibrium records).  Every handle is told the whole grid's size
+(``LbmMix.set_grid_nodes``), by which the step chooses its kernels.  One step
+reads across at most three planes, so with ghost = 3 each slab's interior
+evolves exactly as the same planes of the undivided grid.
 
 The exchange schedule is ``halo_exchange``: slab k sends its top interior
 planes (face 1) to slab k+1, whose bottom ghost region (face 0) receives
@@ -102,6 +103,7 @@ class SlabSet:
         for k, (z0, z1) in enumerate(self.bounds):
             dev = torch.device(devs[k % len(devs)])
             self.handles.append(make_handle((z1 - z0 + 2 * self.ghost, ny, nx), dev))
+            self.handles[-1].set_grid_nodes(nz * ny * nx)
         self.M = self.handles[0].M
         self.bufs = [[torch.empty(h.halo_bytes(self.ghost), dtype=torch.uint8, device=h.device) for _ in range(2)]
                      for h in self.handles]
@@ -213,6 +215,7 @@ class DistributedSlab:
         self.molar_mass = np.asarray(molar_mass, dtype=np.float64)
         self.R_U = float(R_U)
         self.h = make_handle((z1 - z0 + 2 * self.ghost, ny, nx), device)
+        self.h.set_grid_nodes(nz * ny * nx)
         nb = self.h.halo_bytes(self.ghost)
         self.out = [torch.empty(nb, dtype=torch.uint8, device=self.h.device) for _ in range(2)]
         self.inb = [torch.empty(nb, dtype=torch.uint8, device=self.h.device) for _ in range(2)]
