@@ -438,8 +438,9 @@ struct lbm_mix_batch {
   size_t param_bytes = 0;            // one parameter block
   lbm::BatchGeom* d_geom = nullptr;
   void** d_ptrs = nullptr;           // [nd] pops, then [nd] side
-  int2* d_tiles = nullptr;           // collide tiles, then stencil tiles for 128 and 256 threads
-  int ntiles_c = 0, ntiles_128 = 0, ntiles_256 = 0;
+  int2* d_tiles = nullptr;           // collide tiles (a thread per node, split), then stencil tiles for 128 and 256 threads
+  int tiles_collide = 0;             // collide_bs-node tiles of all domains, what grid_c is given in
+  int ntiles_c = 0, ntiles_s = 0, ntiles_128 = 0, ntiles_256 = 0;
   int grid_c = 0, grid_l = 0, block_l = 256;
   int sm_count = 0;
   unsigned* d_err = nullptr;
@@ -462,13 +463,14 @@ struct lbm_mix_batch {
     err = std::string(what) + ": " + cudaGetErrorString(e);
     return LBM_ERR_CUDA;
   }
-  const int2* tiles_l() const { return d_tiles + ntiles_c + (block_l == 128 ? 0 : ntiles_128); }
+  const int2* tiles_l() const { return d_tiles + ntiles_c + ntiles_s + (block_l == 128 ? 0 : ntiles_128); }
   int ntiles_l() const { return block_l == 128 ? ntiles_128 : ntiles_256; }
   lbm::BatchCtx ctx() const {
     lbm::BatchCtx c;
     c.stream = stream; c.params = d_params; c.geom = d_geom;
     c.pops = d_ptrs; c.side = d_ptrs + nd;
     c.tiles_c = d_tiles; c.ntiles_c = ntiles_c; c.grid_c = grid_c;
+    c.tiles_s = d_tiles + ntiles_c; c.ntiles_s = ntiles_s;
     c.tiles_l = tiles_l(); c.ntiles_l = ntiles_l(); c.grid_l = grid_l; c.block_l = block_l;
     c.err = d_err;
     return c;
@@ -1274,17 +1276,22 @@ lbm_status lbm_mix_batch_create(const lbm_mix_params* params, int ndomains, void
       return cleanup(bad(LBM_ERR_ARG, "binding domain buffers failed"));
     geom[d] = lbm::BatchGeom{h->N, h->p64.nx, h->p64.ny, h->p64.nz};
   }
-  // tiles: (domain, first node) for the collide block and for 128/256-thread stencil blocks
+  // tiles: (domain, first node) for the collide blocks, by the collide each
+  // domain's own step takes, and for 128/256-thread stencil blocks
   std::vector<int2> tiles;
-  auto add_tiles = [&](int bs) {
+  auto add_tiles = [&](int bs, int split) {                  // split < 0: every domain
     int cnt = 0;
-    for (int d = 0; d < ndomains; ++d)
+    for (int d = 0; d < ndomains; ++d) {
+      if (split >= 0 && (int)b->ks->split_route(b->dom[d]->ctx()) != split) continue;
       for (long long n0 = 0; n0 < b->dom[d]->N; n0 += bs) { tiles.push_back(make_int2(d, (int)n0)); ++cnt; }
+    }
     return cnt;
   };
-  b->ntiles_c = add_tiles(b->ks->collide_bs);
-  b->ntiles_128 = add_tiles(128);
-  b->ntiles_256 = add_tiles(256);
+  b->ntiles_c = add_tiles(b->ks->collide_bs, 0);
+  b->ntiles_s = add_tiles(32, 1);
+  b->ntiles_128 = add_tiles(128, -1);
+  b->ntiles_256 = add_tiles(256, -1);
+  for (const lbm_mix* h : b->dom) b->tiles_collide += (int)((h->N + b->ks->collide_bs - 1) / b->ks->collide_bs);
   b->param_bytes = b->prec == LBM_PREC_FP64 ? sizeof(lbm::DevParams<double>) : sizeof(lbm::DevParams<float>);
   cudaError_t e = cudaMalloc(&b->d_params, b->param_bytes * ndomains);
   if (e == cudaSuccess) e = cudaMalloc(&b->d_geom, sizeof(lbm::BatchGeom) * ndomains);
@@ -1302,7 +1309,7 @@ lbm_status lbm_mix_batch_create(const lbm_mix_params* params, int ndomains, void
   if (e != cudaSuccess) return cleanup(bad(LBM_ERR_CUDA, std::string("CUDA: ") + cudaGetErrorString(e)));
   b->uploaded.assign(ndomains, -1);
   // default launch shapes (the autotuner may replace them): one block per tile
-  b->grid_c = b->ntiles_c;
+  b->grid_c = b->tiles_collide;
   b->block_l = 256;
   b->grid_l = b->ntiles_256;
   *out = b;
@@ -1370,13 +1377,13 @@ lbm_status lbm_mix_batch_autotune(lbm_mix_batch_t b, int trial_steps, int* confi
   };
   const int sm = b->sm_count > 0 ? b->sm_count : 1;
   double best = 1e300;
-  int bmode = 0, bbr = b->nbranch, bc = b->ntiles_c, bl = 256, bg = b->ntiles_256;
+  int bmode = 0, bbr = b->nbranch, bc = b->tiles_collide, bl = 256, bg = b->ntiles_256;
   st = LBM_OK;
   // mode 0: persistent launches over all tiles
   b->mode = 0;
   b->block_l = 256; b->grid_l = b->ntiles_256;
-  for (int g : {b->ntiles_c, sm, 2 * sm, 3 * sm, 4 * sm}) {
-    if (g > b->ntiles_c || st != LBM_OK) continue;
+  for (int g : {b->tiles_collide, sm, 2 * sm, 3 * sm, 4 * sm}) {
+    if (g > b->tiles_collide || st != LBM_OK) continue;
     b->grid_c = g;
     b->drop_graph();
     double ms;
@@ -1428,7 +1435,7 @@ lbm_status lbm_mix_batch_set_config(lbm_mix_batch_t b, int grid_collide, int blo
   if (!b) return LBM_ERR_ARG;
   if (block_stencil != 128 && block_stencil != 256) return b->fail(LBM_ERR_ARG, "stencil blocks are 128 or 256 threads");
   const int ntl = block_stencil == 128 ? b->ntiles_128 : b->ntiles_256;
-  if (grid_collide < 1 || grid_collide > b->ntiles_c || grid_stencil < 1 || grid_stencil > ntl)
+  if (grid_collide < 1 || grid_collide > b->tiles_collide || grid_stencil < 1 || grid_stencil > ntl)
     return b->fail(LBM_ERR_ARG, "grid sizes must be in 1..number of tiles");
   b->grid_c = grid_collide; b->block_l = block_stencil; b->grid_l = grid_stencil;
   b->use_graph = use_graph != 0;
@@ -1448,7 +1455,7 @@ lbm_status lbm_mix_batch_set_mode(lbm_mix_batch_t b, int mode, int branches) {
 lbm_status lbm_mix_batch_config(lbm_mix_batch_t b, int* config) {
   if (!b || !config) return LBM_ERR_ARG;
   config[0] = b->grid_c; config[1] = b->block_l; config[2] = b->grid_l; config[3] = b->use_graph ? 1 : 0;
-  config[4] = b->ntiles_c; config[5] = b->ntiles_128; config[6] = b->ntiles_256; config[7] = b->ks->collide_bs;
+  config[4] = b->tiles_collide; config[5] = b->ntiles_128; config[6] = b->ntiles_256; config[7] = b->ks->collide_bs;
   config[8] = b->mode; config[9] = b->nbranch;
   return LBM_OK;
 }

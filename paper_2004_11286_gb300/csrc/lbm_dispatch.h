@@ -38,8 +38,10 @@ struct BatchCtx {
   const BatchGeom* geom;    // [domains] (device)
   void* const* pops;        // per-domain population buffers (device array of device pointers)
   void* const* side;        // per-domain scratch buffers
-  const int2* tiles_c;      // collide tiles (domain, first node), collide_bs nodes each
-  int ntiles_c, grid_c;
+  const int2* tiles_c;      // collide tiles (domain, first node) of the domains with a thread per node, collide_bs nodes each
+  const int2* tiles_s;      // those of the domains with the split collide, 32 nodes each
+  int ntiles_c, ntiles_s;
+  int grid_c;               // collide blocks of collide_bs nodes asked for
   const int2* tiles_l;      // stencil tiles, block_l nodes each
   int ntiles_l, grid_l, block_l;
   unsigned* err;
@@ -55,6 +57,7 @@ struct KernelSet {
   cudaError_t (*samples)(const LaunchCtx&, int parity, float* feat, float* tgt);
   cudaError_t (*mlp_forward)(const LaunchCtx&, const float* feat, float* out, long long n);
   cudaError_t (*mlp_pack)(const LaunchCtx&, const float* w, unsigned char* img);
+  bool (*split_route)(const LaunchCtx&);     // whether the step takes the split collide (lbm_split.cuh)
   cudaError_t (*batch_prepare)();
   cudaError_t (*batch_step)(const BatchCtx&, int parity);
   // The complete equilibria of the two inlet states of the opposed-jets frame:

@@ -313,10 +313,11 @@ struct Launch {
     });
     return v > 0 ? v : 1;
   }
+  static constexpr size_t split_smem = Split<M>::REALS * sizeof(Real);
   template <int BND>
   static void split_launch(const LaunchCtx& c, int parity, Real* side) {
     using C = Split<M>;
-    constexpr size_t smem = C::REALS * sizeof(Real);
+    constexpr size_t smem = split_smem;
     static PerDevice blocks;
     const int found = blocks.get(current_device(), [] {      // blocks the device holds at once
       if (!allow_smem(collide_split_kernel<M, Real, Store, 0, BND>, smem) ||
@@ -333,6 +334,15 @@ struct Launch {
     launch_next(parity == 0 ? collide_split_kernel<M, Real, Store, 0, BND> : collide_split_kernel<M, Real, Store, 1, BND>,
                 dim3(grid), C::THREADS, smem, c.stream, P(c), (Store*)c.pops, side, c.err, ntiles, po);
   }
+  static constexpr bool kSplitAlways = kSplit<M, Real, Store> && kSplitTilesPerSm<M, Real, Store> == 0;   // constant heats, exact closure
+  static bool split_route(const LaunchCtx& c) {
+    if constexpr (kSplit<M, Real, Store>) {
+      if (c.closure || P(c).tvar) return false;
+      return kSplitAlways || c.grid_nodes <= kSplitTilesPerSm<M, Real, Store> * 32LL * sm_count();
+    } else {
+      return false;
+    }
+  }
   // Bulk row loads where the blocks are whole row segments and the stage
   // holds the stored type (FP64, FP32).
   template <int CL>
@@ -340,8 +350,7 @@ struct Launch {
     // Walls normal to x (bounce-back), the opposed-jets frame: register
     // loads, exact closure (the host refuses both with the network closure).
     if constexpr (CL == 0 && kSplit<M, Real, Store>) {
-      const long long most = kSplitTilesPerSm<M, Real, Store> * 32LL * sm_count();
-      if (!P(c).tvar && (kSplitTilesPerSm<M, Real, Store> == 0 || c.grid_nodes <= most)) {
+      if (split_route(c)) {
         if (P(c).wall_x) split_launch<1>(c, parity, side);
         else if (P(c).frame) split_launch<EQ ? 0 : 2>(c, parity, side);
         else split_launch<0>(c, parity, side);
@@ -350,7 +359,7 @@ struct Launch {
     }
     constexpr bool bulk = CL == 0 && LBM_COLLIDE_BULK && M >= LBM_COLLIDE_BULK_MIN_M && std::is_same<Real, Store>::value;
     const bool segments = bulk && P(c).nx % collide_block<M, Real, 0, Store>() == 0;
-    if constexpr (CL == 0 && kSplit<M, Real, Store> && kSplitTilesPerSm<M, Real, Store> == 0) {
+    if constexpr (CL == 0 && kSplitAlways) {
       // only temperature-dependent heats get here (FP64, FP32, periodic)
       if constexpr (!EQ) {
         if (segments) collide_launch<0, bulk>(c, parity, side);
@@ -399,21 +408,34 @@ struct Launch {
     return cudaGetLastError();
   }
   static cudaError_t batch_prepare() {
-    constexpr size_t smem = collide_smem<M, Real, 0, 0, Store>();
-    cudaFuncSetAttribute(collide_batch_kernel<M, Real, Store, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaFuncSetAttribute(collide_batch_kernel<M, Real, Store, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if constexpr (!kSplitAlways) {
+      constexpr size_t smem = collide_smem<M, Real, 0, 0, Store>();
+      allow_smem(collide_batch_kernel<M, Real, Store, 0>, smem);
+      allow_smem(collide_batch_kernel<M, Real, Store, 1>, smem);
+    }
+    if constexpr (kSplit<M, Real, Store>) {
+      allow_smem(collide_split_batch_kernel<M, Real, Store, 0>, split_smem);
+      allow_smem(collide_split_batch_kernel<M, Real, Store, 1>, split_smem);
+    }
     return cudaGetLastError();
   }
   static cudaError_t batch_step(const BatchCtx& b, int parity) {
     constexpr int BS = collide_block<M, Real, 0, Store>();
-    constexpr size_t smem = collide_smem<M, Real, 0, 0, Store>();
     const DevParams<Real>* prm = static_cast<const DevParams<Real>*>(b.params);
-    if (parity == 0)
-      collide_batch_kernel<M, Real, Store, 0><<<b.grid_c, BS, smem, b.stream>>>(prm, b.pops, b.side, b.tiles_c,
-                                                                                 b.ntiles_c, b.err);
-    else
-      collide_batch_kernel<M, Real, Store, 1><<<b.grid_c, BS, smem, b.stream>>>(prm, b.pops, b.side, b.tiles_c,
-                                                                                 b.ntiles_c, b.err);
+    if constexpr (!kSplitAlways) {
+      constexpr size_t smem = collide_smem<M, Real, 0, 0, Store>();
+      const int grid = b.grid_c < b.ntiles_c ? b.grid_c : b.ntiles_c;
+      if (grid > 0)
+        (parity == 0 ? collide_batch_kernel<M, Real, Store, 0> : collide_batch_kernel<M, Real, Store, 1>)
+            <<<grid, BS, smem, b.stream>>>(prm, b.pops, b.side, b.tiles_c, b.ntiles_c, b.err);
+    }
+    if constexpr (kSplit<M, Real, Store>) {
+      const long long want = (long long)b.grid_c * ((BS + 31) / 32);
+      const int grid = want < b.ntiles_s ? (int)want : b.ntiles_s;
+      if (grid > 0)
+        (parity == 0 ? collide_split_batch_kernel<M, Real, Store, 0> : collide_split_batch_kernel<M, Real, Store, 1>)
+            <<<grid, Split<M>::THREADS, split_smem, b.stream>>>(prm, b.pops, b.side, b.tiles_s, b.ntiles_s, b.err);
+    }
     grad_GK_batch_kernel<Real><<<b.grid_l, b.block_l, 0, b.stream>>>(b.geom, b.side, b.tiles_l, b.ntiles_l);
     grad_X_batch_kernel<Real><<<b.grid_l, b.block_l, 0, b.stream>>>(b.geom, b.side, b.tiles_l, b.ntiles_l);
     return cudaGetLastError();
@@ -478,7 +500,7 @@ struct Launch {
     k.init = &init; k.step = &step; k.moments = &moments; k.get_pops = &get_pops;
     k.set_pops = &set_pops; k.diag = &diag;
     k.samples = &samples; k.mlp_forward = &mlp_forward; k.mlp_pack = &mlp_pack;
-    k.batch_prepare = &batch_prepare; k.batch_step = &batch_step; k.jet_table = &jet_table;
+    k.split_route = &split_route; k.batch_prepare = &batch_prepare; k.batch_step = &batch_step; k.jet_table = &jet_table;
     k.launches_per_step = 3;
     k.setup_launches = EQ ? 2 : 1;
     k.collide_bs = collide_block<M, Real, 0, Store>();

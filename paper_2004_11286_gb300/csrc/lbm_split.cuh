@@ -386,538 +386,549 @@ constexpr int split_min_blocks() {
   return want < 1 ? 1 : (want < fit ? want : (fit < 1 ? 1 : fit));
 }
 
+// Constants by species pair (a lane-indexed read of the parameter block would
+// be serialised).
+template <int M, class Real>
+__device__ __forceinline__ void split_constants(const DevParams<Real>& p, Real* sm) {
+  using C = Split<M>;
+  constexpr int NP = C::NP, LPN = C::LPN;
+  const int tid = threadIdx.x;
+  Real* t = sm + C::TAB;
+  for (int k = tid; k < 2 * LPN; k += C::THREADS) {
+    const bool on = k < M;
+    const int a = on ? k : 0;
+    t[ST_RL * 2 * LPN + k] = on ? p.RL[a] : Real(0);
+    t[ST_YR * 2 * LPN + k] = on ? p.Yr[a] : Real(0);
+    t[ST_IM * 2 * LPN + k] = on ? p.inv_mass[a] : Real(0);
+    t[ST_CV * 2 * LPN + k] = on ? p.Cv_a[a] : Real(0);
+    t[ST_CP * 2 * LPN + k] = on ? p.Cp_a[a] : Real(0);
+    t[ST_MU * 2 * LPN + k] = on ? p.mu[a] : Real(0);
+    t[ST_LAM * 2 * LPN + k] = on ? p.lam[a] : Real(0);
+    t[ST_ILAM * 2 * LPN + k] = on ? p.inv_lam[a] : Real(0);
+  }
+  t += 16 * LPN;
+  for (int k = tid; k < M * 2 * LPN; k += C::THREADS) {
+    const int b = k / (2 * LPN), a = k % (2 * LPN);
+    t[k] = a < M ? p.phi[a][b] * p.inv_mass[b] : Real(0);
+    t[2 * LPN * M + k] = a < M ? p.Cab[a][b] : Real(0);
+  }
+  for (int k = tid; k < 2 * M * NP; k += C::THREADS) {
+    const int a = k / (2 * NP), b = k % (2 * NP);
+    sm[C::TABC + k] = b < M ? p.Cab[a][b] : Real(0);
+  }
+}
+
+// One tile of 32 nodes.  All threads of the block take part; it ends on a
+// barrier, and reads the constants only behind its first.
 // BND: 0 periodic, 1 bounce-back walls normal to x, 2 opposed-jets frame.
 template <int M, class Real, class Store, int PAR, int BND>
-__global__ void __launch_bounds__(Split<M>::THREADS, split_min_blocks<M, Real>())
-collide_split_kernel(const __grid_constant__ DevParams<Real> p, Store* __restrict__ pops, Real* __restrict__ side,
-                     unsigned* __restrict__ err, int ntiles, const __grid_constant__ PlaneOffsets po) {
+__device__ __forceinline__ void split_tile(const DevParams<Real>& p, Store* __restrict__ pops, Real* __restrict__ side,
+                                           unsigned* __restrict__ err, const PlaneOffsets& po, Real* const sm, int tile) {
   using C = Split<M>;
   using V = typename Pair<Real>::T;
   constexpr int NP = C::NP, LPN = C::LPN, LD = C::LD;
   constexpr bool EQ = kEqCodec<Store, Real>, WALL = BND == 1;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  Real* const sm = reinterpret_cast<Real*>(smem_raw);
   const int tid = threadIdx.x, lane = tid & 31, role = tid >> 5;
   V* const stage = reinterpret_cast<V*>(sm + C::STAGE) + lane;
   Real* const fg = sm + C::FG + lane;
   V* const dif = reinterpret_cast<V*>(sm + C::DIF) + lane;
   Real* const node = sm + C::ND + lane;
   const long long N = p.N;
-
-  // Constants by species pair (a lane-indexed read of the parameter block
-  // would be serialised).
-  {
-    Real* t = sm + C::TAB;
-    for (int k = tid; k < 2 * LPN; k += C::THREADS) {
-      const bool on = k < M;
-      const int a = on ? k : 0;
-      t[ST_RL * 2 * LPN + k] = on ? p.RL[a] : Real(0);
-      t[ST_YR * 2 * LPN + k] = on ? p.Yr[a] : Real(0);
-      t[ST_IM * 2 * LPN + k] = on ? p.inv_mass[a] : Real(0);
-      t[ST_CV * 2 * LPN + k] = on ? p.Cv_a[a] : Real(0);
-      t[ST_CP * 2 * LPN + k] = on ? p.Cp_a[a] : Real(0);
-      t[ST_MU * 2 * LPN + k] = on ? p.mu[a] : Real(0);
-      t[ST_LAM * 2 * LPN + k] = on ? p.lam[a] : Real(0);
-      t[ST_ILAM * 2 * LPN + k] = on ? p.inv_lam[a] : Real(0);
-    }
-    t += 16 * LPN;
-    for (int k = tid; k < M * 2 * LPN; k += C::THREADS) {
-      const int b = k / (2 * LPN), a = k % (2 * LPN);
-      t[k] = a < M ? p.phi[a][b] * p.inv_mass[b] : Real(0);
-      t[2 * LPN * M + k] = a < M ? p.Cab[a][b] : Real(0);
-    }
-    for (int k = tid; k < 2 * M * NP; k += C::THREADS) {
-      const int a = k / (2 * NP), b = k % (2 * NP);
-      sm[C::TABC + k] = b < M ? p.Cab[a][b] : Real(0);
-    }
+  const long long n_raw = (long long)tile * 32 + lane;
+  bool active = n_raw < N;
+  const long long n = active ? n_raw : N - 1;
+  if constexpr (BND == 2) {
+    const long long x = n % p.nx, y = (n / p.nx) % p.ny;
+    if (x == 0 || x == p.nx - 1 || y == 0 || y == p.ny - 1) active = false;
   }
+  const unsigned act = __ballot_sync(0xffffffffu, active);
+  const Nbr nb = make_nbr(p, n);
+  // Lattice 0's slot `slot` at node `nn`; lattice L is po.off[L * Q] further.
+  auto slot_at = [&](int slot, long long nn) { return reinterpret_cast<char*>(pops + nn) + po.off[slot]; };
+  auto lat = [&](char* q, int L) { return reinterpret_cast<Store*>(q + po.off[L * Q]); };
 
-  wait_previous();
-  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const long long n_raw = (long long)tile * 32 + lane;
-    bool active = n_raw < N;
-    const long long n = active ? n_raw : N - 1;
-    if constexpr (BND == 2) {
-      const long long x = n % p.nx, y = (n / p.nx) % p.ny;
-      if (x == 0 || x == p.nx - 1 || y == 0 || y == p.ny - 1) active = false;
-    }
-    const unsigned act = __ballot_sync(0xffffffffu, active);
-    const Nbr nb = make_nbr(p, n);
-    // Lattice 0's slot `slot` at node `nn`; lattice L is po.off[L * Q] further.
-    auto slot_at = [&](int slot, long long nn) { return reinterpret_cast<char*>(pops + nn) + po.off[slot]; };
-    auto lat = [&](char* q, int L) { return reinterpret_cast<Store*>(q + po.off[L * Q]); };
-
-    // ---- 1. load -------------------------------------------------------------
-    // 16-bit storage: rows shared out over the warps.  A row is the three
-    // velocities of one (c_y, c_z), in two parts: 0 its species but, from
-    // five, the last pair, 1 the rest.  What a population lacks is formed at
-    // its sender's x and handed to the neighbouring lane (lbm_eqcodec.cuh);
-    // needL / needR: the lane's sender at x - 1 / x + 1 is in no lane of the warp.
-    auto ysel = [&](const Nbr& b, int cy) { return cy == 0 ? b.ys[1] : (cy > 0 ? b.ys[0] : b.ys[2]); };   // of y - c_y
-    auto zsel = [&](const Nbr& b, int cz) { return cz == 0 ? b.zs[1] : (cz > 0 ? b.zs[0] : b.zs[2]); };
-    const bool needL = EQ && active && (lane == 0 || nb.xs[1] == 0);
-    const bool needR = EQ && active && (lane == 31 || (int)nb.xs[1] == p.nx - 1);
-    if constexpr (EQ) {
-      const float* const rin = eq_rec_buf(side, N, p.rec_w, 1 - PAR);
-      const unsigned long long need = (unsigned long long)__ballot_sync(0xffffffffu, needL) |
-                                      ((unsigned long long)__ballot_sync(0xffffffffu, needR) << 32);
-      const int cnt = 9 * __popcll(need);
+  // ---- 1. load -------------------------------------------------------------
+  // 16-bit storage: rows shared out over the warps.  A row is the three
+  // velocities of one (c_y, c_z), in two parts: 0 its species but, from
+  // five, the last pair, 1 the rest.  What a population lacks is formed at
+  // its sender's x and handed to the neighbouring lane (lbm_eqcodec.cuh);
+  // needL / needR: the lane's sender at x - 1 / x + 1 is in no lane of the warp.
+  auto ysel = [&](const Nbr& b, int cy) { return cy == 0 ? b.ys[1] : (cy > 0 ? b.ys[0] : b.ys[2]); };   // of y - c_y
+  auto zsel = [&](const Nbr& b, int cz) { return cz == 0 ? b.zs[1] : (cz > 0 ? b.zs[0] : b.zs[2]); };
+  const bool needL = EQ && active && (lane == 0 || nb.xs[1] == 0);
+  const bool needR = EQ && active && (lane == 31 || (int)nb.xs[1] == p.nx - 1);
+  if constexpr (EQ) {
+    const float* const rin = eq_rec_buf(side, N, p.rec_w, 1 - PAR);
+    const unsigned long long need = (unsigned long long)__ballot_sync(0xffffffffu, needL) |
+                                    ((unsigned long long)__ballot_sync(0xffffffffu, needR) << 32);
+    const int cnt = 9 * __popcll(need);
 #pragma unroll 1
-      for (int e = tid; e < cnt; e += C::THREADS) {
-        unsigned long long rest = need;
-        for (int k = e / 9; k > 0; --k) rest &= rest - 1;
-        const int who = __ffsll((long long)rest) - 1, row = e % 9;
-        const int cx = who < 32 ? 1 : -1, cy = row % 3 - 1, cz = row / 3 - 1, k = who & 31;
-        const long long nk = (long long)tile * 32 + k;
-        const Nbr nbk = make_nbr(p, nk);
-        const bool refl = WALL && arrives_from_wall_c(nbk, cx);
-        const long long snd = refl ? nk : (long long)(zsel(nbk, cz) + ysel(nbk, cy) + (cx > 0 ? nbk.xs[0] : nbk.xs[2]));
-        const RowLoad<M> in(p, side, rin, snd, cy, cz);
-        float2 v[NP];
-        float fv, gv;
-        edge_terms<M>(p, in, refl, cx, cy, cz, v, fv, gv);
-        const int i = (cx + 1) + 3 * row;
+    for (int e = tid; e < cnt; e += C::THREADS) {
+      unsigned long long rest = need;
+      for (int k = e / 9; k > 0; --k) rest &= rest - 1;
+      const int who = __ffsll((long long)rest) - 1, row = e % 9;
+      const int cx = who < 32 ? 1 : -1, cy = row % 3 - 1, cz = row / 3 - 1, k = who & 31;
+      const long long nk = (long long)tile * 32 + k;
+      const Nbr nbk = make_nbr(p, nk);
+      const bool refl = WALL && arrives_from_wall_c(nbk, cx);
+      const long long snd = refl ? nk : (long long)(zsel(nbk, cz) + ysel(nbk, cy) + (cx > 0 ? nbk.xs[0] : nbk.xs[2]));
+      const RowLoad<M> in(p, side, rin, snd, cy, cz);
+      float2 v[NP];
+      float fv, gv;
+      edge_terms<M>(p, in, refl, cx, cy, cz, v, fv, gv);
+      const int i = (cx + 1) + 3 * row;
 #pragma unroll
-        for (int q = 0; q < NP; ++q) stage[i * NP * 32 + q * 32 + k - lane] = v[q];
-        fg[2 * i * 32 + k - lane] = fv;
-        fg[(2 * i + 1) * 32 + k - lane] = gv;
+      for (int q = 0; q < NP; ++q) stage[i * NP * 32 + q * 32 + k - lane] = v[q];
+      fg[2 * i * 32 + k - lane] = fv;
+      fg[(2 * i + 1) * 32 + k - lane] = gv;
+    }
+    __syncthreads();
+  }
+  if constexpr (EQ) {
+    // Warps take the two parts in turn: WARPS may be even.
+    const float* const rin = eq_rec_buf(side, N, p.rec_w, 1 - PAR);
+#pragma unroll 1
+    for (int it = role, turn = 0; it < 18; it += C::WARPS, turn ^= 1) {
+      const int pair = it >> 1, part = C::WARPS % 2 == 0 ? (it & 1) ^ turn : it & 1;
+      const int row = pair, cy = row % 3 - 1, cz = row / 3 - 1, i0 = 3 * row;
+      const unsigned rb = ysel(nb, cy) + zsel(nb, cz);
+      const long long own = (long long)(rb + nb.xs[1]);                 // the sender at this x
+      char* src[3];
+#pragma unroll
+      for (int x = 0; x < 3; ++x) {
+        const bool here = PAR == 0 || (WALL && arrives_from_wall_c(nb, x - 1));        // aa_read_loc
+        src[x] = slot_at(here ? i0 + x : Q - 1 - i0 - x, here ? n : (long long)(rb + nb.xs[2 - x]));
       }
-      __syncthreads();
-    }
-    if constexpr (EQ) {
-      // Warps take the two parts in turn: WARPS may be even.
-      const float* const rin = eq_rec_buf(side, N, p.rec_w, 1 - PAR);
-#pragma unroll 1
-      for (int it = role, turn = 0; it < 18; it += C::WARPS, turn ^= 1) {
-        const int pair = it >> 1, part = C::WARPS % 2 == 0 ? (it & 1) ^ turn : it & 1;
-        const int row = pair, cy = row % 3 - 1, cz = row / 3 - 1, i0 = 3 * row;
-        const unsigned rb = ysel(nb, cy) + zsel(nb, cz);
-        const long long own = (long long)(rb + nb.xs[1]);                 // the sender at this x
-        char* src[3];
+      const float4* rec = reinterpret_cast<const float4*>(rin) + own;
+      // pairs [q0, q0 + K) of the row
+      auto species = [&](auto Q0_, auto K_, const float4& A) {
+        constexpr int q0 = decltype(Q0_)::value, K = decltype(K_)::value;
+        Store raw[K][3][2];
+        float2 d[K];
 #pragma unroll
-        for (int x = 0; x < 3; ++x) {
-          const bool here = PAR == 0 || (WALL && arrives_from_wall_c(nb, x - 1));        // aa_read_loc
-          src[x] = slot_at(here ? i0 + x : Q - 1 - i0 - x, here ? n : (long long)(rb + nb.xs[2 - x]));
-        }
-        const float4* rec = reinterpret_cast<const float4*>(rin) + own;
-        // pairs [q0, q0 + K) of the row
-        auto species = [&](auto Q0_, auto K_, const float4& A) {
-          constexpr int q0 = decltype(Q0_)::value, K = decltype(K_)::value;
-          Store raw[K][3][2];
-          float2 d[K];
-#pragma unroll
-          for (int k = 0; k < K; ++k) {
-            const int q = q0 + k;
-            d[k] = reinterpret_cast<const float2*>(rec + (2 + q / 2) * N)[q % 2];
-#pragma unroll
-            for (int x = 0; x < 3; ++x) {
-              raw[k][x][0] = *lat(src[x], 2 * q);
-              if (2 * q + 1 < M) raw[k][x][1] = *lat(src[x], 2 * q + 1);
-            }
-          }
-          const float4 w = p.weak ? rec[(2 + (1 + M + 3) / 4) * N] : A;
-          const RowSpecies r(w.x, w.y, w.z, add1(p.Tr, A.w), cy, cz);
-#pragma unroll
-          for (int k = 0; k < K; ++k) {
-            const int q = q0 + k;
-            float2 t[3];
-            row_species(p, r, 2 * q, 2 * q + 1 < M ? 2 * q + 1 : 2 * q, d[k], t);
-            t[2].x = __shfl_up_sync(0xffffffffu, t[2].x, 1);
-            t[2].y = __shfl_up_sync(0xffffffffu, t[2].y, 1);
-            t[0].x = __shfl_down_sync(0xffffffffu, t[0].x, 1);
-            t[0].y = __shfl_down_sync(0xffffffffu, t[0].y, 1);
-            if (needL) t[2] = stage[((i0 + 2) * NP + q) * 32];
-            if (needR) t[0] = stage[(i0 * NP + q) * 32];
-#pragma unroll
-            for (int x = 0; x < 3; ++x) {
-              float2 v;
-              v.x = codec_decode<Store, float>(p, raw[k][x][0], 2 * q) + t[x].x;
-              v.y = 2 * q + 1 < M ? codec_decode<Store, float>(p, raw[k][x][1], 2 * q + 1) + t[x].y : 0.0f;
-              stage[((i0 + x) * NP + q) * 32] = v;
-            }
-          }
-        };
-        constexpr int Q1 = NP >= 3 ? NP - 1 : NP;          // pairs of part 0
-        using Zero = std::integral_constant<int, 0>;
-        using First = std::integral_constant<int, Q1>;
-        using Last = std::integral_constant<int, NP - Q1>;
-        const float4 A = *rec;
-        if (part == 0) {
-          species(Zero{}, First{}, A);
-        } else {
-          Store raw[3][2];
-#pragma unroll
-          for (int x = 0; x < 3; ++x) { raw[x][0] = *lat(src[x], M); raw[x][1] = *lat(src[x], M + 1); }
-          const float4 B = rec[N];
-          const float hq = reinterpret_cast<const float*>(rec + (2 + M / 4) * N)[M % 4];
-          const RowSide<false> sd(side, N, own, cy, cz);
-          if constexpr (Last::value > 0) species(First{}, Last{}, A);
-          float f[3], g[3];
-          row_fg<false>(p, M, A, B, hq, sd.k, sd.x, cy, cz, f, g, nullptr, nullptr);
-          f[2] = __shfl_up_sync(0xffffffffu, f[2], 1);
-          g[2] = __shfl_up_sync(0xffffffffu, g[2], 1);
-          f[0] = __shfl_down_sync(0xffffffffu, f[0], 1);
-          g[0] = __shfl_down_sync(0xffffffffu, g[0], 1);
-          if (needL) { f[2] = fg[2 * (i0 + 2) * 32]; g[2] = fg[(2 * (i0 + 2) + 1) * 32]; }
-          if (needR) { f[0] = fg[2 * i0 * 32]; g[0] = fg[(2 * i0 + 1) * 32]; }
+        for (int k = 0; k < K; ++k) {
+          const int q = q0 + k;
+          d[k] = reinterpret_cast<const float2*>(rec + (2 + q / 2) * N)[q % 2];
 #pragma unroll
           for (int x = 0; x < 3; ++x) {
-            fg[2 * (i0 + x) * 32] = codec_decode<Store, float>(p, raw[x][0], M) + f[x];
-            fg[(2 * (i0 + x) + 1) * 32] = codec_decode<Store, float>(p, raw[x][1], M + 1) + g[x];
+            raw[k][x][0] = *lat(src[x], 2 * q);
+            if (2 * q + 1 < M) raw[k][x][1] = *lat(src[x], 2 * q + 1);
           }
         }
+        const float4 w = p.weak ? rec[(2 + (1 + M + 3) / 4) * N] : A;
+        const RowSpecies r(w.x, w.y, w.z, add1(p.Tr, A.w), cy, cz);
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+          const int q = q0 + k;
+          float2 t[3];
+          row_species(p, r, 2 * q, 2 * q + 1 < M ? 2 * q + 1 : 2 * q, d[k], t);
+          t[2].x = __shfl_up_sync(0xffffffffu, t[2].x, 1);
+          t[2].y = __shfl_up_sync(0xffffffffu, t[2].y, 1);
+          t[0].x = __shfl_down_sync(0xffffffffu, t[0].x, 1);
+          t[0].y = __shfl_down_sync(0xffffffffu, t[0].y, 1);
+          if (needL) t[2] = stage[((i0 + 2) * NP + q) * 32];
+          if (needR) t[0] = stage[(i0 * NP + q) * 32];
+#pragma unroll
+          for (int x = 0; x < 3; ++x) {
+            float2 v;
+            v.x = codec_decode<Store, float>(p, raw[k][x][0], 2 * q) + t[x].x;
+            v.y = 2 * q + 1 < M ? codec_decode<Store, float>(p, raw[k][x][1], 2 * q + 1) + t[x].y : 0.0f;
+            stage[((i0 + x) * NP + q) * 32] = v;
+          }
+        }
+      };
+      constexpr int Q1 = NP >= 3 ? NP - 1 : NP;          // pairs of part 0
+      using Zero = std::integral_constant<int, 0>;
+      using First = std::integral_constant<int, Q1>;
+      using Last = std::integral_constant<int, NP - Q1>;
+      const float4 A = *rec;
+      if (part == 0) {
+        species(Zero{}, First{}, A);
+      } else {
+        Store raw[3][2];
+#pragma unroll
+        for (int x = 0; x < 3; ++x) { raw[x][0] = *lat(src[x], M); raw[x][1] = *lat(src[x], M + 1); }
+        const float4 B = rec[N];
+        const float hq = reinterpret_cast<const float*>(rec + (2 + M / 4) * N)[M % 4];
+        const RowSide<false> sd(side, N, own, cy, cz);
+        if constexpr (Last::value > 0) species(First{}, Last{}, A);
+        float f[3], g[3];
+        row_fg<false>(p, M, A, B, hq, sd.k, sd.x, cy, cz, f, g, nullptr, nullptr);
+        f[2] = __shfl_up_sync(0xffffffffu, f[2], 1);
+        g[2] = __shfl_up_sync(0xffffffffu, g[2], 1);
+        f[0] = __shfl_down_sync(0xffffffffu, f[0], 1);
+        g[0] = __shfl_down_sync(0xffffffffu, g[0], 1);
+        if (needL) { f[2] = fg[2 * (i0 + 2) * 32]; g[2] = fg[(2 * (i0 + 2) + 1) * 32]; }
+        if (needR) { f[0] = fg[2 * i0 * 32]; g[0] = fg[(2 * i0 + 1) * 32]; }
+#pragma unroll
+        for (int x = 0; x < 3; ++x) {
+          fg[2 * (i0 + x) * 32] = codec_decode<Store, float>(p, raw[x][0], M) + f[x];
+          fg[(2 * (i0 + x) + 1) * 32] = codec_decode<Store, float>(p, raw[x][1], M + 1) + g[x];
+        }
       }
-    } else {
-      // FP64 and FP32: the velocities in turn.  (Asynchronous copies of the whole
-      // tile into the stage with the deferred terms formed by rows meanwhile
-      // measured slower: eight species 128^3 FP32 2.07 against 1.95 ms.)
+    }
+  } else {
+    // FP64 and FP32: the velocities in turn.  (Asynchronous copies of the whole
+    // tile into the stage with the deferred terms formed by rows meanwhile
+    // measured slower: eight species 128^3 FP32 2.07 against 1.95 ms.)
 #pragma unroll 1
-      for (int i = role; i < Q; i += C::WARPS) {
-        const int cz = i / 9 - 1, cy = (i / 3) % 3 - 1, cx = i % 3 - 1;
-        const bool refl = WALL && arrives_from_wall_c(nb, cx);
-        const unsigned xs = cx == 0 ? nb.xs[1] : (cx > 0 ? nb.xs[0] : nb.xs[2]);
-        const long long snd = refl ? n : (long long)(xs + ysel(nb, cy) + zsel(nb, cz));   // n - c_i, or n itself at a wall
-        const bool own = PAR == 0 || refl;                                                // aa_read_loc
-        char* const q = slot_at(own ? i : Q - 1 - i, own ? n : snd);
-        Real v[M + 2];
+    for (int i = role; i < Q; i += C::WARPS) {
+      const int cz = i / 9 - 1, cy = (i / 3) % 3 - 1, cx = i % 3 - 1;
+      const bool refl = WALL && arrives_from_wall_c(nb, cx);
+      const unsigned xs = cx == 0 ? nb.xs[1] : (cx > 0 ? nb.xs[0] : nb.xs[2]);
+      const long long snd = refl ? n : (long long)(xs + ysel(nb, cy) + zsel(nb, cz));   // n - c_i, or n itself at a wall
+      const bool own = PAR == 0 || refl;                                                // aa_read_loc
+      char* const q = slot_at(own ? i : Q - 1 - i, own ? n : snd);
+      Real v[M + 2];
 #pragma unroll
-        for (int L = 0; L < M + 2; ++L) v[L] = *lat(q, L);
-        if (i != 13) {
-          // the deferred terms (incoming_corr_th)
-          const Real th = side[SP_THR * N + snd];
-          Real kc = Real(0);
-          if (cx) { const Real k = side[(SP_K + 0) * N + snd]; kc += cx > 0 ? k : -k; }
-          if (cy) { const Real k = side[(SP_K + 1) * N + snd]; kc += cy > 0 ? k : -k; }
-          if (cz) { const Real k = side[(SP_K + 2) * N + snd]; kc += cz > 0 ? k : -k; }
-          const Real w0 = Real(1) - th, w1 = Real(0.5) * th;
-          const Real cg = (cx ? w1 : w0) * (cy ? w1 : w0) * (cz ? w1 : w0) * kc;
-          v[M + 1] += refl ? -cg : cg;
-          if (cx * cx + cy * cy + cz * cz == 1) {
-            const Real X = side[(SP_X + (cx ? 0 : (cy ? 1 : 2))) * N + snd];
-            const Real cf = (cx + cy + cz > 0 ? Real(0.5) : Real(-0.5)) * X;
-            v[M] += refl ? -cf : cf;
-          }
+      for (int L = 0; L < M + 2; ++L) v[L] = *lat(q, L);
+      if (i != 13) {
+        // the deferred terms (incoming_corr_th)
+        const Real th = side[SP_THR * N + snd];
+        Real kc = Real(0);
+        if (cx) { const Real k = side[(SP_K + 0) * N + snd]; kc += cx > 0 ? k : -k; }
+        if (cy) { const Real k = side[(SP_K + 1) * N + snd]; kc += cy > 0 ? k : -k; }
+        if (cz) { const Real k = side[(SP_K + 2) * N + snd]; kc += cz > 0 ? k : -k; }
+        const Real w0 = Real(1) - th, w1 = Real(0.5) * th;
+        const Real cg = (cx ? w1 : w0) * (cy ? w1 : w0) * (cz ? w1 : w0) * kc;
+        v[M + 1] += refl ? -cg : cg;
+        if (cx * cx + cy * cy + cz * cz == 1) {
+          const Real X = side[(SP_X + (cx ? 0 : (cy ? 1 : 2))) * N + snd];
+          const Real cf = (cx + cy + cz > 0 ? Real(0.5) : Real(-0.5)) * X;
+          v[M] += refl ? -cf : cf;
         }
-#pragma unroll
-        for (int a = 0; a < M; a += 2) {
-          V d;
-          d.x = v[a];
-          d.y = a + 1 < M ? v[a + 1] : Real(0);
-          stage[(i * NP + a / 2) * 32] = d;
-        }
-        fg[2 * i * 32] = v[M];
-        fg[(2 * i + 1) * 32] = v[M + 1];
       }
+#pragma unroll
+      for (int a = 0; a < M; a += 2) {
+        V d;
+        d.x = v[a];
+        d.y = a + 1 < M ? v[a + 1] : Real(0);
+        stage[(i * NP + a / 2) * 32] = d;
+      }
+      fg[2 * i * 32] = v[M];
+      fg[(2 * i + 1) * 32] = v[M + 1];
     }
-    __syncthreads();
+  }
+  __syncthreads();
 
-    // ---- 2. moments, each warp its own lattices' ---------------------------
-    Real q3[3] = {Real(0), Real(0), Real(0)};     // g: energy flux
-    if (role < NP) {
-      V r4[4];
-      static_for<0, Q>([&](auto I_) {
-        constexpr int i = decltype(I_)::value;
-        const V v = stage[(i * NP + role) * 32];
-        r4[0] = i == 0 ? v : vadd(r4[0], v);
-        static_for<0, 3>([&](auto A_) {
-          constexpr int c = c_of(i, decltype(A_)::value);
-          V& t = r4[1 + decltype(A_)::value];
-          if constexpr (i == 0) t = vsub(bcast<V>(Real(0)), v);         // c = (-1, -1, -1)
-          else if constexpr (c > 0) t = vadd(t, v);
-          else if constexpr (c < 0) t = vsub(t, v);
-        });
+  // ---- 2. moments, each warp its own lattices' ---------------------------
+  Real q3[3] = {Real(0), Real(0), Real(0)};     // g: energy flux
+  if (role < NP) {
+    V r4[4];
+    static_for<0, Q>([&](auto I_) {
+      constexpr int i = decltype(I_)::value;
+      const V v = stage[(i * NP + role) * 32];
+      r4[0] = i == 0 ? v : vadd(r4[0], v);
+      static_for<0, 3>([&](auto A_) {
+        constexpr int c = c_of(i, decltype(A_)::value);
+        V& t = r4[1 + decltype(A_)::value];
+        if constexpr (i == 0) t = vsub(bcast<V>(Real(0)), v);         // c = (-1, -1, -1)
+        else if constexpr (c > 0) t = vadd(t, v);
+        else if constexpr (c < 0) t = vsub(t, v);
       });
-      V* mom = reinterpret_cast<V*>(sm + C::MOM) + role * LD + lane;
+    });
+    V* mom = reinterpret_cast<V*>(sm + C::MOM) + role * LD + lane;
 #pragma unroll
-      for (int c = 0; c < 4; ++c) mom[c * LPN * LD] = r4[c];
-    } else if (role == NP) {
-      Real rho_dev = Real(0), j[3] = {Real(0), Real(0), Real(0)}, S[6] = {Real(0), Real(0), Real(0), Real(0), Real(0), Real(0)};
-      static_for<0, Q>([&](auto I_) {
-        constexpr int i = decltype(I_)::value;
-        constexpr int cx = cx_of(i), cy = cy_of(i), cz = cz_of(i);
-        const Real v = fg[2 * i * 32];
-        rho_dev += v;
-        if (cx) { j[0] += cx * v; S[0] += v; }
-        if (cy) { j[1] += cy * v; S[1] += v; }
-        if (cz) { j[2] += cz * v; S[2] += v; }
-        if (cx && cy) S[3] += (cx * cy) * v;
-        if (cx && cz) S[4] += (cx * cz) * v;
-        if (cy && cz) S[5] += (cy * cz) * v;
-      });
-      node[SN_RHOD * 32] = rho_dev;
+    for (int c = 0; c < 4; ++c) mom[c * LPN * LD] = r4[c];
+  } else if (role == NP) {
+    Real rho_dev = Real(0), j[3] = {Real(0), Real(0), Real(0)}, S[6] = {Real(0), Real(0), Real(0), Real(0), Real(0), Real(0)};
+    static_for<0, Q>([&](auto I_) {
+      constexpr int i = decltype(I_)::value;
+      constexpr int cx = cx_of(i), cy = cy_of(i), cz = cz_of(i);
+      const Real v = fg[2 * i * 32];
+      rho_dev += v;
+      if (cx) { j[0] += cx * v; S[0] += v; }
+      if (cy) { j[1] += cy * v; S[1] += v; }
+      if (cz) { j[2] += cz * v; S[2] += v; }
+      if (cx && cy) S[3] += (cx * cy) * v;
+      if (cx && cz) S[4] += (cx * cz) * v;
+      if (cy && cz) S[5] += (cy * cz) * v;
+    });
+    node[SN_RHOD * 32] = rho_dev;
 #pragma unroll
-      for (int c = 0; c < 3; ++c) node[(SN_J + c) * 32] = j[c];
+    for (int c = 0; c < 3; ++c) node[(SN_J + c) * 32] = j[c];
 #pragma unroll
-      for (int c = 0; c < 6; ++c) node[(SN_S + c) * 32] = S[c];
-    } else {
-      Real rhoE_dev = Real(0);
-      static_for<0, Q>([&](auto I_) {
-        constexpr int i = decltype(I_)::value;
-        const Real v = fg[(2 * i + 1) * 32];
-        rhoE_dev += v;
-        if (cx_of(i)) q3[0] += cx_of(i) * v;
-        if (cy_of(i)) q3[1] += cy_of(i) * v;
-        if (cz_of(i)) q3[2] += cz_of(i) * v;
-      });
-      node[SN_RHOED * 32] = rhoE_dev;
+    for (int c = 0; c < 6; ++c) node[(SN_S + c) * 32] = S[c];
+  } else {
+    Real rhoE_dev = Real(0);
+    static_for<0, Q>([&](auto I_) {
+      constexpr int i = decltype(I_)::value;
+      const Real v = fg[(2 * i + 1) * 32];
+      rhoE_dev += v;
+      if (cx_of(i)) q3[0] += cx_of(i) * v;
+      if (cy_of(i)) q3[1] += cy_of(i) * v;
+      if (cz_of(i)) q3[2] += cz_of(i) * v;
+    });
+    node[SN_RHOED * 32] = rhoE_dev;
+  }
+  __syncthreads();
+
+  // ---- 3. node closure -----------------------------------------------------
+  if (role < LPN) split_closure<M, Real>(p, sm, tid / LPN, tid % LPN, (act >> (tid / LPN)) & 1u, err);
+  __syncthreads();
+
+  // ---- 4. update, store --------------------------------------------------
+  const Nbr nbw = opaque(nb);
+  const long long nw = opaque_idx(n);
+  const Real dT = node[SN_DT * 32];
+  if (role < NP) {
+    const int a0 = 2 * role;
+    const bool two = M % 2 == 0 || role < NP - 1;
+    const V* sp = reinterpret_cast<const V*>(sm + C::SP) + lane;
+    auto pick = [&](int k) { return sp[(k * LPN + role) * LD]; };
+    V z, dz;                                        // R_a T and R_a (T - T_r)
+    z.x = p.R_a[a0]; z.y = p.R_a[a0 + (two ? 1 : 0)];
+    RestDeviation<V> e;
+    const V half = bcast<V>(Real(0.5));
+    e.r2 = vmul(z, bcast<V>(Real(0.5) * p.Tr));
+    dz = vmul(z, bcast<V>(dT));
+    z = vmul(z, bcast<V>(p.Tr + dT));
+    V b1[3], b2[3], f1[3], f2[3];                   // halved moments of u + V; differences Psi(u) - Psi(u + V)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const Real x = node[(SN_USP + c) * 32];
+      const V Vc = pick(SS_V + c);
+      const V x2 = bcast<V>(x * x);
+      e.h1[c] = bcast<V>(Real(0.5) * x);
+      e.h2[c] = vmul(half, vadd(x2, z));
+      e.d2[c] = vmul(half, vadd(x2, dz));
+      f1[c] = vmul(bcast<V>(Real(-0.5)), Vc);
+      f2[c] = vmul(f1[c], vadd(bcast<V>(x + x), Vc));
+      b1[c] = vsub(e.h1[c], f1[c]);
+      b2[c] = vsub(e.h2[c], f2[c]);
     }
-    __syncthreads();
-
-    // ---- 3. node closure -----------------------------------------------------
-    if (role < LPN) split_closure<M, Real>(p, sm, tid / LPN, tid % LPN, (act >> (tid / LPN)) & 1u, err);
-    __syncthreads();
-
-    // ---- 4. update, store --------------------------------------------------
-    const Nbr nbw = opaque(nb);
-    const long long nw = opaque_idx(n);
-    const Real dT = node[SN_DT * 32];
-    if (role < NP) {
-      const int a0 = 2 * role;
-      const bool two = M % 2 == 0 || role < NP - 1;
-      const V* sp = reinterpret_cast<const V*>(sm + C::SP) + lane;
-      auto pick = [&](int k) { return sp[(k * LPN + role) * LD]; };
-      V z, dz;                                        // R_a T and R_a (T - T_r)
-      z.x = p.R_a[a0]; z.y = p.R_a[a0 + (two ? 1 : 0)];
-      RestDeviation<V> e;
-      const V half = bcast<V>(Real(0.5));
-      e.r2 = vmul(z, bcast<V>(Real(0.5) * p.Tr));
-      dz = vmul(z, bcast<V>(dT));
-      z = vmul(z, bcast<V>(p.Tr + dT));
-      V b1[3], b2[3], f1[3], f2[3];                   // halved moments of u + V; differences Psi(u) - Psi(u + V)
+    // Force moments of each species (density apart): a_p a_q a_r - b_p b_q b_r
+    // with f = a - b, telescoped: f_p a_q a_r + b_p (f_q a_r + b_q f_r).
+    V own[NP > 1 ? 1 : 26];
+    auto fsel = [&](auto P_, int ax) { return decltype(P_)::value == 1 ? f1[ax] : f2[ax]; };
+    auto bsel = [&](auto P_, int ax) { return decltype(P_)::value == 1 ? b1[ax] : b2[ax]; };
+    static_for<0, 9>([&](auto K_) {
+      constexpr int qy = decltype(K_)::value % 3, r = decltype(K_)::value / 3;
+      using QC = std::integral_constant<int, qy>;
+      using RC = std::integral_constant<int, r>;
+      V E;
+      if constexpr (qy == 0 && r == 0) E = bcast<V>(Real(0));
+      else if constexpr (qy == 0) E = fsel(RC{}, 2);
+      else if constexpr (r == 0) E = fsel(QC{}, 1);
+      else E = vfma(fsel(QC{}, 1), e.template a<r>(2), vmul(bsel(QC{}, 1), fsel(RC{}, 2)));
+      static_for<0, 3>([&](auto P_) {
+        constexpr int pp = decltype(P_)::value, t = pp + 3 * qy + 9 * r - 1;
+        if constexpr (t >= 0) {
+          V D;
+          if constexpr (pp == 0) D = E;
+          else if constexpr (qy == 0 && r == 0) D = fsel(P_, 0);
+          else D = vfma(fsel(P_, 0), e.template ayz<qy, r>(), vmul(bsel(P_, 0), E));
+          if constexpr (NP > 1) dif[(t * NP + role) * 32] = D;
+          else own[t] = D;
+        }
+      });
+    });
+    // weights of the force moments: (beta_a - 1) (Y_a / tau_ab) rho_b, species b in pairs
+    const V beta = pick(SS_BETA), tY = pick(SS_TY), ra = pick(SS_RA), rd = pick(SS_RD);
+    const V bm = vsub(beta, bcast<V>(Real(1))), w = vmul(bm, tY);
+    const V cv = vsub(bcast<V>(Real(1)), vadd(beta, beta));       // 1 - 2 beta
+    const V ce = EQ ? vsub(bcast<V>(Real(0)), cv) : vadd(beta, beta);
+    V k0[NP], k1[NP];
+#pragma unroll
+    for (int q = 0; q < NP; ++q) {
+      const V* cab = reinterpret_cast<const V*>(sm + C::TABC) + a0 * NP + q;
+      const V rb = sp[(SS_RA * LPN + q) * LD];
+      k0[q] = vmul(vmul(bcast<V>(w.x), cab[0]), rb);
+      k1[q] = two ? vmul(vmul(bcast<V>(w.y), cab[NP]), rb) : bcast<V>(Real(0));
+    }
+    if constexpr (NP > 1) asm volatile("bar.sync 1, %0;" ::"n"(NP * 32) : "memory");
+    const V cra = vmul(ce, ra), crd = vmul(ce, rd);
+    V rest_w[4];                                     // crd times the rest moments
+    rest_w[0] = crd;
+#pragma unroll
+    for (int k = 1; k < 4; ++k) rest_w[k] = vmul(rest_w[k - 1], e.r2);
+    auto plane = [&](auto R_, V (&mm)[9]) {
+      constexpr int r = decltype(R_)::value;
+      static_for<0, 9>([&](auto K_) {
+        constexpr int k = decltype(K_)::value, pp = k % 3, qy = k / 3, t = pp + 3 * qy + 9 * r - 1;
+        constexpr int rp = RestDeviation<V>::template rest_power<pp, qy, r>();
+        V s;
+        if constexpr (t < 0) {
+          s = crd;
+        } else {
+          if constexpr (rp >= 0) s = vfma(cra, e.template e<pp, qy, r>(), rest_w[rp]);
+          else s = vmul(cra, e.template e<pp, qy, r>());
+          V s0 = bcast<V>(Real(0)), s1 = s0;
+#pragma unroll
+          for (int q = 0; q < NP; ++q) {
+            V D;
+            if constexpr (NP > 1) D = dif[(t * NP + q) * 32]; else D = own[t];
+            s0 = q == 0 ? vmul(k0[q], D) : vfma(k0[q], D, s0);
+            s1 = q == 0 ? vmul(k1[q], D) : vfma(k1[q], D, s1);
+          }
+          s.x += s0.x + s0.y;
+          s.y += s1.x + s1.y;
+        }
+        mm[k] = s;
+      });
+    };
+    char* const first = reinterpret_cast<char*>(pops) + (long long)a0 * po.off[Q];
+    auto put = [&](auto I_, V val) {
+      constexpr int i = decltype(I_)::value;
+      long long nn; int slot;
+      aa_write_loc<WALL>(PAR, nbw, nw, i, nn, slot);
+      char* const q = first + (nn * (long long)sizeof(Store) + po.off[slot]);
+      const V out = vfma(cv, stage[(i * NP + role) * 32], val);
+      if (active) {
+        codec_store<Store, Real>(p, reinterpret_cast<Store*>(q), 0, a0, out.x);
+        if (two) codec_store<Store, Real>(p, lat(q, 1), 0, a0 + 1, out.y);
+      }
+    };
+    from_moments<Real, V>(crd, plane, put, [&](V val) { put(std::integral_constant<int, 13>{}, val); });
+  } else {
+    const Real rho_dev = node[SN_RHOD * 32], dth = node[SN_DTH * 32], om = node[SN_OM * 32], om1 = node[SN_OM1 * 32];
+    const Real rho = p.RL[M] + rho_dev, inv_rho = Real(1) / rho, theta = p.thr + dth, T = p.Tr + dT;
+    const Real j[3] = {node[SN_J * 32], node[(SN_J + 1) * 32], node[(SN_J + 2) * 32]};
+    const Real u[3] = {j[0] * inv_rho, j[1] * inv_rho, j[2] * inv_rho};
+    const Real P = rho * theta, Cp = node[SN_CP * 32];
+    const Real usq = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+    if (role == NP) {
+      if (active) {
+        // side fields (Eqs. Xalpha, corrFourier; see collide_node)
+        const Real a3 = Real(1) - Real(3) * theta;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) side[(SP_PHI + c) * N + n] = j[c] * a3 - rho * u[c] * u[c] * u[c];
+        side[SP_COM * N + n] = Real(1) / om - Real(0.5);
+        side[SP_CP * N + n] = Cp;
+        side[SP_S * N + n] = Real(0.5) * (Real(2) - om1) * P * T / theta;
+        side[SP_TH * N + n] = theta;
+      }
+      // momentum lattice, Eqs. (feq), (fwithcorrection)
+      RestDeviation<Real> e;
+      e.r2 = Real(0.5) * p.thr;
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        const Real x = node[(SN_USP + c) * 32];
-        const V Vc = pick(SS_V + c);
-        const V x2 = bcast<V>(x * x);
-        e.h1[c] = bcast<V>(Real(0.5) * x);
-        e.h2[c] = vmul(half, vadd(x2, z));
-        e.d2[c] = vmul(half, vadd(x2, dz));
-        f1[c] = vmul(bcast<V>(Real(-0.5)), Vc);
-        f2[c] = vmul(f1[c], vadd(bcast<V>(x + x), Vc));
-        b1[c] = vsub(e.h1[c], f1[c]);
-        b2[c] = vsub(e.h2[c], f2[c]);
+        const Real x2 = u[c] * u[c];
+        e.h1[c] = Real(0.5) * u[c];
+        e.h2[c] = Real(0.5) * (x2 + theta);
+        e.d2[c] = Real(0.5) * (x2 + dth);
       }
-      // Force moments of each species (density apart): a_p a_q a_r - b_p b_q b_r
-      // with f = a - b, telescoped: f_p a_q a_r + b_p (f_q a_r + b_q f_r).
-      V own[NP > 1 ? 1 : 26];
-      auto fsel = [&](auto P_, int ax) { return decltype(P_)::value == 1 ? f1[ax] : f2[ax]; };
-      auto bsel = [&](auto P_, int ax) { return decltype(P_)::value == 1 ? b1[ax] : b2[ax]; };
-      static_for<0, 9>([&](auto K_) {
-        constexpr int qy = decltype(K_)::value % 3, r = decltype(K_)::value / 3;
-        using QC = std::integral_constant<int, qy>;
-        using RC = std::integral_constant<int, r>;
-        V E;
-        if constexpr (qy == 0 && r == 0) E = bcast<V>(Real(0));
-        else if constexpr (qy == 0) E = fsel(RC{}, 2);
-        else if constexpr (r == 0) E = fsel(QC{}, 1);
-        else E = vfma(fsel(QC{}, 1), e.template a<r>(2), vmul(bsel(QC{}, 1), fsel(RC{}, 2)));
-        static_for<0, 3>([&](auto P_) {
-          constexpr int pp = decltype(P_)::value, t = pp + 3 * qy + 9 * r - 1;
-          if constexpr (t >= 0) {
-            V D;
-            if constexpr (pp == 0) D = E;
-            else if constexpr (qy == 0 && r == 0) D = fsel(P_, 0);
-            else D = vfma(fsel(P_, 0), e.template ayz<qy, r>(), vmul(bsel(P_, 0), E));
-            if constexpr (NP > 1) dif[(t * NP + role) * 32] = D;
-            else own[t] = D;
-          }
-        });
-      });
-      // weights of the force moments: (beta_a - 1) (Y_a / tau_ab) rho_b, species b in pairs
-      const V beta = pick(SS_BETA), tY = pick(SS_TY), ra = pick(SS_RA), rd = pick(SS_RD);
-      const V bm = vsub(beta, bcast<V>(Real(1))), w = vmul(bm, tY);
-      const V cv = vsub(bcast<V>(Real(1)), vadd(beta, beta));       // 1 - 2 beta
-      const V ce = EQ ? vsub(bcast<V>(Real(0)), cv) : vadd(beta, beta);
-      V k0[NP], k1[NP];
-#pragma unroll
-      for (int q = 0; q < NP; ++q) {
-        const V* cab = reinterpret_cast<const V*>(sm + C::TABC) + a0 * NP + q;
-        const V rb = sp[(SS_RA * LPN + q) * LD];
-        k0[q] = vmul(vmul(bcast<V>(w.x), cab[0]), rb);
-        k1[q] = two ? vmul(vmul(bcast<V>(w.y), cab[NP]), rb) : bcast<V>(Real(0));
-      }
-      if constexpr (NP > 1) asm volatile("bar.sync 1, %0;" ::"n"(NP * 32) : "memory");
-      const V cra = vmul(ce, ra), crd = vmul(ce, rd);
-      V rest_w[4];                                     // crd times the rest moments
-      rest_w[0] = crd;
-#pragma unroll
-      for (int k = 1; k < 4; ++k) rest_w[k] = vmul(rest_w[k - 1], e.r2);
-      auto plane = [&](auto R_, V (&mm)[9]) {
+      const Real cv = Real(1) - om, ce = EQ ? -cv : om;
+      const Real cra = ce * rho, crd = ce * rho_dev;
+      const Real rest_w[4] = {crd, crd * e.r2, crd * e.r2 * e.r2, crd * e.r2 * e.r2 * e.r2};
+      auto plane = [&](auto R_, Real (&mm)[9]) {
         constexpr int r = decltype(R_)::value;
         static_for<0, 9>([&](auto K_) {
-          constexpr int k = decltype(K_)::value, pp = k % 3, qy = k / 3, t = pp + 3 * qy + 9 * r - 1;
-          constexpr int rp = RestDeviation<V>::template rest_power<pp, qy, r>();
-          V s;
-          if constexpr (t < 0) {
-            s = crd;
-          } else {
-            if constexpr (rp >= 0) s = vfma(cra, e.template e<pp, qy, r>(), rest_w[rp]);
-            else s = vmul(cra, e.template e<pp, qy, r>());
-            V s0 = bcast<V>(Real(0)), s1 = s0;
-#pragma unroll
-            for (int q = 0; q < NP; ++q) {
-              V D;
-              if constexpr (NP > 1) D = dif[(t * NP + q) * 32]; else D = own[t];
-              s0 = q == 0 ? vmul(k0[q], D) : vfma(k0[q], D, s0);
-              s1 = q == 0 ? vmul(k1[q], D) : vfma(k1[q], D, s1);
-            }
-            s.x += s0.x + s0.y;
-            s.y += s1.x + s1.y;
-          }
-          mm[k] = s;
+          constexpr int k = decltype(K_)::value, pp = k % 3, qy = k / 3;
+          constexpr int rp = RestDeviation<Real>::template rest_power<pp, qy, r>();
+          if constexpr (pp + qy + r == 0) mm[k] = crd;
+          else if constexpr (rp >= 0) mm[k] = cra * e.template e<pp, qy, r>() + rest_w[rp];
+          else mm[k] = cra * e.template e<pp, qy, r>();
         });
       };
-      char* const first = reinterpret_cast<char*>(pops) + (long long)a0 * po.off[Q];
-      auto put = [&](auto I_, V val) {
+      auto put = [&](auto I_, Real val) {
         constexpr int i = decltype(I_)::value;
         long long nn; int slot;
         aa_write_loc<WALL>(PAR, nbw, nw, i, nn, slot);
-        char* const q = first + (nn * (long long)sizeof(Store) + po.off[slot]);
-        const V out = vfma(cv, stage[(i * NP + role) * 32], val);
-        if (active) {
-          codec_store<Store, Real>(p, reinterpret_cast<Store*>(q), 0, a0, out.x);
-          if (two) codec_store<Store, Real>(p, lat(q, 1), 0, a0 + 1, out.y);
-        }
+        if (active) codec_store<Store, Real>(p, lat(slot_at(slot, nn), M), 0, M, cv * fg[2 * i * 32] + val);
       };
-      from_moments<Real, V>(crd, plane, put, [&](V val) { put(std::integral_constant<int, 13>{}, val); });
+      from_moments<Real, Real>(crd, plane, put, [&](Real val) { put(std::integral_constant<int, 13>{}, val); });
     } else {
-      const Real rho_dev = node[SN_RHOD * 32], dth = node[SN_DTH * 32], om = node[SN_OM * 32], om1 = node[SN_OM1 * 32];
-      const Real rho = p.RL[M] + rho_dev, inv_rho = Real(1) / rho, theta = p.thr + dth, T = p.Tr + dT;
-      const Real j[3] = {node[SN_J * 32], node[(SN_J + 1) * 32], node[(SN_J + 2) * 32]};
-      const Real u[3] = {j[0] * inv_rho, j[1] * inv_rho, j[2] * inv_rho};
-      const Real P = rho * theta, Cp = node[SN_CP * 32];
-      const Real usq = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-      if (role == NP) {
-        if (active) {
-          // side fields (Eqs. Xalpha, corrFourier; see collide_node)
-          const Real a3 = Real(1) - Real(3) * theta;
+      // energy lattice (see collide_node for the closed form)
+      const Real rhoE_dev = node[SN_RHOED * 32];
+      const Real dP = rho_dev * theta + p.RL[M] * dth;
+      const Real hk = Cp * T + Real(0.5) * usq, inv_theta = Real(1) / theta;
+      const Real Gc = rho * (hk + theta) * Real(0.5) * inv_theta;
+      const Real dE0 = rhoE_dev - Real(1.5) * dP - Gc * usq;
+      Real dZ[3], mvec[3], qt[3];
+      {
+        const Real z1 = Real(1) - Real(3) * theta;
+        const Real zb = Real(0.5) * (z1 * dP - Real(3) * dth * p.Pr);
 #pragma unroll
-          for (int c = 0; c < 3; ++c) side[(SP_PHI + c) * N + n] = j[c] * a3 - rho * u[c] * u[c] * u[c];
-          side[SP_COM * N + n] = Real(1) / om - Real(0.5);
-          side[SP_CP * N + n] = Cp;
-          side[SP_S * N + n] = Real(0.5) * (Real(2) - om1) * P * T / theta;
-          side[SP_TH * N + n] = theta;
-        }
-        // momentum lattice, Eqs. (feq), (fwithcorrection)
-        RestDeviation<Real> e;
-        e.r2 = Real(0.5) * p.thr;
+        for (int c = 0; c < 3; ++c) dZ[c] = zb + z1 * Gc * u[c] * u[c];
+        Real S[6];
+#pragma unroll
+        for (int c = 0; c < 6; ++c) S[c] = node[(SN_S + c) * 32];
+        Real dP6[6];                                       // Pi - P^eq
+#pragma unroll
+        for (int c = 0; c < 3; ++c) dP6[c] = p.cPi + S[c] - dP - rho * u[c] * u[c];
+        dP6[3] = S[3] - rho * u[0] * u[1];
+        dP6[4] = S[4] - rho * u[0] * u[2];
+        dP6[5] = S[5] - rho * u[1] * u[2];
+        const Real qb[3] = {q3[0] - (u[0] * dP6[0] + u[1] * dP6[3] + u[2] * dP6[4]),
+                            q3[1] - (u[0] * dP6[3] + u[1] * dP6[1] + u[2] * dP6[5]),
+                            q3[2] - (u[0] * dP6[4] + u[1] * dP6[5] + u[2] * dP6[2])};
+        const Real rY = p.weak ? rho / node[SN_RHOSP * 32] : Real(1);
+        const Real c1 = om1 * T * rY, dw = om - om1;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-          const Real x2 = u[c] * u[c];
-          e.h1[c] = Real(0.5) * u[c];
-          e.h2[c] = Real(0.5) * (x2 + theta);
-          e.d2[c] = Real(0.5) * (x2 + dth);
+          const Real qeq = hk * j[c];
+          qt[c] = qeq * inv_theta;
+          mvec[c] = (om * qeq + dw * (qb[c] - qeq) + c1 * node[(SN_HYV + c) * 32]) * inv_theta;
         }
-        const Real cv = Real(1) - om, ce = EQ ? -cv : om;
-        const Real cra = ce * rho, crd = ce * rho_dev;
-        const Real rest_w[4] = {crd, crd * e.r2, crd * e.r2 * e.r2, crd * e.r2 * e.r2 * e.r2};
-        auto plane = [&](auto R_, Real (&mm)[9]) {
-          constexpr int r = decltype(R_)::value;
-          static_for<0, 9>([&](auto K_) {
-            constexpr int k = decltype(K_)::value, pp = k % 3, qy = k / 3;
-            constexpr int rp = RestDeviation<Real>::template rest_power<pp, qy, r>();
-            if constexpr (pp + qy + r == 0) mm[k] = crd;
-            else if constexpr (rp >= 0) mm[k] = cra * e.template e<pp, qy, r>() + rest_w[rp];
-            else mm[k] = cra * e.template e<pp, qy, r>();
-          });
-        };
-        auto put = [&](auto I_, Real val) {
-          constexpr int i = decltype(I_)::value;
-          long long nn; int slot;
-          aa_write_loc<WALL>(PAR, nbw, nw, i, nn, slot);
-          if (active) codec_store<Store, Real>(p, lat(slot_at(slot, nn), M), 0, M, cv * fg[2 * i * 32] + val);
-        };
-        from_moments<Real, Real>(crd, plane, put, [&](Real val) { put(std::integral_constant<int, 13>{}, val); });
-      } else {
-        // energy lattice (see collide_node for the closed form)
-        const Real rhoE_dev = node[SN_RHOED * 32];
-        const Real dP = rho_dev * theta + p.RL[M] * dth;
-        const Real hk = Cp * T + Real(0.5) * usq, inv_theta = Real(1) / theta;
-        const Real Gc = rho * (hk + theta) * Real(0.5) * inv_theta;
-        const Real dE0 = rhoE_dev - Real(1.5) * dP - Gc * usq;
-        Real dZ[3], mvec[3], qt[3];
-        {
-          const Real z1 = Real(1) - Real(3) * theta;
-          const Real zb = Real(0.5) * (z1 * dP - Real(3) * dth * p.Pr);
-#pragma unroll
-          for (int c = 0; c < 3; ++c) dZ[c] = zb + z1 * Gc * u[c] * u[c];
-          Real S[6];
-#pragma unroll
-          for (int c = 0; c < 6; ++c) S[c] = node[(SN_S + c) * 32];
-          Real dP6[6];                                       // Pi - P^eq
-#pragma unroll
-          for (int c = 0; c < 3; ++c) dP6[c] = p.cPi + S[c] - dP - rho * u[c] * u[c];
-          dP6[3] = S[3] - rho * u[0] * u[1];
-          dP6[4] = S[4] - rho * u[0] * u[2];
-          dP6[5] = S[5] - rho * u[1] * u[2];
-          const Real qb[3] = {q3[0] - (u[0] * dP6[0] + u[1] * dP6[3] + u[2] * dP6[4]),
-                              q3[1] - (u[0] * dP6[3] + u[1] * dP6[1] + u[2] * dP6[5]),
-                              q3[2] - (u[0] * dP6[4] + u[1] * dP6[5] + u[2] * dP6[2])};
-          const Real rY = p.weak ? rho / node[SN_RHOSP * 32] : Real(1);
-          const Real c1 = om1 * T * rY, dw = om - om1;
-#pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            const Real qeq = hk * j[c];
-            qt[c] = qeq * inv_theta;
-            mvec[c] = (om * qeq + dw * (qb[c] - qeq) + c1 * node[(SN_HYV + c) * 32]) * inv_theta;
-          }
-        }
-        if constexpr (EQ) {
-          if (active) {
-            EqRec<M> r;
-#pragma unroll
-            for (int c = 0; c < 3; ++c) { r.u[c] = u[c]; r.usp[c] = node[(SN_USP + c) * 32]; }
-            r.dth = dth; r.dT = dT; r.drho = rho_dev; r.dE0 = dE0;
-            r.Gq = Gc * inv_theta; r.hq = hk * rho * inv_theta;
-#pragma unroll
-            for (int a = 0; a < M; ++a) {
-              const V d = reinterpret_cast<const V*>(sm + C::SP)[(SS_RD * LPN + a / 2) * LD + lane];
-              r.ra[a] = a % 2 ? d.y : d.x;
-            }
-            store_rec<M>(eq_rec_buf(side, N, p.rec_w, PAR), N, n, p.weak, r);
-          }
-        }
-        const Real w0 = Real(1) - theta, w1 = Real(0.5) * theta;          // Eq. (w0)
-        const Real r0 = Real(1) - p.thr, r1 = Real(0.5) * p.thr;
-        const Real d0 = -dth, d1 = Real(0.5) * dth;
-        Real s_g = Real(0);
-        static_for<0, 13>([&](auto I_) {
-          constexpr int i = decltype(I_)::value, o = Q - 1 - i;
-          constexpr int cx = cx_of(i), cy = cy_of(i), cz = cz_of(i);
-          long long node_i, node_o; int slot_i, slot_o;
-          aa_write_loc<WALL>(PAR, nbw, nw, i, node_i, slot_i);
-          aa_write_loc<WALL>(PAR, nbw, nw, o, node_o, slot_o);
-          const Real uc = dotc<Real, i>(u);
-          const Real cc = Real(0.5) * Real(c2_of(i));
-          const Real ucu = Gc * uc * uc * inv_theta;
-          const Real dEi = dE0 + cc * rho_dev + ucu;
-          const Real wx = cx ? w1 : w0, wy = cy ? w1 : w0, wz = cz ? w1 : w0;
-          const Real rx = cx ? r1 : r0, ry = cy ? r1 : r0;
-          const Real dx = cx ? d1 : d0, dy = cy ? d1 : d0, dzz = cz ? d1 : d0;
-          const Real wi = wx * wy * wz;
-          const Real dwi = dx * wy * wz + rx * dy * wz + rx * ry * dzz;
-          const Real eg = wi * dEi + dwi * energy_rest(p, M, c2_of(i)) + BdotZ<Real, i>(dZ);
-          s_g += eg + eg;
-          const Real fl = wi * dotc<Real, i>(mvec);
-          const Real gi = fg[(2 * i + 1) * 32], go = fg[(2 * o + 1) * 32];
-          const Real out_i = gi + om * (eg - gi) + fl;
-          const Real out_o = go + om * (eg - go) - fl;
-          if (active) {
-            const Real sq = EQ ? wi * dotc<Real, i>(qt) : Real(0);
-            codec_store<Store, Real>(p, lat(slot_at(slot_i, node_i), M + 1), 0, M + 1, EQ ? out_i - (eg + sq) : out_i);
-            codec_store<Store, Real>(p, lat(slot_at(slot_o, node_o), M + 1), 0, M + 1, EQ ? out_o - (eg - sq) : out_o);
-          }
-        });
-        long long nn; int slot;
-        aa_write_loc<WALL>(PAR, nbw, nw, 13, nn, slot);
-        const Real e13 = rhoE_dev - s_g;
-        const Real gr = fg[(2 * 13 + 1) * 32];
-        const Real out = gr + om * (e13 - gr);
-        if (active) codec_store<Store, Real>(p, lat(slot_at(slot, nn), M + 1), 0, M + 1, EQ ? out - e13 : out);
       }
+      if constexpr (EQ) {
+        if (active) {
+          EqRec<M> r;
+#pragma unroll
+          for (int c = 0; c < 3; ++c) { r.u[c] = u[c]; r.usp[c] = node[(SN_USP + c) * 32]; }
+          r.dth = dth; r.dT = dT; r.drho = rho_dev; r.dE0 = dE0;
+          r.Gq = Gc * inv_theta; r.hq = hk * rho * inv_theta;
+#pragma unroll
+          for (int a = 0; a < M; ++a) {
+            const V d = reinterpret_cast<const V*>(sm + C::SP)[(SS_RD * LPN + a / 2) * LD + lane];
+            r.ra[a] = a % 2 ? d.y : d.x;
+          }
+          store_rec<M>(eq_rec_buf(side, N, p.rec_w, PAR), N, n, p.weak, r);
+        }
+      }
+      const Real w0 = Real(1) - theta, w1 = Real(0.5) * theta;          // Eq. (w0)
+      const Real r0 = Real(1) - p.thr, r1 = Real(0.5) * p.thr;
+      const Real d0 = -dth, d1 = Real(0.5) * dth;
+      Real s_g = Real(0);
+      static_for<0, 13>([&](auto I_) {
+        constexpr int i = decltype(I_)::value, o = Q - 1 - i;
+        constexpr int cx = cx_of(i), cy = cy_of(i), cz = cz_of(i);
+        long long node_i, node_o; int slot_i, slot_o;
+        aa_write_loc<WALL>(PAR, nbw, nw, i, node_i, slot_i);
+        aa_write_loc<WALL>(PAR, nbw, nw, o, node_o, slot_o);
+        const Real uc = dotc<Real, i>(u);
+        const Real cc = Real(0.5) * Real(c2_of(i));
+        const Real ucu = Gc * uc * uc * inv_theta;
+        const Real dEi = dE0 + cc * rho_dev + ucu;
+        const Real wx = cx ? w1 : w0, wy = cy ? w1 : w0, wz = cz ? w1 : w0;
+        const Real rx = cx ? r1 : r0, ry = cy ? r1 : r0;
+        const Real dx = cx ? d1 : d0, dy = cy ? d1 : d0, dzz = cz ? d1 : d0;
+        const Real wi = wx * wy * wz;
+        const Real dwi = dx * wy * wz + rx * dy * wz + rx * ry * dzz;
+        const Real eg = wi * dEi + dwi * energy_rest(p, M, c2_of(i)) + BdotZ<Real, i>(dZ);
+        s_g += eg + eg;
+        const Real fl = wi * dotc<Real, i>(mvec);
+        const Real gi = fg[(2 * i + 1) * 32], go = fg[(2 * o + 1) * 32];
+        const Real out_i = gi + om * (eg - gi) + fl;
+        const Real out_o = go + om * (eg - go) - fl;
+        if (active) {
+          const Real sq = EQ ? wi * dotc<Real, i>(qt) : Real(0);
+          codec_store<Store, Real>(p, lat(slot_at(slot_i, node_i), M + 1), 0, M + 1, EQ ? out_i - (eg + sq) : out_i);
+          codec_store<Store, Real>(p, lat(slot_at(slot_o, node_o), M + 1), 0, M + 1, EQ ? out_o - (eg - sq) : out_o);
+        }
+      });
+      long long nn; int slot;
+      aa_write_loc<WALL>(PAR, nbw, nw, 13, nn, slot);
+      const Real e13 = rhoE_dev - s_g;
+      const Real gr = fg[(2 * 13 + 1) * 32];
+      const Real out = gr + om * (e13 - gr);
+      if (active) codec_store<Store, Real>(p, lat(slot_at(slot, nn), M + 1), 0, M + 1, EQ ? out - e13 : out);
     }
-    __syncthreads();      // the next tile's moments take the place of this tile's
   }
+  __syncthreads();      // the next tile's moments take the place of this tile's
+}
+
+template <int M, class Real, class Store, int PAR, int BND>
+__global__ void __launch_bounds__(Split<M>::THREADS, split_min_blocks<M, Real>())
+collide_split_kernel(const __grid_constant__ DevParams<Real> p, Store* __restrict__ pops, Real* __restrict__ side,
+                     unsigned* __restrict__ err, int ntiles, const __grid_constant__ PlaneOffsets po) {
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  Real* const sm = reinterpret_cast<Real*>(smem_raw);
+  split_constants<M, Real>(p, sm);
+  wait_previous();
+  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x)
+    split_tile<M, Real, Store, PAR, BND>(p, pops, side, err, po, sm, tile);
 }
 
 }  // namespace lbm
