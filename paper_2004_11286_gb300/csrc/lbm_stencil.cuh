@@ -335,27 +335,50 @@ __device__ __forceinline__ void grad_GK_node(const G& p, Real* __restrict__ side
   const Nbr nb = make_nbr(p, n);
   Real d[3] = {Real(0), Real(0), Real(0)}, dc[3] = {Real(0), Real(0), Real(0)};
   const Real Tn = tvar ? side[SP_T * N + n] : Real(0);
-  auto phi = [&](int c, long long nn) { return side[(SP_PHI + c) * N + nn]; };
-  auto cp = [&](long long nn) {
-    Real v = side[SP_CP * N + nn];
-    if (tvar) v = fma1(Tn, fma1(Tn, side[SP_HC3 * N + nn], side[SP_HC2 * N + nn]), v);
-    return v;
-  };
+  if constexpr (ROWS) {
 #pragma unroll
-  for (int cz = -1; cz <= 1; ++cz)
+    for (int cz = -1; cz <= 1; ++cz)
 #pragma unroll
-    for (int cy = -1; cy <= 1; ++cy) {
-      const long long lo = nb.idx(-1, cy, cz), mid = nb.idx(0, cy, cz), hi = nb.idx(1, cy, cz);
+      for (int cy = -1; cy <= 1; ++cy) {
+        const long long lo = nb.idx(-1, cy, cz), mid = nb.idx(0, cy, cz), hi = nb.idx(1, cy, cz);
+        auto row = [&](int plane, auto A_, bool odd, Real acc) {
+          const Real* f = side + plane * N;
+          const Real l = f[lo], m = f[mid], h = f[hi];
+          return row_term<Real, decltype(A_)::value, true>(odd && (nb.wall & 1u) ? -l : l, m,
+                                                           odd && (nb.wall & 2u) ? -h : h, cy, cz, acc);
+        };
+        using A0 = std::integral_constant<int, 0>;
+        using A1 = std::integral_constant<int, 1>;
+        using A2 = std::integral_constant<int, 2>;
+        d[0] = row(SP_PHI, A0{}, true, d[0]);              // beyond a wall Phi_x is odd, the others even
+        if (cy) d[1] = row(SP_PHI + 1, A1{}, false, d[1]);
+        if (cz) d[2] = row(SP_PHI + 2, A2{}, false, d[2]);
+        dc[0] = row(SP_CP, A0{}, false, dc[0]);
+        if (cy) dc[1] = row(SP_CP, A1{}, false, dc[1]);
+        if (cz) dc[2] = row(SP_CP, A2{}, false, dc[2]);
+      }
+  } else {
+    // velocity by velocity, all fields of one neighbour at a time (row by row
+    // this took 18.5 against 15.0 us at 45 x 75 x 101 FP32)
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+      const int cx = cx_of(i), cy = cy_of(i), cz = cz_of(i);
+      if (i == 13) continue;
+      const long long nn = nb.idx(cx, cy, cz);
+      const Real w = iso_w<Real>(i);
+      Real cp = side[SP_CP * N + nn];
+      if (tvar) cp += Tn * (side[SP_HC2 * N + nn] + Tn * side[SP_HC3 * N + nn]);
       // beyond a wall the mirror image of Phi_x is odd, the other fields even
-      const Real plo = phi(0, lo), phi_hi = phi(0, hi);
-      d[0] = row_term<Real, 0, ROWS>((nb.wall & 1u) ? -plo : plo, Real(0), (nb.wall & 2u) ? -phi_hi : phi_hi, cy, cz, d[0]);
-      if (cy) d[1] = row_term<Real, 1, ROWS>(phi(1, lo), phi(1, mid), phi(1, hi), cy, cz, d[1]);
-      if (cz) d[2] = row_term<Real, 2, ROWS>(phi(2, lo), phi(2, mid), phi(2, hi), cy, cz, d[2]);
-      const Real clo = cp(lo), chi = cp(hi), cm = cy || cz ? cp(mid) : Real(0);
-      dc[0] = row_term<Real, 0, ROWS>(clo, cm, chi, cy, cz, dc[0]);
-      if (cy) dc[1] = row_term<Real, 1, ROWS>(clo, cm, chi, cy, cz, dc[1]);
-      if (cz) dc[2] = row_term<Real, 2, ROWS>(clo, cm, chi, cy, cz, dc[2]);
+      const bool mirror = (cx < 0 && (nb.wall & 1u)) || (cx > 0 && (nb.wall & 2u));
+      if (cx) {
+        const Real phx = side[(SP_PHI + 0) * N + nn];
+        d[0] += (cx * w) * (mirror ? -phx : phx);
+        dc[0] += (cx * w) * cp;
+      }
+      if (cy) { d[1] += (cy * w) * side[(SP_PHI + 1) * N + nn]; dc[1] += (cy * w) * cp; }
+      if (cz) { d[2] += (cz * w) * side[(SP_PHI + 2) * N + nn]; dc[2] += (cz * w) * cp; }
     }
+  }
   const Real co = side[SP_COM * N + n], sv = side[SP_S * N + n];
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
@@ -559,7 +582,7 @@ __device__ __forceinline__ void grad_GK_field(const DevParams<Real>& p, Real* __
       return F == 0 && ((cx < 0 && (nb.wall & 1u)) || (cx > 0 && (nb.wall & 2u))) ? -v : v;   // Phi_x is odd beyond a wall
     } else {
       Real v = side[SP_CP * N + nn];
-      if (p.tvar) v = fma1(Tn, fma1(Tn, side[SP_HC3 * N + nn], side[SP_HC2 * N + nn]), v);
+      if (p.tvar) v += Tn * (side[SP_HC2 * N + nn] + Tn * side[SP_HC3 * N + nn]);
       return v;
     }
   };
