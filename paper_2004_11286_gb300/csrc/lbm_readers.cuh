@@ -135,15 +135,17 @@ get_pops_kernel(const DevParams<Real> p, const Store* __restrict__ pops, const R
   const long long N = p.N, n = active ? gtid() : N - 1;
   const Nbr nb = make_nbr(p, n);
   if constexpr (kEqCodec<Store, Real>) {
+    // bound by the FP64 unit: the terms that are zero for the velocity (f's off
+    // the faces) are not added (96^3 FP16: 0.92 ms with them)
     row_populations<M, Store, true>(p, side, parity, nb, n, active,
-                                    [&](int i, int, int, int, int slot, long long node, const float (&sh)[M + 2], float cf,
-                                        float cg) {
+                                    [&](int i, int cx, int cy, int cz, int slot, long long node, const float (&sh)[M + 2],
+                                        float cf, float cg) {
       if (!active) return;
 #pragma unroll
       for (int L = 0; L < M + 2; ++L) {
         double v = (double)codec_load<Store, Real>(p, pops, (L * Q + slot) * N + node, L) + (double)sh[L];
-        if (L == M) v += (double)cf;
-        if (L == M + 1) v += (double)cg;
+        if (L == M && cx * cx + cy * cy + cz * cz == 1) v += (double)cf;
+        if (L == M + 1 && i != 13) v += (double)cg;
         out[(L * Q + i) * N + n] = base[L * Q + i] + v;
       }
     });
