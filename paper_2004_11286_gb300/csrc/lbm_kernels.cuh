@@ -228,15 +228,6 @@ diag_final_kernel(const double* __restrict__ partials, int nblocks, int nv, doub
 // ---------------------------------------------------------------------------
 // Host launchers.
 // ---------------------------------------------------------------------------
-// Grids of at most this many nodes take the stencil passes with a thread per
-// node and field: the row-blocked form leaves a 1024-node grid on one SM.
-// Measured (GB300, first / second pass, us): FP64 1024 nodes 10.6 / 6.3
-// against 40.1 / 22.9, 65,536 nodes 36 / 15 against 41 / 23, 262,144 nodes
-// 99 / 35 against 75 / 40; FP32 4096 nodes 7.1 / 6.4 against 8.2 / 6.5, 32,768
-// nodes 8.3 / 7.6 against 8.3 / 8.1, 65,536 nodes 10.3 / 8.8 against 9.7 / 8.5.
-template <class Real>
-constexpr long long kFieldStencilNodes = sizeof(Real) == 8 ? 131072 : 32768;
-
 // A kernel of the step, behind another one on the stream: its blocks may start
 // when the last block of that one has exited, before its completion has been
 // signalled (every kernel launched so calls wait_previous before it touches
@@ -334,21 +325,25 @@ struct Launch {
     launch_next(parity == 0 ? collide_split_kernel<M, Real, Store, 0, BND> : collide_split_kernel<M, Real, Store, 1, BND>,
                 dim3(grid), C::THREADS, smem, c.stream, P(c), (Store*)c.pops, side, c.err, ntiles, po);
   }
-  static constexpr bool kSplitAlways = kSplit<M, Real, Store> && kSplitTilesPerSm<M, Real, Store> == 0;   // constant heats, exact closure
+  // Bulk row loads where the blocks are whole row segments and the stage
+  // holds the stored type (FP64, FP32).
+  static constexpr bool kBulk = LBM_COLLIDE_BULK && M >= LBM_COLLIDE_BULK_MIN_M && std::is_same<Real, Store>::value;
+  static bool segments(const LaunchCtx& c) { return kBulk && P(c).nx % collide_block<M, Real, 0, Store>() == 0; }
+  // Whether the step takes the split collide (lbm_split.cuh).
   static bool split_route(const LaunchCtx& c) {
     if constexpr (kSplit<M, Real, Store>) {
       if (c.closure || P(c).tvar) return false;
-      return kSplitAlways || c.grid_nodes <= kSplitTilesPerSm<M, Real, Store> * 32LL * sm_count();
+      const int most = split_tiles_per_sm<M, Real, Store>(P(c).wall_x != 0, segments(c));
+      return most == kAnyTiles || c.grid_nodes <= most * 32LL * sm_count();
     } else {
       return false;
     }
   }
-  // Bulk row loads where the blocks are whole row segments and the stage
-  // holds the stored type (FP64, FP32).
   template <int CL>
   static void collide(const LaunchCtx& c, int parity, Real* side) {
-    // Walls normal to x (bounce-back), the opposed-jets frame: register
-    // loads, exact closure (the host refuses both with the network closure).
+    // Walls normal to x (bounce-back), the opposed-jets frame: exact closure,
+    // constant heats; a thread per node reads them by register loads (the host
+    // refuses both with the network closure and with variable heats).
     if constexpr (CL == 0 && kSplit<M, Real, Store>) {
       if (split_route(c)) {
         if (P(c).wall_x) split_launch<1>(c, parity, side);
@@ -357,22 +352,43 @@ struct Launch {
         return;
       }
     }
-    constexpr bool bulk = CL == 0 && LBM_COLLIDE_BULK && M >= LBM_COLLIDE_BULK_MIN_M && std::is_same<Real, Store>::value;
-    const bool segments = bulk && P(c).nx % collide_block<M, Real, 0, Store>() == 0;
-    if constexpr (CL == 0 && kSplitAlways) {
-      // only temperature-dependent heats get here (FP64, FP32, periodic)
-      if constexpr (!EQ) {
-        if (segments) collide_launch<0, bulk>(c, parity, side);
+    if constexpr (CL == 0) {
+      if constexpr (!kSplitWallsAlways<M, Real, Store>) {
+        if (P(c).wall_x) {
+          collide_launch<0, 0, 1>(c, parity, side);
+          return;
+        }
+      }
+      if constexpr (!kSplitAlways<M, Real, Store>) {
+        if (P(c).frame) {
+          collide_launch<0, 0, EQ ? 0 : 2>(c, parity, side);
+          return;
+        }
+      }
+      // (16-bit storage from four species: only temperature-dependent heats
+      // would get here, which the host refuses)
+      if constexpr (!(kSplitAlways<M, Real, Store> && EQ)) {
+        if (segments(c)) collide_launch<0, kBulk>(c, parity, side);
         else collide_launch<0, 0>(c, parity, side);
       }
-    } else if constexpr (CL == 0) {
-      if (P(c).wall_x) collide_launch<0, 0, 1>(c, parity, side);
-      else if (P(c).frame) collide_launch<0, 0, EQ ? 0 : 2>(c, parity, side);
-      else if (segments) collide_launch<0, bulk>(c, parity, side);
-      else collide_launch<0, 0>(c, parity, side);
     } else {
       collide_launch<CL, 0>(c, parity, side);
     }
+  }
+  // Grids of at most this many nodes take the stencil passes with a thread per
+  // node and field: with four nodes to a thread a 1024-node grid lies on one SM.
+  // The passes' sums are the same (lbm_stencil.cuh).  Measured (GB300, first +
+  // second pass, us, by field / otherwise):
+  //   rows of a multiple of four: FP64 1024 nodes 14.5 / 63, 98,304 50 / 64, 262,144
+  //     107 / 115; FP32 8192 nodes 12.7 / 14.9, 32,768 15.9 / 16.5, 110,592 23.3 / 18.7;
+  //   other rows: FP64 4224 nodes 17.1 / 27.5, 18,216 21.9 / 27.1, 32,736 29.4 / 27.0,
+  //     112,896 69 / 54; FP32 18,216 14.8 / 15.3, 32,736 16.0 / 14.8, 52,480 17.9 / 15.2;
+  //   variable heats: FP64 52,480 42 / 48, 76,032 50 / 48; FP32 32,736 16.0 / 16.8,
+  //     52,480 18.2 / 17.2.
+  static long long field_stencil_nodes(bool rows, bool tvar) {
+    if (rows) return sizeof(Real) == 8 ? 131072 : 32768;
+    if (tvar) return sizeof(Real) == 8 ? 65536 : 32768;
+    return 24576;
   }
   static cudaError_t step(const LaunchCtx& c, int parity) {
     Real* side = (Real*)c.side;
@@ -392,8 +408,8 @@ struct Launch {
     if (c.ev) cudaEventRecord(c.ev[1], c.stream);
     // Row-blocked stencils (ROWV nodes per thread) where rows split evenly; a
     // thread per node and field on grids of few nodes.
-    const bool few = c.N <= kFieldStencilNodes<Real>;
     const bool rows = P(c).nx % ROWV == 0 && !P(c).tvar;
+    const bool few = c.N <= field_stencil_nodes(rows, P(c).tvar != 0);
     const dim3 fg(grid_for(c.N, BLOCK_FIELD), 4), fx(fg.x, 3);
     if (few) launch_next(rows ? grad_GK_field_kernel<Real, true> : grad_GK_field_kernel<Real, false>, fg, BLOCK_FIELD, 0, c.stream, P(c), side);
     else if (rows) launch_next(grad_GK_row_kernel<Real>, dim3(grid_for(c.N / ROWV, BLOCK_LIGHT)), BLOCK_LIGHT, 0, c.stream, P(c), side);
@@ -408,7 +424,7 @@ struct Launch {
     return cudaGetLastError();
   }
   static cudaError_t batch_prepare() {
-    if constexpr (!kSplitAlways) {
+    if constexpr (!kSplitAlways<M, Real, Store>) {
       constexpr size_t smem = collide_smem<M, Real, 0, 0, Store>();
       allow_smem(collide_batch_kernel<M, Real, Store, 0>, smem);
       allow_smem(collide_batch_kernel<M, Real, Store, 1>, smem);
@@ -422,7 +438,7 @@ struct Launch {
   static cudaError_t batch_step(const BatchCtx& b, int parity) {
     constexpr int BS = collide_block<M, Real, 0, Store>();
     const DevParams<Real>* prm = static_cast<const DevParams<Real>*>(b.params);
-    if constexpr (!kSplitAlways) {
+    if constexpr (!kSplitAlways<M, Real, Store>) {
       constexpr size_t smem = collide_smem<M, Real, 0, 0, Store>();
       const int grid = b.grid_c < b.ntiles_c ? b.grid_c : b.ntiles_c;
       if (grid > 0)

@@ -351,28 +351,60 @@ __device__ __forceinline__ void split_closure(const DevParams<Real>& p, Real* sm
   }
 }
 
-// Where the host takes this kernel (constant heats, exact closure).
-//   * From four species always.  There a thread per node needs 255 registers
-//     and a stage of 690 to 1080 bytes, which leaves 4 to 8 warps on an SM.
-//     Measured (GB300), collide here against a thread per node: eight species
-//     FP32 128^3 1.95 against 3.18 ms, BF16 192^3 7.5 against 15.7 ms, FP64 64^3
-//     4.3 against 13.2 ms.
-//   * With two or three species on grids of few tiles per SM, where the time
-//     is one node's latency: three species FP64 1024 nodes 59 against 121 us
-//     (16,384 nodes 156 against 132), FP32 1024 nodes 12.1 against 14.8 us
-//     (16,384 nodes 14.3 against 15.7, 32,768 nodes 22.4 against 16.6); two
-//     species FP64 1024 nodes 52 against 97 us, but FP32 12.0 against 10.3.
-//     Not with 16-bit storage (three species BF16 1024 nodes 14.2 against 22.4
-//     us): there the network closure's step, which stays with a thread per
-//     node, is held to the exact step to less than a change of rounding moves
-//     a 16-bit value.
+// Where the host takes this kernel (constant heats, exact closure), by the
+// 32-node tiles per SM of the grid.  Measured (GB300, 152 SMs), collide here
+// against a thread per node:
+//   * From four species in FP64 and with 16-bit storage, and from seven in FP32,
+//     always.  There a thread per node needs 255 registers and a stage of 690 to
+//     1080 bytes, which leaves 4 to 8 warps on an SM.  FP64 48^3: M = 4 0.89
+//     against 2.06 ms, 5 1.60 / 2.78, 6 1.63 / 3.37, 7 1.89 / 4.86; BF16 96^3
+//     (thread per node before it formed the senders' terms by rows): M = 4 0.55 /
+//     1.02 ms, 5 0.72 / 1.10, 6 0.76 / 1.29, 7 0.92 / 1.69; 192^3 M = 8 7.5 /
+//     15.7.  FP32 128^3: M = 7 2.00 / 2.67 ms, M = 8 2.05 / 3.16; 48^3 M = 7 0.115 /
+//     0.136; ragged rows and walls by more.
+//   * FP32, four to six species.  The fewer the species, the less a thread per
+//     node suffers, and on large grids its time per node falls (bulk row loads,
+//     no last wave) where the split's stays.  M = 4: 16,384 nodes 15.9 / 19.2 us,
+//     32,768 24.5 / 23.8, 49,152 33.1 / 38.9, 65,536 42.4 / 39.5, 80,400 in the
+//     opposed-jets frame 57.0 / 57.6, 110,592 63.5 / 59.3, 262,144 169 / 143, 96^3
+//     554 / 428, 128^3 1290 / 1035.  M = 5: 8192 nodes 14.6 / 22.0 us, 16,384 23.0 /
+//     22.1, 32,768 33.2 / 26.8, 49,152 42.4 / 45.2, 147,456 129 / 100, 96^3 724 / 490.
+//     M = 6, rows of whole 128-node blocks: 262,144 nodes 217 / 229 us, 524,288
+//     431 / 431, 128^3 1705 / 1535; other rows 96^3 722 / 745, 127 x 129 x 130 1694 /
+//     1775.  With walls the thread per node loses its bulk loads and reads the
+//     wall per population: M = 4 65,536 nodes 40.1 / 45.3, 96^3 504 / 512; M = 5 65,536
+//     51.4 / 52.4, 147,456 124 / 120, 96^3 676 / 613; M = 6 96^3 692 / 795, 128^3 1628 /
+//     1824.
+//   * With two or three species on grids of few tiles, where the time is one
+//     node's latency: three species FP64 1024 nodes 59 / 121 us (16,384 nodes 156 /
+//     132), FP32 1024 nodes 12.1 / 14.8 us (16,384 nodes 14.3 / 15.7, 32,768 nodes
+//     22.4 / 16.6); two species FP64 1024 nodes 52 / 97 us, but FP32 12.0 / 10.3.
+//     Not with 16-bit storage (three species BF16 1024 nodes 14.2 / 22.4 us): a step
+//     whose network is rejected at every node runs a thread per node, and at
+//     M <= 3 it is held to the exact step within 1e-6 over steps, less than a
+//     changed rounding moves a stored value.  From four species the two agree to
+//     one unit of the stored part (after a step, 1e-7 to 5e-7 of the largest
+//     population at M = 4, 5, 8).
+// The tiles are those of the whole grid where the handle holds a slab of it
+// (LaunchCtx::grid_nodes): the two collides differ in rounding, and a slab
+// agrees with the undivided grid bit for bit.
 template <int M, class Real, class Store>
 constexpr bool kSplit = M >= 4 || (sizeof(Store) >= 4 && (M == 3 || (M == 2 && sizeof(Real) == 8)));
-// The largest number of tiles per SM taken (0: any), of the whole grid where
-// the handle holds a slab of it (LaunchCtx::grid_nodes): the two collides differ
-// in rounding, and a slab agrees with the undivided grid bit for bit.
+// The largest number of tiles per SM taken.  walls: bounce-back walls normal to
+// x; segments: rows of whole blocks of the thread-per-node collide (bulk loads).
+constexpr int kAnyTiles = 1 << 30;
 template <int M, class Real, class Store>
-constexpr int kSplitTilesPerSm = M >= 4 ? 0 : (sizeof(Real) == 8 ? 1 : 3);
+constexpr int split_tiles_per_sm(bool walls, bool segments) {
+  if (M <= 3) return sizeof(Real) == 8 ? 1 : 3;
+  if (sizeof(Store) != 4 || M >= 7) return kAnyTiles;
+  if (M == 4) return walls ? kAnyTiles : 12;
+  if (M == 5) return walls ? 14 : 3;
+  return segments && !walls ? 108 : kAnyTiles;
+}
+template <int M, class Real, class Store>
+constexpr bool kSplitAlways = kSplit<M, Real, Store> && split_tiles_per_sm<M, Real, Store>(false, true) == kAnyTiles;
+template <int M, class Real, class Store>
+constexpr bool kSplitWallsAlways = kSplit<M, Real, Store> && split_tiles_per_sm<M, Real, Store>(true, false) == kAnyTiles;
 
 // Blocks per SM asked of the register allocator.
 #ifndef LBM_SPLIT_THREADS

@@ -3,8 +3,9 @@ from grids above them: the undivided grid and the slabs take different stencil
 passes (whose sums are the same operation by operation) and would take
 different collides (the slabs know the whole grid's size), and the interiors
 must agree bit for bit.  The stencil lines are 32,768 nodes (FP32 fields) and
-131,072 (FP64); the collide lines 32 nodes an SM (FP64, two and three species)
-and 96 (FP32, three)."""
+131,072 (FP64) with rows of a multiple of four, 24,576 with others; the collide
+lines, in nodes an SM: 32 (FP64, two and three species), and in FP32 96 (three
+and five species) and 384 (four)."""
 
 import numpy as np
 import pytest
@@ -20,9 +21,10 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("M,precision,shape,walls", [
     # stencils: rows of a multiple of four, and not
     (2, "fp32", (64, 32, 32), False), (2, "fp32", (64, 32, 33), True), (1, "fp64", (64, 64, 64), True),
-    (1, "fp64", (64, 63, 65), False), (2, "bf16", (64, 32, 36), False),
+    (1, "fp64", (64, 27, 37), False), (2, "bf16", (64, 32, 36), False),
     # collides
     (2, "fp64", (24, 16, 16), False), (3, "fp64", (24, 17, 15), True), (3, "fp32", (48, 20, 20), False),
+    (4, "fp32", (64, 32, 31), False), (4, "fp32", (16, 32, 128), False), (5, "fp32", (24, 28, 28), False),
 ])
 def test_slabs_on_the_other_side_of_a_size_line(M, precision, shape, walls):
     wl = W.random_mixture(M=M, shape=shape, seed=90 + M, velocity=0.02)
