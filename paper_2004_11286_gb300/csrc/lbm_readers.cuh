@@ -149,21 +149,21 @@ get_pops_kernel(const DevParams<Real> p, const Store* __restrict__ pops, const R
         out[(L * Q + i) * N + n] = base[L * Q + i] + v;
       }
     });
-    return;
+  } else {
+    static_for<0, Q>([&](auto I_) {
+      constexpr int i = decltype(I_)::value;
+      long long node; int slot;
+      aa_read_loc<true>(parity, nb, n, i, node, slot);
+      Real cf = Real(0), cg = Real(0);
+      if constexpr (i != 13) deferred_terms<Real, i, true, true>(side, N, nb, n, cf, cg);
+      for (int L = 0; L < M + 2; ++L) {
+        double v = (double)pops[(L * Q + slot) * N + node];
+        if (L == M) v += (double)cf;
+        if (L == M + 1) v += (double)cg;
+        out[(L * Q + i) * N + n] = base[L * Q + i] + v;
+      }
+    });
   }
-  static_for<0, Q>([&](auto I_) {
-    constexpr int i = decltype(I_)::value;
-    long long node; int slot;
-    aa_read_loc<true>(parity, nb, n, i, node, slot);
-    Real cf = Real(0), cg = Real(0);
-    if constexpr (i != 13) deferred_terms<Real, i, true, true>(side, N, nb, n, cf, cg);
-    for (int L = 0; L < M + 2; ++L) {
-      double v = (double)codec_load<Store, Real>(p, pops, (L * Q + slot) * N + node, L);
-      if (L == M) v += (double)cf;
-      if (L == M + 1) v += (double)cg;
-      out[(L * Q + i) * N + n] = base[L * Q + i] + v;
-    }
-  });
 }
 
 // 16-bit storage: each node's equilibrium record (lbm_eqcodec.cuh) from
@@ -224,15 +224,15 @@ set_pops_kernel(const DevParams<Real> p, Store* __restrict__ pops, const Real* _
         codec_store<Store, Real>(p, pops, (L * Q + slot) * N + node, L,
                                  (Real)((in[(L * Q + i) * N + n] - base[L * Q + i]) - (double)sh[L]));
     });
-    return;
+  } else {
+    static_for<0, Q>([&](auto I_) {
+      constexpr int i = decltype(I_)::value;
+      long long node; int slot;
+      aa_read_loc<true>(parity, nb, n, i, node, slot);
+      for (int L = 0; L < M + 2; ++L)
+        pops[(L * Q + slot) * N + node] = (Store)(Real)(in[(L * Q + i) * N + n] - base[L * Q + i]);
+    });
   }
-  static_for<0, Q>([&](auto I_) {
-    constexpr int i = decltype(I_)::value;
-    long long node; int slot;
-    aa_read_loc<true>(parity, nb, n, i, node, slot);
-    for (int L = 0; L < M + 2; ++L)
-      codec_store<Store, Real>(p, pops, (L * Q + slot) * N + node, L, (Real)(in[(L * Q + i) * N + n] - base[L * Q + i]));
-  });
 }
 
 // Training pairs of the learned closure at every node: the network's

@@ -376,9 +376,13 @@ __device__ __forceinline__ void split_closure(const DevParams<Real>& p, Real* sm
 //     51.4 / 52.4, 147,456 124 / 120, 96^3 676 / 613; M = 6 96^3 692 / 795, 128^3 1628 /
 //     1824.
 //   * With two or three species on grids of few tiles, where the time is one
-//     node's latency: three species FP64 1024 nodes 59 / 121 us (16,384 nodes 156 /
-//     132), FP32 1024 nodes 12.1 / 14.8 us (16,384 nodes 14.3 / 15.7, 32,768 nodes
-//     22.4 / 16.6); two species FP64 1024 nodes 52 / 97 us, but FP32 12.0 / 10.3.
+//     node's latency.  The crossings lie where a second wave of tiles begins:
+//     three species FP32 1024 nodes 12.1 / 14.8 us, 14,336 14.5 / 15.2, 19,008 15.0 /
+//     16.5, 20,064 21.9 / 16.4; FP64 three species 1024 nodes 59 / 121 us, 4608 60 /
+//     114, 8448 82 / 114, 10,560 134 / 126; two species 1024 nodes 52 / 97 us, 4608
+//     52 / 97, 8448 63 / 97, 10,560 109 / 97.  The lines taken are 14,592 nodes (FP32)
+//     and 4864 (FP64), the measured side of each.  FP32 with two species not:
+//     1024 nodes 12.0 / 10.3.
 //     Not with 16-bit storage (three species BF16 1024 nodes 14.2 / 22.4 us): a step
 //     whose network is rejected at every node runs a thread per node, and at
 //     M <= 3 it is held to the exact step within 1e-6 over steps, less than a

@@ -238,30 +238,31 @@ __device__ __forceinline__ void load_state_moments(const DevParams<Real>& p, con
       j[0] += fx * fv; j[1] += fy * fv; j[2] += fz * fv;
       rhoE_dev += codec_decode<Store, float>(p, q[(long long)(M + 1) * Q * N], M + 1) + sh[M + 1];
     });
-    return;
-  }
-  static_for<0, Q>([&](auto I_) {
-    constexpr int i = decltype(I_)::value;
-    constexpr int cx = cx_of(i), cy = cy_of(i), cz = cz_of(i);
-    long long node; int slot;
-    aa_read_loc<true>(parity, nb, n, i, node, slot);
-    Real cf, cg, sh[M + 2];
-    incoming_terms<M, Real, Store, i>(p, side, nb, n, parity, cf, cg, sh);
+  } else {
+    (void)active;
+    static_for<0, Q>([&](auto I_) {
+      constexpr int i = decltype(I_)::value;
+      constexpr int cx = cx_of(i), cy = cy_of(i), cz = cz_of(i);
+      long long node; int slot;
+      aa_read_loc<true>(parity, nb, n, i, node, slot);
+      Real cf = Real(0), cg = Real(0);
+      if constexpr (i != 13) deferred_terms<Real, i, true, true>(side, N, nb, n, cf, cg);
 #pragma unroll
-    for (int a = 0; a < M; ++a) {
-      const Real v = codec_load<Store, Real>(p, pops, (a * Q + slot) * N + node, a) + sh[a];
-      rdev[a] += v;
-      if (cx) ja[a][0] += cx * v;
-      if (cy) ja[a][1] += cy * v;
-      if (cz) ja[a][2] += cz * v;
-    }
-    const Real fv = codec_load<Store, Real>(p, pops, (M * Q + slot) * N + node, M) + cf + sh[M];
-    rho_dev += fv;
-    if (cx) j[0] += cx * fv;
-    if (cy) j[1] += cy * fv;
-    if (cz) j[2] += cz * fv;
-    rhoE_dev += codec_load<Store, Real>(p, pops, ((M + 1) * Q + slot) * N + node, M + 1) + cg + sh[M + 1];
-  });
+      for (int a = 0; a < M; ++a) {
+        const Real v = pops[(a * Q + slot) * N + node];
+        rdev[a] += v;
+        if (cx) ja[a][0] += cx * v;
+        if (cy) ja[a][1] += cy * v;
+        if (cz) ja[a][2] += cz * v;
+      }
+      const Real fv = pops[(M * Q + slot) * N + node] + cf;
+      rho_dev += fv;
+      if (cx) j[0] += cx * fv;
+      if (cy) j[1] += cy * fv;
+      if (cz) j[2] += cz * fv;
+      rhoE_dev += pops[((M + 1) * Q + slot) * N + node] + cg;
+    });
+  }
 }
 
 // Stencil pass 1 (after a collision): G_alpha = c_omega d_alpha Phi_alpha (the

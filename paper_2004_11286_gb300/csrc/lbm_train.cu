@@ -14,7 +14,9 @@
 // tile).  The former chain of 16 launches spent its time in the weight
 // gradients, which it computed on 2 to 4 blocks walking all rows in series.
 // Measured (GB300, M = 8, call to loss on the host): 76 against 1475 us at
-// 4096 rows, 505 against 48300 us at 100,000 rows, 66 against 226 us at 256.
+// 4096 rows (67 against 1487 back to back), 505 against 48300 us at 100,000
+// rows, 66 against 226 us at 256.  A handle's first call also allocates the
+// blocks' partials (0.17 ms).
 #include <cmath>
 
 #include <cuda_runtime.h>
