@@ -355,7 +355,7 @@ __device__ __forceinline__ void collide_node(const DevParams<Real>& p, Store* __
     // what its (y, z) factors cost is shared.  Values that would come from
     // outside the warp, or around the end of a grid row, are formed first,
     // one velocity per lane, and wait in their place of the stage.
-    // Measured (GB300): 256^3 two-species BF16 layers collide 4.95 ms against
+    // Measured (GB300): 256^3 two-species BF16 layers collide 4.98 ms against
     // 6.01 with the 27 velocities unrolled, each reading its own sender's
     // record (8500 instructions a node and 13 % of the gathers served by L1);
     // ternary BF16 ensemble step 2.44 against 3.44 ms, 96^3 FP16 0.267

@@ -143,7 +143,7 @@ __device__ __forceinline__ void incoming_terms(const DevParams<Real>& p, const R
 // those past the grid with active = false and the last node.  Measured (GB300):
 // observables of the 192^3 eight-species BF16 state 4.4 against 9.3 ms with
 // every population's terms formed from its own gathered record, restart copies
-// of 96^3 FP16 0.77 against 0.92 ms, two-species 256^3 BF16 4.2 ms either way.
+// of 96^3 FP16 0.86 against 0.92 ms, two-species 256^3 BF16 4.2 ms either way.
 template <int M, class Store, bool SEP, class F>
 __device__ __forceinline__ void row_populations(const DevParams<float>& p, const float* __restrict__ side, int parity,
                                                 const Nbr& nb, long long n, bool active, F&& f) {
